@@ -1,0 +1,1094 @@
+// Several levels of the median k-d partition (Sec. 4.1 of arXiv 2404.02826) in
+// two launches, for 16-bit codes split on axis depth mod 3.
+//
+// A level of the level-by-level path (k_tree.cu, k_scatter.cu) moves every
+// particle once and takes eight launches.  Here the split planes of up to
+// kSplitMaxLevels levels are found without moving anything - a byte per
+// particle holds its node below the subroot (the node of depth `depth` it lies
+// in) - and then every particle moves once, straight into its node of depth +
+// levels.
+//
+// k_split: one persistent CTA per SM, launched cooperatively; CTA c owns the
+// contiguous positions [c * chunk, (c + 1) * chunk), and a segment is what a
+// CTA holds of one subroot.  Per level:
+//   A     every particle takes its child of the level above (code against the
+//         split plane) and is counted in a shared histogram of its code on the
+//         level's axis, one run of bins per node; the bins of all nodes share
+//         16384 counters, so a bin spans 2^shift codes with the smallest shift
+//         that fits the nodes' real code ranges (0 for most of them);
+//   sel1  every CTA scans the summed histogram: the bin of every node's median;
+//   B     only with shift > 0: the particles of those bins are counted per code
+//         (with shift 0 the counters of A already hold every code);
+//   sel2  every CTA derives the split code v and, from the counts of the
+//         segments before its own, how many of its particles with code v go
+//         left: all, none, or (one segment per node) the first `quota` in
+//         position order.  The next A lists those ties as it meets them and
+//         moves the first `quota` over at its end.
+// Then F gives every particle its final child and counts the children.  Every
+// step between two grid barriers reads only what was complete before the first
+// of them; a barrier costs 1.3 us.
+//
+// k_move: ranks each tile's particles within their children (warp ballots),
+// gathers them in shared memory in runs aligned as their destinations are, and
+// stores 16 bytes at a time.
+// All waits are bounded.
+//
+// What bounds it (2^27 particles, 13-bit codes, two launches of six levels): a
+// pass A reads two code arrays and the node bytes and writes those, 6 bytes a
+// particle, in 115 us (7.0 TB/s, the copy rate of the memory and what L2
+// keeps); level 0 reads one array in 70 us, bound by the shared-memory atomics;
+// B 80 us where a level needs it.  A launch takes 1.25 ms; the move 0.61 ms
+// (13 bytes a particle, 2.9 TB/s), bound by its instructions (78 a row of 32
+// particles) and shared-memory passes (18 a row).  Twelve levels: 3.7 ms, against
+// 5.9 ms level by level (96 launches).  At 2^20 particles the seven levels take
+// 0.13 ms in two launches, against 0.28 ms in 42.
+#include <cstddef>
+#include <cstdint>
+
+#include "pc_internal.cuh"
+
+namespace pcx {
+namespace {
+
+constexpr int kT = 1024;
+constexpr int kW = kT / 32;
+constexpr uint32_t kBins = kSplitBins;
+constexpr uint32_t kLow = kSplitLow;
+constexpr uint32_t kHalf = 1u << (kSplitMaxLevels - 1);  // nodes that split, at most
+constexpr uint32_t kNodes = 1u << kSplitMaxLevels;        // children of the last level, at most
+constexpr uint32_t kStep = 8u * kT;                       // particles of one step of a pass
+constexpr uint32_t kTieBins = 2048;                       // digit of the tie selection by a block
+constexpr uint32_t kTieWarp = 1024;                       // a warp selects among at most this many ties
+constexpr uint32_t kGridSpin = 1u << 21;                  // polls of a grid barrier before it gives up
+
+// State of one segment's nodes.  With several segments in a CTA it is kept in
+// global memory between the steps (the first kStateWords words).
+struct NodeTab {
+  uint32_t blo[2][3][kHalf], bhi[2][3][kHalf];  // code bounds of the nodes, by parity of the level
+  uint32_t plane[kHalf];  // a particle goes right if 2 code + 1 >= plane; odd: 2 v + 1, ties at v are listed
+  uint32_t quota[kHalf];  // listed ties that go left
+  uint32_t mine[kHalf];   // the segment's ties
+  uint32_t bk[kHalf];     // median bin (code >> shift)
+  uint32_t below[kHalf];  // particles of the node in lower bins
+  // derived, not kept
+  int32_t off[kHalf];     // bin of code x: off + (x >> shift)
+  uint32_t roff[kHalf], rcnt[kHalf];  // node's place in the subroot
+  uint32_t lbase[kHalf], cursor[kHalf];  // the node's part of the tie list, and its end so far
+};
+constexpr uint32_t kStateWords = kSplitStateWords;
+static_assert(kStateWords == 17 * kHalf, "kept part of NodeTab");
+
+struct Misc {
+  uint32_t s0, s1;              // subroots of this CTA
+  uint32_t soff, scnt;          // current subroot
+  uint32_t b0, b1;              // current segment
+  uint32_t clo;                 // first CTA of the current subroot
+  uint32_t shift, nbins;
+  uint32_t ties;                // listed ties of the segment
+  uint32_t fd, fbefore;         // tie selection: digit, ties below it
+  uint32_t wt[kW + 1];
+  uint32_t wh[kW][32];
+  uint32_t th[kTieBins];
+};
+
+struct Smem {
+  Misc M;
+  NodeTab N;
+  alignas(16) uint32_t bins[kBins];
+  alignas(16) uint32_t sum[kBins];  // sel1: prefixes of the summed histogram; B: counts per code; A, F: the tie list
+};
+static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
+static_assert(offsetof(Smem, bins) % 16 == 0 && offsetof(Smem, sum) % 16 == 0, "16-byte accesses");
+
+// Grid barrier; bounded.  True when it gave up or the call has failed: the
+// caller leaves the kernel, as every other CTA does at its next barrier.
+__device__ __forceinline__ bool grid_sync(const SplitLaunch &a, uint32_t &epoch) {
+  __syncthreads();
+  bool bad = false;
+  ++epoch;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(a.barrier, 1u);
+    const uint32_t want = epoch * gridDim.x;
+    uint32_t spins = 0;
+    for (;;) {
+      uint32_t v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.barrier) : "memory");
+      if (v >= want) break;
+      ++spins;
+      if (spins > kGridSpin) {
+        atomicOr(a.err, kErrTimeout);
+        bad = true;
+        break;
+      }
+      if ((spins & 255u) == 0 && *reinterpret_cast<volatile uint32_t *>(a.err)) {
+        bad = true;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  return __syncthreads_or(bad) != 0;
+}
+
+__device__ __forceinline__ uint32_t half_of(const uint4 &w, int e) {
+  const uint32_t x = e < 2 ? w.x : (e < 4 ? w.y : (e < 6 ? w.z : w.w));
+  return (e & 1) ? x >> 16 : x & 0xffffu;
+}
+__device__ __forceinline__ uint32_t word_of(const uint4 &w, int i) { return i == 0 ? w.x : (i == 1 ? w.y : (i == 2 ? w.z : w.w)); }
+__device__ __forceinline__ uint32_t byte_of(const uint2 &w, int e) { return ((e < 4 ? w.x : w.y) >> (8 * (e & 3))) & 0xffu; }
+
+struct Ctx {
+  const SplitLaunch &a;
+  Misc &M;
+  NodeTab &N;
+  uint32_t *const bins, *const sum;
+  int lane, warp;
+};
+
+// The segment of subroot s (thread 0 fills the geometry), its kept state when
+// the CTA has several (`load`), and the places of the nodes of level l.
+__device__ __forceinline__ void enter_seg(const Ctx &x, uint32_t s, int l, bool load) {
+  const SplitLaunch &a = x.a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint64_t off, cnt;
+    node_range(a.n, a.depth, s, off, cnt);
+    x.M.soff = uint32_t(off);
+    x.M.scnt = uint32_t(cnt);
+    const uint32_t r0 = blockIdx.x * a.chunk;
+    const uint64_t r1 = min(uint64_t(r0) + a.chunk, a.n);
+    x.M.b0 = max(uint32_t(off), r0);
+    x.M.b1 = uint32_t(min(off + cnt, r1));
+    x.M.clo = uint32_t(off) / a.chunk;
+  }
+  if (load) {
+    const uint32_t *src = a.state + uint64_t(blockIdx.x + s) * kStateWords;
+    uint32_t *dst = reinterpret_cast<uint32_t *>(&x.N);
+    for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
+  }
+  if (l == 0 && !load && threadIdx.x < 3) {  // the subroot's bounds from its parent's split
+    const uint32_t d = threadIdx.x;
+    uint32_t lo = 0, hi = a.root_hi[d];
+    if (a.depth > 0) {
+      const LevelNode &p = a.parents[s >> 1];
+      lo = p.blo[d];
+      hi = p.bhi[d];
+      if (p.v != 0xffffffffu && p.axis == d) {
+        if (s & 1) lo = p.v;
+        else hi = p.v;
+      }
+    }
+    x.N.blo[0][d][0] = lo;
+    x.N.bhi[0][d][0] = hi;
+  }
+  __syncthreads();
+  if (l < a.levels && threadIdx.x < (1u << l)) {
+    uint64_t off, cnt;
+    node_range(x.M.scnt, l, threadIdx.x, off, cnt);
+    x.N.roff[threadIdx.x] = uint32_t(off);
+    x.N.rcnt[threadIdx.x] = uint32_t(cnt);
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void keep_seg(const Ctx &x, uint32_t s) {
+  __syncthreads();
+  uint32_t *dst = x.a.state + uint64_t(blockIdx.x + s) * kStateWords;
+  const uint32_t *src = reinterpret_cast<const uint32_t *>(&x.N);
+  for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
+}
+
+// Bins of level l: the smallest shift whose bins fit, and every node's offset.
+__device__ __forceinline__ void level_bins(const Ctx &x, int l) {
+  const int ax = (x.a.depth + l) % 3, p = l & 1;
+  if (x.warp == 0) {
+    const uint32_t nodes = 1u << l;
+    const uint32_t j0 = 2 * x.lane, j1 = j0 + 1;
+    const bool v0 = j0 < nodes, v1 = j1 < nodes;
+    const uint32_t l0 = v0 ? x.N.blo[p][ax][j0] : 0, h0 = v0 ? x.N.bhi[p][ax][j0] : 0;
+    const uint32_t l1 = v1 ? x.N.blo[p][ax][j1] : 0, h1 = v1 ? x.N.bhi[p][ax][j1] : 0;
+    uint32_t sh = 0, c0, c1, tot;
+    for (;; ++sh) {
+      c0 = v0 ? (h0 >> sh) - (l0 >> sh) + 1u : 0u;
+      c1 = v1 ? (h1 >> sh) - (l1 >> sh) + 1u : 0u;
+      tot = __reduce_add_sync(0xffffffffu, c0 + c1);
+      if (tot <= kBins || sh >= 16) break;
+    }
+    uint32_t incl = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (x.lane >= o) incl += y;
+    }
+    const uint32_t ex = incl - c0 - c1;
+    if (v0) x.N.off[j0] = int32_t(ex) - int32_t(l0 >> sh);
+    if (v1) x.N.off[j1] = int32_t(ex + c0) - int32_t(l1 >> sh);
+    if (x.lane == 0) {
+      x.M.shift = sh;
+      x.M.nbins = min(tot, kBins);
+    }
+  }
+  __syncthreads();
+}
+
+// Lays out the segment's tie list: a run of `mine` places per node with an odd plane.
+__device__ __forceinline__ void tie_lists(const Ctx &x, uint32_t half) {
+  if (x.warp == 0) {
+    const uint32_t j0 = 2 * x.lane, j1 = j0 + 1;
+    const uint32_t t0 = j0 < half && (x.N.plane[j0] & 1u) ? x.N.mine[j0] : 0u;
+    const uint32_t t1 = j1 < half && (x.N.plane[j1] & 1u) ? x.N.mine[j1] : 0u;
+    uint32_t incl = t0 + t1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (x.lane >= o) incl += y;
+    }
+    const uint32_t ex = incl - t0 - t1;
+    x.N.lbase[j0] = x.N.cursor[j0] = ex;
+    x.N.lbase[j1] = x.N.cursor[j1] = ex + t0;
+    if (x.lane == 31) x.M.ties = incl;
+  }
+  __syncthreads();
+}
+
+// The value of rank `rank` among list[0 .. m), positions in [b0, 2^bits + b0): by
+// one warp, 5 bits at a time.
+__device__ __forceinline__ uint32_t select_warp(const uint32_t *list, uint32_t m, uint32_t rank, uint32_t b0, int bits,
+                                                uint32_t *h, int lane) {
+  uint32_t prefix = 0;
+  for (int sh = (bits + 4) / 5 * 5 - 5; sh >= 0; sh -= 5) {
+    h[lane] = 0;
+    __syncwarp();
+    for (uint32_t i = lane; i < m; i += 32) {
+      const uint32_t v = list[i] - b0;
+      if ((v >> sh >> 5) == prefix) atomicAdd(&h[(v >> sh) & 31u], 1u);
+    }
+    __syncwarp();
+    const uint32_t c = h[lane];
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint32_t hit = __ballot_sync(0xffffffffu, incl > rank);
+    const int d = hit ? __ffs(hit) - 1 : 31;
+    rank -= __shfl_sync(0xffffffffu, incl - c, d);
+    prefix = (prefix << 5) | uint32_t(d);
+  }
+  return b0 + prefix;
+}
+
+// The same by the whole block, 11 bits at a time; every thread calls it.
+__device__ __noinline__ uint32_t select_block(Misc &M, const uint32_t *list, uint32_t m, uint32_t rank, uint32_t b0,
+                                              int bits) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t prefix = 0;
+  for (int sh = (bits + 10) / 11 * 11 - 11; sh >= 0; sh -= 11) {
+    for (uint32_t i = threadIdx.x; i < kTieBins; i += kT) M.th[i] = 0;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < m; i += kT) {
+      const uint32_t v = list[i] - b0;
+      if ((v >> sh >> 11) == prefix) atomicAdd(&M.th[(v >> sh) & (kTieBins - 1)], 1u);
+    }
+    __syncthreads();
+    const uint32_t c0 = M.th[2 * threadIdx.x], c1 = M.th[2 * threadIdx.x + 1];
+    uint32_t incl = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) M.wt[warp] = incl;
+    __syncthreads();
+    const uint32_t t = M.wt[lane];
+    const uint32_t ex = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u) + incl - c0 - c1;
+    if (c0 && ex <= rank && rank < ex + c0) {
+      M.fd = 2 * threadIdx.x;
+      M.fbefore = ex;
+    }
+    if (c1 && ex + c0 <= rank && rank < ex + c0 + c1) {
+      M.fd = 2 * threadIdx.x + 1;
+      M.fbefore = ex + c0;
+    }
+    __syncthreads();
+    rank -= M.fbefore;
+    prefix = (prefix << 11) | M.fd;
+    __syncthreads();
+  }
+  return b0 + prefix;
+}
+
+// Counters of the children in F: one row per part of the chunk and warp.
+__device__ __forceinline__ uint32_t part_of(const SplitLaunch &a, uint32_t pos) {
+  const uint32_t q = (pos - blockIdx.x * a.chunk) / a.part;
+  return min(q, uint32_t(kSplitParts - 1));
+}
+
+// The CTA of the move that holds a position.
+__device__ __forceinline__ uint32_t move_part(const SplitLaunch &a, uint32_t pos) {
+  const uint32_t c = pos / a.chunk;
+  return c * kSplitParts + min((pos - c * a.chunk) / a.part, uint32_t(kSplitParts - 1));
+}
+
+// A pass over the segment.  FIRST: level 0, nothing to classify.  LAST: the
+// final children are counted instead of codes.  TIES: ties of some node are listed.
+template <bool FIRST, bool LAST, bool TIES>
+__device__ __forceinline__ void pass_a(const Ctx &x, const uint16_t *__restrict__ prev, const uint16_t *__restrict__ cur,
+                                       uint32_t half, uint32_t *list) {
+  NodeTab &N = x.N;
+  const uint32_t b0 = x.M.b0, b1 = x.M.b1, shift = x.M.shift;
+  uint8_t *const nid = x.a.node;
+  const int32_t off0 = FIRST ? N.off[0] : 0;
+  const uint32_t room = TIES ? x.M.ties : 0u;
+  uint32_t pos = (b0 & ~7u) + 8u * threadIdx.x;
+  uint4 np = make_uint4(0, 0, 0, 0), nc = np;
+  uint2 nn = make_uint2(0, 0);
+  auto load = [&](uint32_t p) {
+    if (!FIRST) {
+      np = __ldcg(reinterpret_cast<const uint4 *>(prev + p));
+      if (half > 1) nn = __ldcg(reinterpret_cast<const uint2 *>(nid + p));  // else the subroot itself, node 0
+    }
+    if (!LAST) nc = __ldcg(reinterpret_cast<const uint4 *>(cur + p));
+  };
+  if (pos < b1) load(pos);
+  for (; pos < b1; pos += kStep) {
+    const uint4 p = np, c = nc;
+    const uint2 n0 = nn;
+    if (pos + kStep < b1) load(pos + kStep);
+    uint32_t mask = 0xffu;
+    if (pos < b0) mask &= 0xffu << (b0 - pos);
+    if (pos + 8u > b1) mask &= 0xffu >> (pos + 8u - b1);
+    uint32_t *const bins = LAST ? x.bins + (part_of(x.a, pos) * kW + x.warp) * kNodes : x.bins;
+    uint32_t w0 = 0, w1 = 0;
+    auto one = [&](int e) {
+      uint32_t child = 0;
+      if (!FIRST) {
+        const uint32_t j = byte_of(n0, e) & (kHalf - 1);
+        const uint32_t pl = N.plane[j], t = 2 * half_of(p, e) + 1;
+        child = 2 * j + (t >= pl ? 1u : 0u);
+        if (TIES && t == pl) {
+          const uint32_t at = atomicAdd(&N.cursor[j], 1u);
+          if (at + 1u <= room) list[at] = pos + uint32_t(e);
+        }
+        if (e < 4) w0 |= child << (8 * e);
+        else w1 |= child << (8 * (e - 4));
+      }
+      if (LAST) atomicAdd(&bins[child], 1u);
+      else atomicAdd(&bins[uint32_t(int32_t(half_of(c, e) >> shift) + (FIRST ? off0 : N.off[child])) & (kBins - 1)], 1u);
+    };
+    if (mask == 0xffu) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) one(e);
+      if (!FIRST) *reinterpret_cast<uint2 *>(nid + pos) = make_uint2(w0, w1);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if ((mask >> e) & 1u) one(e);
+      if (!FIRST) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if ((mask >> e) & 1u) nid[pos + e] = uint8_t((e < 4 ? w0 : w1) >> (8 * (e & 3)));
+      }
+    }
+  }
+}
+
+// The listed ties, all counted as going right so far: the first `quota` of each
+// node in position order go left after all.
+template <bool LAST>
+__device__ __forceinline__ void resolve_ties(const Ctx &x, const uint16_t *__restrict__ cur, uint32_t half,
+                                             const uint32_t *list) {
+  NodeTab &N = x.N;
+  const uint32_t b0 = x.M.b0, shift = x.M.shift;
+  const int bits = int(bit_length(x.M.b1 - b0));
+  auto fix = [&](uint32_t j, uint32_t i0, uint32_t step, uint32_t limit) {
+    const uint32_t *l = list + N.lbase[j];
+    for (uint32_t i = i0; i < N.mine[j]; i += step) {
+      const uint32_t p = l[i];
+      if (p >= limit) continue;
+      x.a.node[p] = uint8_t(2 * j);
+      uint32_t *l_, *r_;
+      if (LAST) {
+        l_ = x.bins + (part_of(x.a, p) * kW + x.warp) * kNodes + 2 * j;
+        r_ = l_ + 1;
+      } else {
+        const int32_t b = int32_t(uint32_t(__ldcg(cur + p)) >> shift);
+        l_ = x.bins + (uint32_t(b + N.off[2 * j]) & (kBins - 1));
+        r_ = x.bins + (uint32_t(b + N.off[2 * j + 1]) & (kBins - 1));
+      }
+      atomicAdd(l_, 1u);
+      atomicSub(r_, 1u);
+    }
+  };
+  // a node whose list is not full (never expected) is left alone, and the call fails
+  auto full = [&](uint32_t j) {
+    if (N.cursor[j] - N.lbase[j] == N.mine[j]) return true;
+    atomicOr(x.a.err, kErrInternal);
+    return false;
+  };
+  for (uint32_t j = x.warp; j < half; j += kW) {
+    if (!(N.plane[j] & 1u) || N.mine[j] > kTieWarp || !full(j)) continue;
+    const uint32_t limit = select_warp(list + N.lbase[j], N.mine[j], N.quota[j], b0, bits, x.M.wh[x.warp], x.lane);
+    fix(j, x.lane, 32, limit);
+    __syncwarp();
+  }
+  for (uint32_t j = 0; j < half; ++j) {
+    if (!(N.plane[j] & 1u) || N.mine[j] <= kTieWarp || !full(j)) continue;
+    const uint32_t limit = select_block(x.M, list + N.lbase[j], N.mine[j], N.quota[j], b0, bits);
+    fix(j, threadIdx.x, kT, limit);
+  }
+}
+
+template <bool FIRST, bool LAST>
+__device__ __forceinline__ void run_a(const Ctx &x, const uint16_t *prev, const uint16_t *cur, uint32_t half) {
+  if (!FIRST && x.M.ties) {
+    // in shared memory when they fit, else in this segment's part of the global list
+    uint32_t *list = x.M.ties <= kBins ? x.sum : x.a.ties + x.M.b0;
+    pass_a<FIRST, LAST, true>(x, prev, cur, half, list);
+    __syncthreads();
+    resolve_ties<LAST>(x, cur, half, list);
+  } else {
+    pass_a<FIRST, LAST, false>(x, prev, cur, half, nullptr);
+  }
+  __syncthreads();
+}
+
+// B: the particles in their node's median bin, counted per code.
+template <bool FIRST>
+__device__ __forceinline__ void pass_b(const Ctx &x, const uint16_t *__restrict__ cur) {
+  const NodeTab &N = x.N;
+  const uint32_t b0 = x.M.b0, b1 = x.M.b1, shift = x.M.shift, cm = (1u << shift) - 1u;
+  const uint8_t *const nid = x.a.node;
+  uint32_t *const low = x.sum;
+  const uint32_t bk0 = N.bk[0];
+  uint32_t pos = (b0 & ~7u) + 8u * threadIdx.x;
+  uint4 nc = make_uint4(0, 0, 0, 0);
+  uint2 nn = make_uint2(0, 0);
+  auto load = [&](uint32_t p) {
+    nc = __ldcg(reinterpret_cast<const uint4 *>(cur + p));
+    if (!FIRST) nn = __ldcg(reinterpret_cast<const uint2 *>(nid + p));
+  };
+  if (pos < b1) load(pos);
+  for (; pos < b1; pos += kStep) {
+    const uint4 c = nc;
+    const uint2 n0 = nn;
+    if (pos + kStep < b1) load(pos + kStep);
+    uint32_t mask = 0xffu;
+    if (pos < b0) mask &= 0xffu << (b0 - pos);
+    if (pos + 8u > b1) mask &= 0xffu >> (pos + 8u - b1);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint32_t q = half_of(c, e), j = FIRST ? 0u : byte_of(n0, e) & (kHalf - 1);
+      if ((q >> shift) == (FIRST ? bk0 : N.bk[j]) && ((mask >> e) & 1u))
+        atomicAdd(&low[((j << shift) | (q & cm)) & (kLow - 1)], 1u);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLaunch a) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  Smem &P = *reinterpret_cast<Smem *>(sm);
+  Misc &M = P.M;
+  NodeTab &N = P.N;
+  if (call_failed(a.err)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const Ctx x = {a, M, N, P.bins, P.sum, lane, warp};
+  const uint32_t c = blockIdx.x, S = 1u << a.depth;
+  const int K = a.levels;
+  uint32_t epoch = 0;
+  if (threadIdx.x == 0) {
+    const uint64_t r0 = uint64_t(c) * a.chunk;
+    M.s0 = 1;
+    M.s1 = 0;
+    if (r0 < a.n) {  // the subroots holding the first and the last position
+      const uint64_t r1 = min(r0 + a.chunk, a.n) - 1;
+      for (int e = 0; e < 2; ++e) {
+        uint32_t lo = 0, hi = S - 1;
+        while (lo < hi) {
+          const uint32_t mid = (lo + hi + 1) >> 1;
+          uint64_t off, cnt;
+          node_range(a.n, a.depth, mid, off, cnt);
+          if (off <= (e ? r1 : r0)) lo = mid;
+          else hi = mid - 1;
+        }
+        if (e) M.s1 = lo;
+        else M.s0 = lo;
+      }
+    }
+  }
+  __syncthreads();
+  const uint32_t s0 = M.s0, s1 = M.s1;
+  const bool multi = s1 > s0;
+  const uint32_t gthreads = gridDim.x * kT, gtid = c * kT + threadIdx.x;
+
+  for (int l = 0; l < K; ++l) {
+    const uint32_t nodes = 1u << l, half = nodes >> 1;
+    const uint16_t *const cur = a.src[(a.depth + l) % 3];
+    const uint16_t *const prev = a.src[(a.depth + l + 2) % 3];
+    uint32_t *const hist = a.hist + uint64_t(l & 1) * S * kBins;
+    uint32_t *const low = a.low + uint64_t(l & 1) * S * kLow;
+    // ---- A ----
+    if (l > 0) {  // the other histogram was read by every CTA before the last barrier
+      uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * kBins);
+      for (uint32_t i = gtid; i < S * (kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+    }
+    for (uint32_t s = s0; s <= s1; ++s) {
+      enter_seg(x, s, l, multi && l > 0);
+      level_bins(x, l);
+      tie_lists(x, half);
+      const uint32_t nbins = M.nbins;
+      for (uint32_t b = threadIdx.x; b < nbins; b += kT) P.bins[b] = 0;
+      __syncthreads();
+      if (l == 0) run_a<true, false>(x, prev, cur, half);
+      else run_a<false, false>(x, prev, cur, half);
+      uint32_t *const h = hist + uint64_t(s) * kBins;
+      uint32_t *const own = a.seghist + uint64_t(2 * s + (c != M.clo)) * kBins;
+      for (uint32_t b = threadIdx.x; b < nbins; b += kT) {
+        const uint32_t v = P.bins[b];
+        if (v) atomicAdd(h + b, v);
+        if (multi) own[b] = v;
+      }
+      if (multi) keep_seg(x, s);
+    }
+    if (grid_sync(a, epoch)) return;
+    // ---- sel1 and B ----
+    if (l > 0) {
+      uint4 *z = reinterpret_cast<uint4 *>(a.low + uint64_t((l + 1) & 1) * S * kLow);
+      for (uint32_t i = gtid; i < S * (kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+    }
+    for (uint32_t s = s0; s <= s1; ++s) {
+      if (multi) {
+        enter_seg(x, s, l, l > 0);
+        level_bins(x, l);
+      }
+      const uint32_t nbins = M.nbins, shift = M.shift;
+      {  // exclusive prefixes within each warp's 512 bins, and the warps' totals
+        const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + uint64_t(s) * kBins);
+        constexpr uint32_t kPer = kBins / kW;
+        uint4 v[kPer / 128];
+#pragma unroll
+        for (uint32_t i = 0; i < kPer / 128; ++i) {
+          const uint32_t b = warp * kPer + i * 128 + lane * 4;
+          v[i] = b < nbins ? __ldcg(h4 + b / 4) : make_uint4(0, 0, 0, 0);
+        }
+        uint32_t run = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < kPer / 128; ++i) {
+          const uint32_t b = warp * kPer + i * 128 + lane * 4;
+          const uint32_t t = v[i].x + v[i].y + v[i].z + v[i].w;
+          uint32_t incl = t;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          const uint32_t ex = run + incl - t;
+          *reinterpret_cast<uint4 *>(&P.sum[b]) =
+              make_uint4(ex, ex + v[i].x, ex + v[i].x + v[i].y, ex + v[i].x + v[i].y + v[i].z);
+          run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) M.wt[warp] = run;
+        __syncthreads();
+        uint32_t wb = 0;
+        if (warp == 0) {
+          const uint32_t t = M.wt[lane];
+          uint32_t incl = t;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          wb = incl - t;
+        }
+        __syncthreads();
+        if (warp == 0) M.wt[lane] = wb;
+        __syncthreads();
+        if (threadIdx.x < nodes) {
+          // the last bin of the node whose prefix does not exceed the median's rank
+          const uint32_t j = threadIdx.x;
+          const int ax = (a.depth + l) % 3;
+          const uint32_t cl = N.blo[l & 1][ax][j] >> shift, ch = N.bhi[l & 1][ax][j] >> shift;
+          const uint32_t target = N.roff[j] + (N.rcnt[j] >> 1);
+          uint32_t lo = uint32_t(N.off[j] + int32_t(cl)), hi = uint32_t(N.off[j] + int32_t(ch));
+          if (hi >= kBins) hi = kBins - 1;
+          while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (M.wt[mid / kPer] + P.sum[mid] <= target) lo = mid;
+            else hi = mid - 1;
+          }
+          N.bk[j] = uint32_t(int32_t(lo) - N.off[j]);
+          N.below[j] = M.wt[lo / kPer] + P.sum[lo] - N.roff[j];
+        }
+        __syncthreads();
+      }
+      const uint32_t nlow = min(nodes << shift, kLow);
+      uint32_t *const sl = a.seglow + c + s;  // counter i of this segment: sl[i * segs]
+      const uint64_t segs = gridDim.x + S;
+      if (shift == 0) {  // A's counters hold the ties of every node
+        if (threadIdx.x < nodes) {
+          const uint32_t b = uint32_t(N.off[threadIdx.x] + int32_t(N.bk[threadIdx.x])) & (kBins - 1);
+          sl[threadIdx.x * segs] = multi ? __ldcg(a.seghist + uint64_t(2 * s + (c != M.clo)) * kBins + b) : P.bins[b];
+        }
+      } else {
+        for (uint32_t i = threadIdx.x; i < nlow; i += kT) P.sum[i] = 0;
+        __syncthreads();
+        if (l == 0) pass_b<true>(x, cur);
+        else pass_b<false>(x, cur);
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < nlow; i += kT) {
+          const uint32_t v = P.sum[i];
+          sl[i * segs] = v;
+          if (v) atomicAdd(low + uint64_t(s) * kLow + i, v);
+        }
+      }
+      if (multi) keep_seg(x, s);
+    }
+    if (grid_sync(a, epoch)) return;
+    // ---- sel2: a warp per node ----
+    for (uint32_t s = s0; s <= s1; ++s) {
+      if (multi) {
+        enter_seg(x, s, l, true);
+        level_bins(x, l);
+      }
+      const uint32_t shift = M.shift;
+      const int ax = (a.depth + l) % 3;
+      const bool writer = l == K - 1 && c == M.clo;
+      for (uint32_t j = warp; j < nodes; j += kW) {
+        const uint32_t target = (N.rcnt[j] >> 1) - N.below[j];
+        uint32_t vlow = 0, less = 0;
+        if (shift) {
+          const uint32_t *lw = low + uint64_t(s) * kLow + (j << shift);
+          uint32_t run = 0;
+          for (uint32_t i0 = 0; i0 < (1u << shift); i0 += 32) {
+            const uint32_t v = i0 + lane < (1u << shift) ? __ldcg(lw + i0 + lane) : 0u;
+            uint32_t incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+              if (lane >= o) incl += y;
+            }
+            const uint32_t hit = __ballot_sync(0xffffffffu, v && run + incl - v <= target && target < run + incl);
+            if (hit) {
+              const int src = __ffs(hit) - 1;
+              vlow = i0 + src;
+              less = run + __shfl_sync(0xffffffffu, incl - v, src);
+              break;
+            }
+            run += __shfl_sync(0xffffffffu, incl, 31);
+          }
+        }
+        const uint32_t v = (N.bk[j] << shift) | vlow;
+        const uint32_t tleft = target - less, slot = ((j << shift) | vlow) & (kLow - 1);
+        uint32_t before = 0;
+        const uint32_t *const row = a.seglow + uint64_t(slot) * (gridDim.x + S) + s;
+        const uint32_t mine = __ldcg(row + c);
+#pragma unroll 4
+        for (uint32_t k = M.clo + lane; k < c; k += 32) before += __ldcg(row + k);
+        before = __reduce_add_sync(0xffffffffu, before);
+        const uint32_t quota = tleft > before ? min(tleft - before, mine) : 0u;
+        if (lane == 0) {
+          N.plane[j] = 2 * v + (quota == 0 ? 0u : (quota == mine ? 2u : 1u));
+          N.quota[j] = quota;
+          N.mine[j] = mine;
+          const int p = l & 1, q = p ^ 1;
+          if (l + 1 < K) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const uint32_t lo = N.blo[p][d][j], hi = N.bhi[p][d][j];
+              N.blo[q][d][2 * j] = lo;
+              N.bhi[q][d][2 * j] = d == ax ? v : hi;
+              N.blo[q][d][2 * j + 1] = d == ax ? v : lo;
+              N.bhi[q][d][2 * j + 1] = hi;
+            }
+          }
+          if (writer) {  // the record the next levels take as parent
+            LevelNode nd = {};
+            for (int d = 0; d < 3; ++d) {
+              nd.blo[d] = N.blo[p][d][j];
+              nd.bhi[d] = N.bhi[p][d][j];
+            }
+            nd.axis = uint32_t(ax);
+            nd.lo = nd.blo[ax];
+            nd.hi = nd.bhi[ax];
+            nd.v = v;
+            nd.less = N.below[j] + less;
+            nd.tleft = tleft;
+            a.out_nodes[(uint64_t(s) << l) + j] = nd;
+          }
+        }
+      }
+      if (multi) keep_seg(x, s);
+      else __syncthreads();
+    }
+  }
+
+  // ---- F: final children, counted per segment and part of the chunk ----
+  const uint32_t half = 1u << (K - 1);
+  for (uint32_t s = s0; s <= s1; ++s) {
+    enter_seg(x, s, K, multi);
+    tie_lists(x, half);
+    for (uint32_t b = threadIdx.x; b < kSplitParts * kW * kNodes; b += kT) P.bins[b] = 0;
+    __syncthreads();
+    run_a<false, true>(x, a.src[(a.depth + K + 2) % 3], nullptr, half);
+    for (uint32_t i = threadIdx.x; i < kSplitParts * kNodes; i += kT) {
+      const uint32_t q = i / kNodes, b = i % kNodes;
+      if (q < part_of(a, M.b0) || q > part_of(a, M.b1 - 1) || b >= 2 * half) continue;
+      uint32_t v = 0;
+#pragma unroll 8
+      for (int w = 0; w < kW; ++w) v += P.bins[(q * kW + w) * kNodes + b];
+      a.segcnt[uint64_t(b) * (gridDim.x * kSplitParts + S) + c * kSplitParts + q + s] = v;
+    }
+  }
+  if (grid_sync(a, epoch)) return;
+  // first place of every child for every part: exclusive sums along the parts of a
+  // subroot, in place, a warp per subroot and child
+  const uint64_t msegs = uint64_t(gridDim.x) * kSplitParts + S;
+  for (uint32_t i = c + gridDim.x * warp; i < S << K; i += gridDim.x * kW) {
+    const uint32_t s = i >> K, b = i & ((1u << K) - 1u);
+    uint64_t soff, scnt, off, cnt;
+    node_range(a.n, a.depth, s, soff, scnt);
+    node_range(scnt, K, b, off, cnt);
+    uint32_t run = uint32_t(soff + off);
+    uint32_t *const row = a.segcnt + b * msegs + s;
+    const uint32_t m0 = move_part(a, uint32_t(soff)), m1 = move_part(a, uint32_t(soff + scnt - 1));
+    for (uint32_t k0 = m0; k0 <= m1; k0 += 4 * 32) {
+      uint32_t v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t k = k0 + 32 * u + lane;
+        v[u] = k <= m1 ? __ldcg(row + k) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t k = k0 + 32 * u + lane;
+        uint32_t incl = v[u];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        if (k <= m1) row[k] = run + incl - v[u];
+        run += __shfl_sync(0xffffffffu, incl, 31);
+      }
+    }
+  }
+  if (a.clear) {  // another launch follows: the histograms are left zero
+    uint4 *z = reinterpret_cast<uint4 *>(a.hist);
+    for (uint64_t i = gtid; i < uint64_t(S) * (2 * kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+    z = reinterpret_cast<uint4 *>(a.low);
+    for (uint64_t i = gtid; i < uint64_t(S) * (2 * kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+  }
+}
+
+// ---- the move ----
+
+constexpr int kMT = 512;
+constexpr int kMW = kMT / 32;
+
+template <bool IDX>
+struct MoveSmem {
+  static constexpr int kRows = IDX ? 8 : 16;                // rows of 32 particles per warp and tile
+  static constexpr uint32_t kTile = uint32_t(kRows) * kMT;
+  static constexpr uint32_t kStage = kTile + kNodes * 14u;  // every child's run padded to whole groups of 8
+  alignas(16) uint2 st[kStage];  // x | y << 16, z; place p at stage_slot(p)
+  // per warp: first the nodes of its particles, then child << 9 | rank of every particle
+  alignas(16) uint16_t code[kMW][32 * kRows];
+  alignas(16) uint32_t sti[IDX ? kStage : 4];
+  // counts of a child by warp, then the place in the stage of the warp's first one; 16 bits, so
+  // that the counts of 64 children span the 32 banks once
+  uint16_t wcnt[kMW][kNodes + 2];
+  uint32_t tot[kNodes], lst[kNodes], lend[kNodes], gof[kNodes], run[kNodes];
+  uint8_t grp[kStage / 8 + 8];
+  uint32_t s0, s1, b0, b1, ngroups;
+};
+
+// Where place p of the stage lies: the four 16-byte pieces of a group of 8 are
+// permuted by the group, so that the threads reading a group each meet no bank conflict.
+__device__ __forceinline__ uint32_t stage_slot(uint32_t p) { return p ^ ((p >> 3) & 6u); }
+
+// One tile, up to its particles in the stage by child.  WHOLE: the tile lies in
+// the segment.  A warp ranks rows of 32 consecutive particles: the lanes with
+// the same child, and the warp's count of that child so far from shared memory.
+template <bool IDX, int BITS, bool WHOLE>
+__device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T, uint4 nodes, uint32_t t0, uint32_t b0,
+                                          uint32_t b1, uint32_t NB, int lane, int warp) {
+  using V = MoveSmem<IDX>;
+  constexpr int kRows = V::kRows;
+  const uint32_t ltm = (1u << lane) - 1u;
+  const uint32_t w0 = t0 + uint32_t(warp) * (32 * kRows);  // the warp's first particle
+  uint16_t *const wc = T.wcnt[warp], *const cb = T.code[warp];
+  auto inside = [&](uint32_t p) { return WHOLE || (p >= b0 && p < b1); };
+  for (uint32_t i = lane; i < (NB + 1u) / 2u; i += 32) reinterpret_cast<uint32_t *>(wc)[i] = 0;
+  if (lane < 2 * kRows) reinterpret_cast<uint4 *>(cb)[lane] = nodes;
+  __syncwarp();
+  {
+    uint32_t nd[kRows];
+    const uint8_t *const nb = reinterpret_cast<const uint8_t *>(cb);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) nd[r] = uint32_t(nb[32 * r + lane]) & (NB - 1u);
+    // the lanes with this lane's child: one ballot per bit (with a match instruction, which
+    // takes as long as the row has different children, the move took 1.07 ms at 2^27)
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      uint32_t peers = WHOLE ? 0xffffffffu : __ballot_sync(0xffffffffu, inside(w0 + 32 * r + lane));
+#pragma unroll
+      for (int k = 0; k < BITS; ++k) {
+        uint32_t v;  // the lanes whose bit k is this lane's
+        asm(
+            "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t"
+            "vote.sync.ballot.b32 %0, p, 0xffffffff;\n\t@!p not.b32 %0, %0;\n\t}"
+            : "=r"(v)
+            : "r"(nd[r]), "r"(1u << k));
+        peers &= v;
+      }
+      nd[r] |= (__popc(peers & ltm) << 8) | (__popc(peers) << 16);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const uint32_t b = nd[r] & 0xffu, old = wc[b];
+      __syncwarp();
+      if (inside(w0 + 32 * r + lane)) wc[b] = uint16_t(old + (nd[r] >> 16));  // every lane of the child: the same
+      cb[32 * r + lane] = uint16_t((b << 9) | (old + ((nd[r] >> 8) & 0xffu)));
+      __syncwarp();
+    }
+  }
+  // from here on a lane holds 8 consecutive particles of every 256: its codes
+  constexpr int kOct = kRows / 8;
+  uint4 x[kOct], y[kOct], z[kOct], ix[IDX ? 2 * kOct : 1];
+#pragma unroll
+  for (int i = 0; i < kOct; ++i) {
+    const uint32_t p = w0 + 256u * i + 8u * lane;
+    x[i] = y[i] = z[i] = make_uint4(0, 0, 0, 0);
+    if (WHOLE || p < b1) {
+      x[i] = __ldcg(reinterpret_cast<const uint4 *>(a.src[0] + p));
+      y[i] = __ldcg(reinterpret_cast<const uint4 *>(a.src[1] + p));
+      z[i] = __ldcg(reinterpret_cast<const uint4 *>(a.src[2] + p));
+      if (IDX) {
+        ix[2 * i] = __ldcg(reinterpret_cast<const uint4 *>(a.src_idx + p));
+        ix[2 * i + 1] = __ldcg(reinterpret_cast<const uint4 *>(a.src_idx + p) + 1);
+      }
+    }
+  }
+  __syncthreads();
+  // per child the warps' counts summed up, a half-warp per child
+  for (uint32_t b = 2 * warp + (lane >> 4); b < NB; b += 2 * kMW) {
+    const uint32_t v = T.wcnt[lane & 15][b];
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const uint32_t w = __shfl_up_sync(0xffffffffu, incl, o, 16);
+      if ((lane & 15) >= o) incl += w;
+    }
+    T.wcnt[lane & 15][b] = uint16_t(incl - v);
+    if ((lane & 15) == 15) T.tot[b] = incl;
+  }
+  __syncthreads();
+  // the children's runs in the stage: whole groups of 8, aligned as their destinations
+  if (warp == 0) {
+    constexpr int kPer = int(kNodes) / 32;
+    uint32_t sz[kPer], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const uint32_t b = lane * kPer + i;
+      const uint32_t tot = b < NB ? T.tot[b] : 0u;
+      sz[i] = tot ? ((T.run[b] & 7u) + tot + 7u) & ~7u : 0u;
+      sum += sz[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t w = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += w;
+    }
+    uint32_t at = incl - sum;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const uint32_t b = lane * kPer + i;
+      if (b < NB) {
+        const uint32_t g = T.run[b], l0 = at + (g & 7u), tot = T.tot[b];
+        T.lst[b] = l0;
+        T.lend[b] = l0 + tot;
+        T.gof[b] = g - l0;
+        T.run[b] = g + tot;
+      }
+      at += sz[i];
+    }
+    if (lane == 31) T.ngroups = incl / 8u;
+  }
+  __syncthreads();
+  for (uint32_t b = lane; b < NB; b += 32) wc[b] = uint16_t(wc[b] + T.lst[b]);
+  __syncwarp();
+  for (uint32_t b = warp; b < NB; b += kMW) {
+    const uint32_t l0 = T.lst[b], l1 = T.lend[b];
+    if (l1 > l0)
+      for (uint32_t g = l0 / 8u + lane; g < (l1 + 7u) / 8u; g += 32) T.grp[g] = uint8_t(b);
+  }
+#pragma unroll
+  for (int i = 0; i < kOct; ++i) {
+    const uint4 cd = reinterpret_cast<const uint4 *>(cb)[32 * i + lane];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (inside(w0 + 256u * i + 8u * lane + e)) {
+        const uint32_t c = half_of(cd, e), at = wc[c >> 9] + (c & 511u);
+        const uint32_t xw = word_of(x[i], e >> 1), yw = word_of(y[i], e >> 1), zw = word_of(z[i], e >> 1);
+        T.st[stage_slot(at)] = make_uint2(__byte_perm(xw, yw, (e & 1) ? 0x7632 : 0x5410), (e & 1) ? zw >> 16 : zw);
+        if (IDX) T.sti[at] = word_of(ix[2 * i + (e >> 2)], e & 3);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// CTA m takes part m % kSplitParts of the chunk m / kSplitParts, tile by tile in
+// position order.  A tile's particles are gathered in shared memory by child,
+// every child's run starting at the same offset modulo 8 as its destination,
+// so that whole groups of 8 leave as 16-byte stores.  BITS: at least `levels`,
+// the bits of a child.
+template <bool IDX, int BITS>
+__global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLaunch a) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  using V = MoveSmem<IDX>;
+  V &T = *reinterpret_cast<V *>(sm);
+  constexpr uint32_t kTile = V::kTile;
+  if (call_failed(a.err)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t m = blockIdx.x, S = 1u << a.depth;
+  const int K = a.levels;
+  const uint32_t NB = 1u << K;
+  const uint64_t c0 = uint64_t(m / kSplitParts) * a.chunk, c1 = min(c0 + a.chunk, a.n);
+  const uint64_t q0 = c0 + uint64_t(m % kSplitParts) * a.part;
+  const uint64_t q1 = m % kSplitParts == kSplitParts - 1 ? c1 : min(q0 + a.part, c1);
+  if (q0 >= q1) return;
+  if (threadIdx.x < 2) {  // the subroots holding the first and the last position
+    const uint64_t p = threadIdx.x ? q1 - 1 : q0;
+    uint32_t lo = 0, hi = S - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      uint64_t off, cnt;
+      node_range(a.n, a.depth, mid, off, cnt);
+      if (off <= p) lo = mid;
+      else hi = mid - 1;
+    }
+    if (threadIdx.x) T.s1 = lo;
+    else T.s0 = lo;
+  }
+  __syncthreads();
+  const uint32_t s0 = T.s0, s1 = T.s1;
+  for (uint32_t s = s0; s <= s1; ++s) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint64_t off, cnt;
+      node_range(a.n, a.depth, s, off, cnt);
+      T.b0 = uint32_t(max(off, q0));
+      T.b1 = uint32_t(min(off + cnt, q1));
+    }
+    if (threadIdx.x < NB) T.run[threadIdx.x] = __ldcg(a.segcnt + uint64_t(threadIdx.x) * (gridDim.x + S) + m + s);
+    __syncthreads();
+    const uint32_t b0 = T.b0, b1 = T.b1;
+    // 16 consecutive particles' nodes of the tile at t0, loaded a tile ahead
+    uint4 nodes = make_uint4(0, 0, 0, 0);
+    auto load_nodes = [&](uint32_t t0) {
+      const uint32_t p = t0 + uint32_t(warp) * (32 * V::kRows) + 16u * lane;
+      if (lane < 2 * V::kRows && p < b1) nodes = __ldcg(reinterpret_cast<const uint4 *>(a.node + p));
+    };
+    load_nodes(b0 & ~31u);
+    for (uint32_t t0 = b0 & ~31u; t0 < b1; t0 += kTile) {
+      if (t0 >= b0 && t0 + kTile <= b1) move_tile<IDX, BITS, true>(a, T, nodes, t0, b0, b1, NB, lane, warp);
+      else move_tile<IDX, BITS, false>(a, T, nodes, t0, b0, b1, NB, lane, warp);
+      if (t0 + kTile < b1) load_nodes(t0 + kTile);
+      const uint32_t ngroups = T.ngroups;
+      for (uint32_t g = threadIdx.x; g < ngroups; g += kMT) {
+        const uint32_t b = T.grp[g], li = 8u * g, gi = li + T.gof[b];
+        if (li >= T.lst[b] && li + 8u <= T.lend[b] && uint64_t(gi) + 8u <= a.n) {
+          uint32_t u[8], w[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(&T.st[stage_slot(li + 2 * i)]);
+            u[2 * i] = v.x;
+            w[2 * i] = v.y;
+            u[2 * i + 1] = v.z;
+            w[2 * i + 1] = v.w;
+          }
+          uint32_t ox[4], oy[4], oz[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            ox[i] = __byte_perm(u[2 * i], u[2 * i + 1], 0x5410);
+            oy[i] = __byte_perm(u[2 * i], u[2 * i + 1], 0x7632);
+            oz[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
+          }
+          __stcg(reinterpret_cast<uint4 *>(a.dst[0] + gi), make_uint4(ox[0], ox[1], ox[2], ox[3]));
+          __stcg(reinterpret_cast<uint4 *>(a.dst[1] + gi), make_uint4(oy[0], oy[1], oy[2], oy[3]));
+          __stcg(reinterpret_cast<uint4 *>(a.dst[2] + gi), make_uint4(oz[0], oz[1], oz[2], oz[3]));
+          if (IDX) {
+            const uint4 *q = reinterpret_cast<const uint4 *>(&T.sti[li]);
+            __stcg(reinterpret_cast<uint4 *>(a.dst_idx + gi), q[0]);
+            __stcg(reinterpret_cast<uint4 *>(a.dst_idx + gi) + 1, q[1]);
+          }
+        }
+      }
+      // the groups at the two ends of every run, a lane per particle
+      for (uint32_t i = threadIdx.x; i < NB * 16u; i += kMT) {
+        const uint32_t b = i >> 4, l0 = T.lst[b], l1 = T.lend[b];
+        const uint32_t g0 = l0 & ~7u, g1 = (l1 - 1u) & ~7u;
+        const uint32_t g = (i & 8u) ? g1 : g0, li = g | (i & 7u);
+        const bool mine = l1 > l0 && li >= l0 && li < l1 && (g < l0 || g + 8u > l1) && !((i & 8u) && g1 == g0);
+        if (mine) {
+          const uint32_t gi = li + T.gof[b];
+          if (gi < a.n) {
+            const uint2 v = T.st[stage_slot(li)];
+            __stcg(a.dst[0] + gi, uint16_t(v.x));
+            __stcg(a.dst[1] + gi, uint16_t(v.x >> 16));
+            __stcg(a.dst[2] + gi, uint16_t(v.y));
+            if (IDX) __stcg(a.dst_idx + gi, T.sti[li]);
+          } else {
+            atomicOr(a.err, kErrInternal);
+          }
+        }
+      }
+      // the next tile writes these tables and the stage after its first barriers
+    }
+  }
+}
+
+template <bool IDX, int BITS>
+cudaError_t move_launch(const SplitLaunch &a, cudaStream_t st) {
+  constexpr size_t smem = sizeof(MoveSmem<IDX>);
+  int per_sm = 0;
+  cudaError_t e = resident_blocks<k_move<IDX, BITS>>(kMT, smem, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  TraceScope ts("k_move", st);
+  k_move<IDX, BITS><<<unsigned(a.grid) * kSplitParts, kMT, smem, st>>>(a);
+  return cudaGetLastError();
+}
+template <bool IDX>
+cudaError_t move_dispatch(const SplitLaunch &a, cudaStream_t st) {
+  if (a.levels <= 4) return move_launch<IDX, 4>(a, st);
+  if (a.levels == 5) return move_launch<IDX, 5>(a, st);
+  return a.levels == 6 ? move_launch<IDX, 6>(a, st) : move_launch<IDX, 7>(a, st);
+}
+
+}  // namespace
+
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st) {
+  constexpr size_t smem = sizeof(Smem);
+  int per_sm = 0;
+  cudaError_t e = resident_blocks<k_split>(kT, smem, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1 || a.grid < 1 || a.grid > per_sm * device_sm_count()) return cudaErrorInvalidConfiguration;
+  SplitLaunch arg = a;
+  arg.part = ((a.chunk + kSplitParts - 1) / kSplitParts + 31u) & ~31u;
+  void *args[] = {&arg};
+  {
+    TraceScope ts("k_split", st);
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_split), dim3(unsigned(a.grid)), dim3(kT), args,
+                                    smem, st);
+    if (e != cudaSuccess) return e;
+  }
+  return a.src_idx ? move_dispatch<true>(arg, st) : move_dispatch<false>(arg, st);
+}
+
+}  // namespace pcx

@@ -1,5 +1,6 @@
 // C ABI (include/pc.h): argument checks, the error-bound arithmetic of Sec. 3
 // on the host, workspace layout, and the launch sequence of the hot path.
+#include <algorithm>
 #include <cfloat>
 #include <chrono>
 #include <cmath>
@@ -216,6 +217,7 @@ struct Plan {
   bool tune = false;  // leaf size chosen by descending from r_hi while the stream shrinks (sized for r)
   uint32_t r_hi = 0;
   int tune_first = 0, tune_last = 0;  // candidate depths
+  uint64_t off_split = 0;             // several levels per launch (k_split.cu): histograms and barriers (zeroed)
   uint64_t off_tunecost = 0;          // leaf-size search: payload words per in-CTA depth (zeroed)
   uint64_t total = 0;
   int range_blocks = 0;
@@ -280,6 +282,31 @@ uint32_t digit_bits_for(int level) {
   if (d < 6) d = 6;
   return uint32_t(d);
 }
+
+// Several levels per launch (k_split.cu).  A launch below depth 0 needs subroots
+// of at least kSplitMinRoot particles, so that their histograms stay small
+// beside the data, and its levels are limited by the codes' bits: at level l of
+// a launch the 2^l nodes share kSplitBins bins and the codes of their median
+// bins kSplitLow counters, which holds for every data while
+// bits <= 26 - 2 l, i.e. 7 levels up to 14 bits, else 6.
+constexpr uint64_t kSplitMinRoot = 1u << 17;
+constexpr uint64_t kSplitMinChunk = 4096;  // particles of a CTA: fewer CTAs for small inputs
+constexpr int kSplitLaunches = 16;         // barrier words
+
+bool split_roots_ok(uint64_t n, int depth) {
+  return depth == 0 || ((1ull << depth) <= kSplitMaxRoots && (n >> depth) >= kSplitMinRoot);
+}
+uint64_t split_roots_max(uint64_t n) {
+  int d = 0;
+  while (split_roots_ok(n, d + 1)) ++d;
+  return 1ull << d;
+}
+uint64_t split_zero_bytes(uint64_t n) {
+  return 4 * kSplitLaunches * 32 + split_roots_max(n) * 2 * 4 * uint64_t(kSplitBins + kSplitLow);
+}
+
+// Bytes of one axis's u16 code array (the same padding).
+inline uint64_t code_stride16(uint64_t n) { return align_up(2 * n + 64); }
 
 // Bytes of one axis's code array: room for u32 codes and for the 16-byte
 // loads of a tile's last group, which may reach up to 64 bytes past n.
@@ -407,6 +434,8 @@ int make_plan(uint64_t n, int dtype, const pc_config *cfg, bool idx, int sm_coun
   o = align_up(o + 4 * (p.levels + 2));
   p.off_tunecost = o;
   o = align_up(o + 8 * (kSubMaxLevels + 1));
+  p.off_split = o;
+  if (p.levels > 0) o = align_up(o + split_zero_bytes(n));
   p.off_status = o;
   o = align_up(o + 8 * subtree_status_entries(p.levels));
   p.off_err = o;
@@ -540,7 +569,8 @@ struct RunFacts {
 
 int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                   void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                  uint32_t *perm, cudaStream_t st, Sweep *sweep = nullptr, RunFacts *facts = nullptr) {
+                  uint32_t *perm, cudaStream_t st, int share = 1, Sweep *sweep = nullptr,
+                  RunFacts *facts = nullptr) {
   if (sweep) {
     if (!cfg || !(cfg->flags & PC_FLAG_AUTOTUNE_LEAF) || perm) return PC_ERR_ARG;
   } else if (!out || !out_size) {
@@ -602,11 +632,16 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     const uint32_t qmax = L.qmax[0] > L.qmax[1] ? (L.qmax[0] > L.qmax[2] ? L.qmax[0] : L.qmax[2])
                                                  : (L.qmax[1] > L.qmax[2] ? L.qmax[1] : L.qmax[2]);
     const int cb = (qmax < 65536u && !L.raw) ? 2 : 4;
+    // u16 codes lie at the two ends of the room for u32 codes; what they leave
+    // between them is scratch of the levels
     void *codes_a[3], *codes_b[3];
+    const uint64_t cstride = cb == 2 ? code_stride16(n) : code_stride(n);
     for (int d = 0; d < 3; ++d) {
-      codes_a[d] = ws + p.off_codes_a + uint64_t(d) * code_stride(n);
-      codes_b[d] = ws + p.off_codes_b + uint64_t(d) * code_stride(n);
+      codes_a[d] = ws + p.off_codes_a + uint64_t(d) * cstride;
+      codes_b[d] = ws + p.off_codes_b + 3 * code_stride(n) - uint64_t(3 - d) * cstride;
     }
+    uint8_t *const spare = ws + p.off_codes_a + 3 * cstride;
+    const uint64_t spare_bytes = (p.off_codes_b + 3 * code_stride(n) - 3 * cstride) - (p.off_codes_a + 3 * cstride);
     uint32_t *idx_a = use_idx ? reinterpret_cast<uint32_t *>(ws + p.off_idx_a) : nullptr;
     uint32_t *idx_b = use_idx ? reinterpret_cast<uint32_t *>(ws + p.off_idx_b) : nullptr;
 
@@ -819,7 +854,78 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       if (l > first_depth && bytes >= best_bytes) chosen = l - 1;
       else best_bytes = bytes;
     };
-    for (int l = 0; l < global_levels; ++l) {
+    // several levels per launch while every node is larger than a leaf and than what a
+    // warp splits (k_split.cu; u16 codes, depth mod 3); the leaf-size search needs the
+    // arrangement of every candidate depth.  Two launches for up to seven levels against
+    // eight a level: faster at every size measured (one level of 10,007 particles 30 us
+    // against 39; seven of 2^20 130 us against 280; twelve of 2^27 3.7 ms against 5.9)
+    int split_to = 0;
+    if (cb == 2 && !p.widest && !t_drop_tile_copies) {
+      const int most = p.tune && first_depth < global_levels ? first_depth : global_levels;
+      while (split_to < most && (n >> split_to) > p.r &&
+             ((n + (1ull << split_to) - 1) >> split_to) > p.warp_node_max)
+        ++split_to;
+    }
+    for (int launches = 0; src_depth < split_to && split_roots_ok(n, src_depth) && launches < kSplitLaunches;
+         ++launches) {
+      // even shares of what is left, or as many as one launch takes where a second one's
+      // subroots would be too small
+      const int max_levels = bit_length(qmax) <= 14 ? 7 : 6, left = split_to - src_depth;
+      const int parts = (left + max_levels - 1) / max_levels;
+      SplitLaunch sl = {};
+      sl.n = n;
+      sl.depth = src_depth;
+      sl.levels = (left + parts - 1) / parts;
+      if (parts > 1 && !split_roots_ok(n, src_depth + sl.levels)) sl.levels = max_levels;
+      // a CTA per SM, fewer for small inputs, and this call's share of them when others run
+      // beside it: 48 snapshots of 10^4 to 10^7 particles on 8 lanes took 8.3 ms when every
+      // launch asked for all SMs, 5.8 with its share
+      const uint64_t sms = uint64_t(device_sm_count());
+      const uint64_t cap = share > 1 ? std::max<uint64_t>(1, sms / uint64_t(share)) : sms;
+      sl.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap)));
+      sl.chunk = uint32_t(((n + sl.grid - 1) / sl.grid + 15) & ~15ull);
+      const uint64_t roots = 1ull << sl.depth, segs = uint64_t(sl.grid) + roots;
+      uint64_t used = 0;
+      auto take = [&](uint64_t bytes) {
+        uint8_t *q = spare + used;
+        used += align_up(bytes);
+        return reinterpret_cast<uint32_t *>(q);
+      };
+      sl.node = reinterpret_cast<uint8_t *>(take(n + 64));
+      sl.seglow = take(segs * kSplitLow * 4);
+      sl.segcnt = take((kSplitParts * uint64_t(sl.grid) + roots) * 4 << kSplitMaxLevels);
+      sl.ties = take(4 * n);
+      if (sl.depth > 0) {
+        sl.state = take(segs * kSplitStateWords * 4);
+        sl.seghist = take(2 * roots * kSplitBins * 4);
+      }
+      if (used > spare_bytes) break;
+      sl.barrier = reinterpret_cast<uint32_t *>(ws + p.off_split) + 32 * launches;
+      sl.hist = reinterpret_cast<uint32_t *>(ws + p.off_split) + 32 * kSplitLaunches;
+      sl.low = sl.hist + split_roots_max(n) * 2 * kSplitBins;
+      for (int d = 0; d < 3; ++d) {
+        sl.root_hi[d] = L.qmax[d];
+        sl.src[d] = static_cast<const uint16_t *>(src[d]);
+        sl.dst[d] = static_cast<uint16_t *>(dst[d]);
+      }
+      sl.src_idx = isrc;
+      sl.dst_idx = idst;
+      sl.parents = sl.depth > 0 ? nodes + ((1ull << (sl.depth - 1)) - 1) : nullptr;
+      sl.out_nodes = nodes + ((1ull << (sl.depth + sl.levels - 1)) - 1);
+      sl.clear = sl.levels < left;
+      sl.err = err;
+      PC_TRY(launch_split(sl, st));
+      if (facts)
+        for (int l = sl.depth; l < sl.depth + sl.levels; ++l) facts->hbm_levels |= 1ull << l;
+      void **t = src;
+      src = dst;
+      dst = t;
+      uint32_t *ti = isrc;
+      isrc = idst;
+      idst = ti;
+      src_depth = sl.depth + sl.levels;
+    }
+    for (int l = src_depth; l < global_levels; ++l) {
       if (p.tune && l >= first_depth) {
         uint64_t bytes = 0;
         rc = depth_cost(src, l, &bytes);
@@ -1218,10 +1324,10 @@ int knob_find(uint64_t key, uint32_t leaf_size, bool claim, bool *claimed) {
 // same stream into `out` (its size is checked).
 int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config &base,
                void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-               uint32_t *perm, cudaStream_t st, uint32_t *node_max, uint32_t *leaf_max) {
+               uint32_t *perm, cudaStream_t st, int share, uint32_t *node_max, uint32_t *leaf_max) {
   RunFacts facts;
   int rc = compress_impl(positions, n, dtype, eb_mode, eb, &base, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st, nullptr, &facts);
+                         workspace_bytes, perm, st, share, nullptr, &facts);
   if (rc) return rc;
   const uint64_t size0 = *out_size;
   uint32_t best_node = base.warp_node_max ? base.warp_node_max : PC_DEFAULT_WARP_NODE_MAX;
@@ -1235,7 +1341,7 @@ int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double
       uint64_t size = 0;
       const auto t0 = std::chrono::steady_clock::now();
       const int r = compress_impl(positions, n, dtype, eb_mode, eb, &c, out, out_capacity, &size, workspace,
-                                  workspace_bytes, perm, st);
+                                  workspace_bytes, perm, st, share);
       const double t = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
       if (r) return r;
       if (size != size0) return PC_ERR_CUDA;  // a launch knob changed the stream: never expected
@@ -1306,10 +1412,10 @@ int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double
 // the call's class (tuning the class when this call is its first).
 int compress_entry(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                    void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                   uint32_t *perm, cudaStream_t st) {
+                   uint32_t *perm, cudaStream_t st, int share = 1) {
   if (!cfg || !(cfg->flags & PC_FLAG_AUTOTUNE_KNOBS))
     return compress_impl(positions, n, dtype, eb_mode, eb, cfg, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st);
+                         workspace_bytes, perm, st, share);
   pc_config base = *cfg;
   base.flags &= ~PC_FLAG_AUTOTUNE_KNOBS;
   {
@@ -1337,10 +1443,10 @@ int compress_entry(const void *positions, uint64_t n, int dtype, int eb_mode, do
   }
   if (!claimed)
     return compress_impl(positions, n, dtype, eb_mode, eb, &base, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st);
+                         workspace_bytes, perm, st, share);
   uint32_t node_max = 0, leaf_max = 0;
   const int rc = tune_knobs(positions, n, dtype, eb_mode, eb, base, out, out_capacity, out_size, workspace,
-                            workspace_bytes, perm, st, &node_max, &leaf_max);
+                            workspace_bytes, perm, st, share, &node_max, &leaf_max);
   std::lock_guard<std::mutex> g(g_knob_mu);
   if (g_knob_gen == gen) {
     if (rc == PC_OK) {
@@ -1360,9 +1466,9 @@ namespace pcx {
 
 int compress_device(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                     void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                    cudaStream_t st) {
+                    cudaStream_t st, int share) {
   return compress_entry(positions, n, dtype, eb_mode, eb, cfg, out, out_capacity, out_size, workspace,
-                        workspace_bytes, nullptr, st);
+                        workspace_bytes, nullptr, st, share);
 }
 
 }  // namespace pcx
@@ -1520,7 +1626,7 @@ int pc_leaf_size_sweep(const void *positions, uint64_t n, int dtype, int eb_mode
   pc_config cfg = {r_max, PC_FLAG_AUTOTUNE_LEAF};
   Sweep sw = {points, capacity, 0, r_min};
   int rc = compress_impl(positions, n, dtype, eb_mode, eb, &cfg, nullptr, 0, nullptr, workspace, workspace_bytes,
-                         nullptr, static_cast<cudaStream_t>(stream), &sw);
+                         nullptr, static_cast<cudaStream_t>(stream), 1, &sw);
   *count = sw.count;
   return rc;
 }

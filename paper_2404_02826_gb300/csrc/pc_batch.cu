@@ -417,6 +417,8 @@ struct pc_server {
         cv_work.wait(lk);
       }
       ++running;
+      // compressions that may run beside this one
+      const int share = int(std::min<uint64_t>(lanes.size(), running + queue.size()));
       lk.unlock();
       pc_completion c = {};
       c.tag = job.req.tag;
@@ -429,7 +431,7 @@ struct pc_server {
         pc_config cfg = {r.leaf_size, r.flags};
         uint64_t size = 0;
         c.status = pcx::compress_device(r.input, r.n, r.dtype, r.eb_mode, r.eb, &cfg, base + ooff, obytes, &size,
-                                        base + soff, sbytes, s);
+                                        base + soff, sbytes, s, share);
         c.output_bytes = size;
       } else {
         c.status = pc_decompress(r.input, r.input_bytes, base + ooff, obytes, base + soff, sbytes, s);
@@ -487,7 +489,7 @@ int pc_compress_batch(pc_compress_item *items, uint32_t count, uint32_t lanes, v
     pc_config cfg = {it.leaf_size, it.flags};
     uint64_t size = 0;
     it.status = pcx::compress_device(it.positions, it.n, it.dtype, it.eb_mode, it.eb, &cfg, it.out, it.out_capacity,
-                                     &size, ws + lane * slice, slice, s);
+                                     &size, ws + lane * slice, slice, s, int(lanes));
     it.out_size = it.status == PC_OK ? size : 0;
   });
   if (rc) return rc;

@@ -188,6 +188,41 @@ struct LevelLaunch {
 };
 cudaError_t launch_level(const LevelLaunch &a, cudaStream_t st);
 cudaError_t launch_scatter(const LevelLaunch &a, cudaStream_t st);
+// Several levels in one cooperative launch (k_split.cu): 16-bit codes, split
+// axis depth mod 3, every node above depth + levels larger than a leaf.
+constexpr int kSplitMaxLevels = 7;         // a particle's node below its subroot fits a byte
+constexpr uint32_t kSplitBins = 16384;     // counters of one level's histogram, shared by its nodes
+constexpr uint32_t kSplitLow = 4096;       // counters of the codes in the nodes' median bins
+constexpr uint32_t kSplitStateWords = 17u << (kSplitMaxLevels - 1);
+constexpr int kSplitParts = 2;             // parts of a CTA's positions, one per CTA of the move
+constexpr uint32_t kSplitMaxRoots = 512;   // subroots of one launch
+struct SplitLaunch {
+  uint64_t n;
+  int depth, levels;          // the subroots' depth, levels below them (1 .. kSplitMaxLevels)
+  int grid;                   // CTAs, at most one per SM
+  uint32_t chunk;             // positions per CTA, a multiple of 16
+  uint32_t root_hi[3];        // codes of axis d lie in [0, root_hi[d]]
+  const LevelNode *parents;   // the records of depth - 1 (null at depth 0)
+  LevelNode *out_nodes;       // the records of depth + levels - 1 (written)
+  const uint16_t *src[3];     // arrangement at depth
+  uint16_t *dst[3];           // arrangement at depth + levels (written)
+  const uint32_t *src_idx;    // optional
+  uint32_t *dst_idx;
+  uint8_t *node;              // [n + 64] scratch: node below the subroot
+  uint32_t *hist;             // [2][2^depth][kSplitBins], zero on entry
+  uint32_t *low;              // [2][2^depth][kSplitLow], zero on entry
+  uint32_t part;              // positions per CTA of the move (set by launch_split)
+  // scratch; a segment is what a CTA holds of a subroot (at most grid + 2^depth of them)
+  uint32_t *seglow;           // [kSplitLow][grid + 2^depth] codes in the median bins, by segment
+  uint32_t *segcnt;           // [2^kSplitMaxLevels][kSplitParts grid + 2^depth] children, by part of a segment
+  uint32_t *ties;             // [n] positions of ties
+  uint32_t *state;            // [grid + 2^depth][kSplitStateWords] (depth > 0)
+  uint32_t *seghist;          // [2^(depth + 1)][kSplitBins] (depth > 0)
+  bool clear;                 // leave hist and low zero (another launch uses them)
+  uint32_t *barrier;          // zero on entry
+  uint32_t *err;
+};
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st);
 uint32_t scatter_tile(int code_bytes, bool with_idx);    // largest tile of one scatter CTA
 uint32_t scatter_groups(int code_bytes, bool with_idx);  // 16-byte group records per tile
 
@@ -403,9 +438,10 @@ cudaError_t resident_blocks(int threads, size_t smem, int *per_sm) {
 // Self-test switch of the calling host thread: its compress calls issue no
 // tile copy in the partition's scatter (pc_selftest_scatter_timeout).
 void set_drop_tile_copies(bool on);
-// pc_compress without the optional permutation, on a caller-provided workspace.
+// pc_compress without the optional permutation, on a caller-provided workspace;
+// `share`: compressions that run at the same time (the lanes of a batch or a server).
 int compress_device(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                     void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                    cudaStream_t st);
+                    cudaStream_t st, int share = 1);
 
 }  // namespace pcx
