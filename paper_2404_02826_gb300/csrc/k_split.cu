@@ -84,7 +84,7 @@ struct Misc {
   uint32_t b0, b1;              // current segment
   uint32_t clo;                 // first CTA of the current subroot
   uint32_t shift, nbins;
-  uint32_t ties;                // listed ties of the segment
+  uint32_t ties, many;          // listed ties of the segment; whether a node has more than a warp selects among
   uint32_t fd, fbefore;         // tie selection: digit, ties below it
   uint32_t wt[kW + 1];
   uint32_t wh[kW][32];
@@ -100,15 +100,20 @@ struct Smem {
 static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
 static_assert(offsetof(Smem, bins) % 16 == 0 && offsetof(Smem, sum) % 16 == 0, "16-byte accesses");
 
-// Grid barrier; bounded.  True when it gave up or the call has failed: the
+// Grid barrier in two halves: between them a CTA does what no other CTA waits
+// for.  Bounded; the wait is true when it gave up or the call has failed: the
 // caller leaves the kernel, as every other CTA does at its next barrier.
-__device__ __forceinline__ bool grid_sync(const SplitLaunch &a, uint32_t &epoch) {
+__device__ __forceinline__ void grid_arrive(const SplitLaunch &a) {
   __syncthreads();
-  bool bad = false;
-  ++epoch;
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(a.barrier, 1u);
+  }
+}
+__device__ __forceinline__ bool grid_wait(const SplitLaunch &a, uint32_t &epoch) {
+  bool bad = false;
+  ++epoch;
+  if (threadIdx.x == 0) {
     const uint32_t want = epoch * gridDim.x;
     uint32_t spins = 0;
     for (;;) {
@@ -130,6 +135,10 @@ __device__ __forceinline__ bool grid_sync(const SplitLaunch &a, uint32_t &epoch)
   }
   return __syncthreads_or(bad) != 0;
 }
+__device__ __forceinline__ bool grid_sync(const SplitLaunch &a, uint32_t &epoch) {
+  grid_arrive(a);
+  return grid_wait(a, epoch);
+}
 
 __device__ __forceinline__ uint32_t half_of(const uint4 &w, int e) {
   const uint32_t x = e < 2 ? w.x : (e < 4 ? w.y : (e < 6 ? w.z : w.w));
@@ -146,8 +155,8 @@ struct Ctx {
   int lane, warp;
 };
 
-// The segment of subroot s (thread 0 fills the geometry), its kept state when
-// the CTA has several (`load`), and the places of the nodes of level l.
+// The segment of subroot s (thread 0 fills the geometry) and its kept state when
+// the CTA has several (`load`), else at level 0 the subroot's bounds.
 __device__ __forceinline__ void enter_seg(const Ctx &x, uint32_t s, int l, bool load) {
   const SplitLaunch &a = x.a;
   __syncthreads();
@@ -183,13 +192,6 @@ __device__ __forceinline__ void enter_seg(const Ctx &x, uint32_t s, int l, bool 
     x.N.bhi[0][d][0] = hi;
   }
   __syncthreads();
-  if (l < a.levels && threadIdx.x < (1u << l)) {
-    uint64_t off, cnt;
-    node_range(x.M.scnt, l, threadIdx.x, off, cnt);
-    x.N.roff[threadIdx.x] = uint32_t(off);
-    x.N.rcnt[threadIdx.x] = uint32_t(cnt);
-  }
-  __syncthreads();
 }
 
 __device__ __forceinline__ void keep_seg(const Ctx &x, uint32_t s) {
@@ -199,10 +201,13 @@ __device__ __forceinline__ void keep_seg(const Ctx &x, uint32_t s) {
   for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
 }
 
-// Bins of level l: the smallest shift whose bins fit, and every node's offset.
-__device__ __forceinline__ void level_bins(const Ctx &x, int l) {
-  const int ax = (x.a.depth + l) % 3, p = l & 1;
-  if (x.warp == 0) {
+// Level l of the segment, by different warps: the smallest shift whose bins fit
+// and every node's offset (warp 0); the tie list of the level above, a run of
+// `mine` places per node with an odd plane (warp 1); the nodes' places in the
+// subroot.  l == levels: the tie list alone.
+__device__ __forceinline__ void level_setup(const Ctx &x, int l) {
+  if (x.warp == 0 && l < x.a.levels) {
+    const int ax = (x.a.depth + l) % 3, p = l & 1;
     const uint32_t nodes = 1u << l;
     const uint32_t j0 = 2 * x.lane, j1 = j0 + 1;
     const bool v0 = j0 < nodes, v1 = j1 < nodes;
@@ -228,14 +233,8 @@ __device__ __forceinline__ void level_bins(const Ctx &x, int l) {
       x.M.shift = sh;
       x.M.nbins = min(tot, kBins);
     }
-  }
-  __syncthreads();
-}
-
-// Lays out the segment's tie list: a run of `mine` places per node with an odd plane.
-__device__ __forceinline__ void tie_lists(const Ctx &x, uint32_t half) {
-  if (x.warp == 0) {
-    const uint32_t j0 = 2 * x.lane, j1 = j0 + 1;
+  } else if (x.warp == 1) {
+    const uint32_t half = (1u << l) >> 1, j0 = 2 * x.lane, j1 = j0 + 1;
     const uint32_t t0 = j0 < half && (x.N.plane[j0] & 1u) ? x.N.mine[j0] : 0u;
     const uint32_t t1 = j1 < half && (x.N.plane[j1] & 1u) ? x.N.mine[j1] : 0u;
     uint32_t incl = t0 + t1;
@@ -247,7 +246,16 @@ __device__ __forceinline__ void tie_lists(const Ctx &x, uint32_t half) {
     const uint32_t ex = incl - t0 - t1;
     x.N.lbase[j0] = x.N.cursor[j0] = ex;
     x.N.lbase[j1] = x.N.cursor[j1] = ex + t0;
-    if (x.lane == 31) x.M.ties = incl;
+    const bool many = __any_sync(0xffffffffu, max(t0, t1) > kTieWarp);
+    if (x.lane == 31) {
+      x.M.ties = incl;
+      x.M.many = many;
+    }
+  } else if (l < x.a.levels && threadIdx.x >= 64 && threadIdx.x - 64 < (1u << l)) {
+    uint64_t off, cnt;
+    node_range(x.M.scnt, l, threadIdx.x - 64, off, cnt);
+    x.N.roff[threadIdx.x - 64] = uint32_t(off);
+    x.N.rcnt[threadIdx.x - 64] = uint32_t(cnt);
   }
   __syncthreads();
 }
@@ -332,46 +340,63 @@ __device__ __forceinline__ uint32_t move_part(const SplitLaunch &a, uint32_t pos
   return c * kSplitParts + min((pos - c * a.chunk) / a.part, uint32_t(kSplitParts - 1));
 }
 
-// A pass over the segment.  FIRST: level 0, nothing to classify.  LAST: the
-// final children are counted instead of codes.  TIES: ties of some node are listed.
-template <bool FIRST, bool LAST, bool TIES>
-__device__ __forceinline__ void pass_a(const Ctx &x, const uint16_t *__restrict__ prev, const uint16_t *__restrict__ cur,
-                                       uint32_t half, uint32_t *list) {
+// 8 consecutive particles: their codes on the axis of the level above and on
+// this one's, and their nodes.
+struct Step {
+  uint4 p, c;
+  uint2 n;
+};
+// What a pass reads.  FIRST: level 0, nothing to classify.  LAST: F, which counts
+// children per part of the chunk and warp instead of codes.
+struct Pass {
+  const uint16_t *prev, *cur;
+  uint32_t half;  // nodes of the level above
+};
+template <bool FIRST, bool LAST>
+__device__ __forceinline__ void load_step(const Ctx &x, const Pass &a, Step &t, uint32_t pos) {
+  if (!FIRST) {
+    t.p = __ldcg(reinterpret_cast<const uint4 *>(a.prev + pos));
+    if (a.half > 1) t.n = __ldcg(reinterpret_cast<const uint2 *>(x.a.node + pos));
+    else t.n = make_uint2(0, 0);  // the subroot itself
+  }
+  if (!LAST) t.c = __ldcg(reinterpret_cast<const uint4 *>(a.cur + pos));
+}
+// The pass's first step, loaded ahead of the level's setup.
+template <bool FIRST, bool LAST>
+__device__ __forceinline__ void first_step(const Ctx &x, const Pass &a, Step &t) {
+  const uint32_t pos = (x.M.b0 & ~7u) + 8u * threadIdx.x;
+  if (pos < x.M.b1) load_step<FIRST, LAST>(x, a, t, pos);
+}
+
+// A pass over the segment, whose first step is loaded.  The ties of nodes with
+// an odd plane go right and are listed; there is no variant without the list,
+// since a barrier waits for the CTAs that list anyway and code that runs for the
+// first time costs microseconds of instruction fetches (at 2^20 particles 104 us
+// a launch with both variants, 94 with one).
+template <bool FIRST, bool LAST>
+__device__ __forceinline__ void pass_a(const Ctx &x, const Pass &a, Step &next, uint32_t *list) {
   NodeTab &N = x.N;
   const uint32_t b0 = x.M.b0, b1 = x.M.b1, shift = x.M.shift;
   uint8_t *const nid = x.a.node;
-  const int32_t off0 = FIRST ? N.off[0] : 0;
-  const uint32_t room = TIES ? x.M.ties : 0u;
+  const uint32_t room = x.M.ties;
   uint32_t pos = (b0 & ~7u) + 8u * threadIdx.x;
-  uint4 np = make_uint4(0, 0, 0, 0), nc = np;
-  uint2 nn = make_uint2(0, 0);
-  auto load = [&](uint32_t p) {
-    if (!FIRST) {
-      np = __ldcg(reinterpret_cast<const uint4 *>(prev + p));
-      if (half > 1) nn = __ldcg(reinterpret_cast<const uint2 *>(nid + p));  // else the subroot itself, node 0
-    }
-    if (!LAST) nc = __ldcg(reinterpret_cast<const uint4 *>(cur + p));
-  };
-  if (pos < b1) load(pos);
   for (; pos < b1; pos += kStep) {
-    const uint4 p = np, c = nc;
-    const uint2 n0 = nn;
-    if (pos + kStep < b1) load(pos + kStep);
+    const uint4 p = next.p, c = next.c;
+    const uint2 n0 = next.n;
+    if (pos + kStep < b1) load_step<FIRST, LAST>(x, a, next, pos + kStep);
     uint32_t mask = 0xffu;
     if (pos < b0) mask &= 0xffu << (b0 - pos);
     if (pos + 8u > b1) mask &= 0xffu >> (pos + 8u - b1);
     uint32_t *const bins = LAST ? x.bins + (part_of(x.a, pos) * kW + x.warp) * kNodes : x.bins;
-    uint32_t w0 = 0, w1 = 0;
+    const int32_t off0 = FIRST ? N.off[0] : 0;
+    uint32_t w0 = 0, w1 = 0, hit = 0;
     auto one = [&](int e) {
       uint32_t child = 0;
       if (!FIRST) {
         const uint32_t j = byte_of(n0, e) & (kHalf - 1);
         const uint32_t pl = N.plane[j], t = 2 * half_of(p, e) + 1;
         child = 2 * j + (t >= pl ? 1u : 0u);
-        if (TIES && t == pl) {
-          const uint32_t at = atomicAdd(&N.cursor[j], 1u);
-          if (at + 1u <= room) list[at] = pos + uint32_t(e);
-        }
+        if (t == pl) hit |= 1u << e;
         if (e < 4) w0 |= child << (8 * e);
         else w1 |= child << (8 * (e - 4));
       }
@@ -383,13 +408,19 @@ __device__ __forceinline__ void pass_a(const Ctx &x, const uint16_t *__restrict_
       for (int e = 0; e < 8; ++e) one(e);
       if (!FIRST) *reinterpret_cast<uint2 *>(nid + pos) = make_uint2(w0, w1);
     } else {
-#pragma unroll
+#pragma unroll 1
       for (int e = 0; e < 8; ++e)
-        if ((mask >> e) & 1u) one(e);
-      if (!FIRST) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if ((mask >> e) & 1u) nid[pos + e] = uint8_t((e < 4 ? w0 : w1) >> (8 * (e & 3)));
+        if ((mask >> e) & 1u) {
+          one(e);
+          if (!FIRST) nid[pos + e] = uint8_t((e < 4 ? w0 : w1) >> (8 * (e & 3)));
+        }
+    }
+    for (; hit; hit &= hit - 1) {
+      const int e = __ffs(hit) - 1;
+      const uint32_t at = atomicAdd(&N.cursor[byte_of(n0, e) & (kHalf - 1)], 1u);
+      if (at < room) {
+        list[at] = pos + uint32_t(e);
+        if (!LAST && room <= kBins / 2) list[at + kBins / 2] = half_of(c, e);
       }
     }
   }
@@ -398,8 +429,7 @@ __device__ __forceinline__ void pass_a(const Ctx &x, const uint16_t *__restrict_
 // The listed ties, all counted as going right so far: the first `quota` of each
 // node in position order go left after all.
 template <bool LAST>
-__device__ __forceinline__ void resolve_ties(const Ctx &x, const uint16_t *__restrict__ cur, uint32_t half,
-                                             const uint32_t *list) {
+__device__ __forceinline__ void resolve_ties(const Ctx &x, const Pass &a, const uint32_t *list) {
   NodeTab &N = x.N;
   const uint32_t b0 = x.M.b0, shift = x.M.shift;
   const int bits = int(bit_length(x.M.b1 - b0));
@@ -409,17 +439,17 @@ __device__ __forceinline__ void resolve_ties(const Ctx &x, const uint16_t *__res
       const uint32_t p = l[i];
       if (p >= limit) continue;
       x.a.node[p] = uint8_t(2 * j);
-      uint32_t *l_, *r_;
+      uint32_t *left, *right;
       if (LAST) {
-        l_ = x.bins + (part_of(x.a, p) * kW + x.warp) * kNodes + 2 * j;
-        r_ = l_ + 1;
-      } else {
-        const int32_t b = int32_t(uint32_t(__ldcg(cur + p)) >> shift);
-        l_ = x.bins + (uint32_t(b + N.off[2 * j]) & (kBins - 1));
-        r_ = x.bins + (uint32_t(b + N.off[2 * j + 1]) & (kBins - 1));
+        left = x.bins + (part_of(x.a, p) * kW + x.warp) * kNodes + 2 * j;
+        right = left + 1;
+      } else {  // the code lies beside a list of up to half the room
+        const uint32_t c = x.M.ties <= kBins / 2 ? l[i + kBins / 2] : uint32_t(__ldcg(a.cur + p));
+        left = x.bins + (uint32_t(int32_t(c >> shift) + N.off[2 * j]) & (kBins - 1));
+        right = x.bins + (uint32_t(int32_t(c >> shift) + N.off[2 * j + 1]) & (kBins - 1));
       }
-      atomicAdd(l_, 1u);
-      atomicSub(r_, 1u);
+      atomicAdd(left, 1u);
+      atomicSub(right, 1u);
     }
   };
   // a node whose list is not full (never expected) is left alone, and the call fails
@@ -428,13 +458,14 @@ __device__ __forceinline__ void resolve_ties(const Ctx &x, const uint16_t *__res
     atomicOr(x.a.err, kErrInternal);
     return false;
   };
-  for (uint32_t j = x.warp; j < half; j += kW) {
+  for (uint32_t j = x.warp; j < a.half; j += kW) {
     if (!(N.plane[j] & 1u) || N.mine[j] > kTieWarp || !full(j)) continue;
     const uint32_t limit = select_warp(list + N.lbase[j], N.mine[j], N.quota[j], b0, bits, x.M.wh[x.warp], x.lane);
     fix(j, x.lane, 32, limit);
     __syncwarp();
   }
-  for (uint32_t j = 0; j < half; ++j) {
+  if (!x.M.many) return;
+  for (uint32_t j = 0; j < a.half; ++j) {
     if (!(N.plane[j] & 1u) || N.mine[j] <= kTieWarp || !full(j)) continue;
     const uint32_t limit = select_block(x.M, list + N.lbase[j], N.mine[j], N.quota[j], b0, bits);
     fix(j, threadIdx.x, kT, limit);
@@ -442,17 +473,15 @@ __device__ __forceinline__ void resolve_ties(const Ctx &x, const uint16_t *__res
 }
 
 template <bool FIRST, bool LAST>
-__device__ __forceinline__ void run_a(const Ctx &x, const uint16_t *prev, const uint16_t *cur, uint32_t half) {
-  if (!FIRST && x.M.ties) {
-    // in shared memory when they fit, else in this segment's part of the global list
-    uint32_t *list = x.M.ties <= kBins ? x.sum : x.a.ties + x.M.b0;
-    pass_a<FIRST, LAST, true>(x, prev, cur, half, list);
-    __syncthreads();
-    resolve_ties<LAST>(x, cur, half, list);
-  } else {
-    pass_a<FIRST, LAST, false>(x, prev, cur, half, nullptr);
-  }
+__device__ __forceinline__ void run_a(const Ctx &x, const Pass &a, Step &t) {
+  // in shared memory when the list fits, else in this segment's part of the global one
+  uint32_t *const list = x.M.ties <= kBins ? x.sum : x.a.ties + x.M.b0;
+  pass_a<FIRST, LAST>(x, a, t, list);
   __syncthreads();
+  if (!FIRST && x.M.ties) {
+    resolve_ties<LAST>(x, a, list);
+    __syncthreads();
+  }
 }
 
 // B: the particles in their node's median bin, counted per code.
@@ -502,6 +531,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     const uint64_t r0 = uint64_t(c) * a.chunk;
     M.s0 = 1;
     M.s1 = 0;
+    M.nbins = 0;
     if (r0 < a.n) {  // the subroots holding the first and the last position
       const uint64_t r1 = min(r0 + a.chunk, a.n) - 1;
       for (int e = 0; e < 2; ++e) {
@@ -530,19 +560,21 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     uint32_t *const hist = a.hist + uint64_t(l & 1) * S * kBins;
     uint32_t *const low = a.low + uint64_t(l & 1) * S * kLow;
     // ---- A ----
-    if (l > 0) {  // the other histogram was read by every CTA before the last barrier
-      uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * kBins);
-      for (uint32_t i = gtid; i < S * (kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
-    }
+    Step step;
+    const Pass pa = {prev, cur, half};
+    if (!multi && l > 0 && s0 <= s1) first_step<false, false>(x, pa, step);
     for (uint32_t s = s0; s <= s1; ++s) {
-      enter_seg(x, s, l, multi && l > 0);
-      level_bins(x, l);
-      tie_lists(x, half);
+      if (multi || l == 0) enter_seg(x, s, l, multi && l > 0);
+      if (multi && l > 0) first_step<false, false>(x, pa, step);
+      if (l == 0) first_step<true, false>(x, pa, step);
+      level_setup(x, l);
       const uint32_t nbins = M.nbins;
-      for (uint32_t b = threadIdx.x; b < nbins; b += kT) P.bins[b] = 0;
-      __syncthreads();
-      if (l == 0) run_a<true, false>(x, prev, cur, half);
-      else run_a<false, false>(x, prev, cur, half);
+      if (multi || l == 0) {  // else zeroed after their last use
+        for (uint32_t b = threadIdx.x; b < (multi ? nbins : kBins); b += kT) P.bins[b] = 0;
+        __syncthreads();
+      }
+      if (l == 0) run_a<true, false>(x, pa, step);
+      else run_a<false, false>(x, pa, step);
       uint32_t *const h = hist + uint64_t(s) * kBins;
       uint32_t *const own = a.seghist + uint64_t(2 * s + (c != M.clo)) * kBins;
       for (uint32_t b = threadIdx.x; b < nbins; b += kT) {
@@ -552,16 +584,17 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       }
       if (multi) keep_seg(x, s);
     }
-    if (grid_sync(a, epoch)) return;
-    // ---- sel1 and B ----
-    if (l > 0) {
-      uint4 *z = reinterpret_cast<uint4 *>(a.low + uint64_t((l + 1) & 1) * S * kLow);
-      for (uint32_t i = gtid; i < S * (kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+    grid_arrive(a);
+    if (l > 0) {  // the other histogram was read by every CTA before the last barrier
+      uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * kBins);
+      for (uint32_t i = gtid; i < S * (kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
     }
+    if (grid_wait(a, epoch)) return;
+    // ---- sel1 and B ----
     for (uint32_t s = s0; s <= s1; ++s) {
       if (multi) {
         enter_seg(x, s, l, l > 0);
-        level_bins(x, l);
+        level_setup(x, l);
       }
       const uint32_t nbins = M.nbins, shift = M.shift;
       {  // exclusive prefixes within each warp's 512 bins, and the warps' totals
@@ -605,21 +638,23 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
         __syncthreads();
         if (warp == 0) M.wt[lane] = wb;
         __syncthreads();
-        if (threadIdx.x < nodes) {
-          // the last bin of the node whose prefix does not exceed the median's rank
-          const uint32_t j = threadIdx.x;
-          const int ax = (a.depth + l) % 3;
-          const uint32_t cl = N.blo[l & 1][ax][j] >> shift, ch = N.bhi[l & 1][ax][j] >> shift;
+        // per node, by a warp: the last of its bins whose prefix does not exceed the median's rank
+        const int ax = (a.depth + l) % 3;
+        for (uint32_t j = warp; j < nodes; j += kW) {
           const uint32_t target = N.roff[j] + (N.rcnt[j] >> 1);
-          uint32_t lo = uint32_t(N.off[j] + int32_t(cl)), hi = uint32_t(N.off[j] + int32_t(ch));
-          if (hi >= kBins) hi = kBins - 1;
+          uint32_t lo = uint32_t(N.off[j] + int32_t(N.blo[l & 1][ax][j] >> shift));
+          uint32_t hi = min(uint32_t(N.off[j] + int32_t(N.bhi[l & 1][ax][j] >> shift)), kBins - 1u);
           while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (M.wt[mid / kPer] + P.sum[mid] <= target) lo = mid;
-            else hi = mid - 1;
+            const uint32_t by = (hi - lo) / 32u + 1u, at = lo + by * lane;
+            const bool le = at <= hi && M.wt[min(at, kBins - 1u) / kPer] + P.sum[min(at, kBins - 1u)] <= target;
+            const uint32_t m = __ballot_sync(0xffffffffu, le);
+            lo += by * (m ? 31u - uint32_t(__clz(m)) : 0u);
+            hi = min(hi, lo + by - 1u);
           }
-          N.bk[j] = uint32_t(int32_t(lo) - N.off[j]);
-          N.below[j] = M.wt[lo / kPer] + P.sum[lo] - N.roff[j];
+          if (lane == 0) {
+            N.bk[j] = uint32_t(int32_t(lo) - N.off[j]);
+            N.below[j] = M.wt[lo / kPer] + P.sum[lo] - N.roff[j];
+          }
         }
         __syncthreads();
       }
@@ -645,12 +680,19 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       }
       if (multi) keep_seg(x, s);
     }
-    if (grid_sync(a, epoch)) return;
+    grid_arrive(a);
+    if (l > 0) {  // read by every CTA before the barrier before
+      uint4 *z = reinterpret_cast<uint4 *>(a.low + uint64_t((l + 1) & 1) * S * kLow);
+      for (uint32_t i = gtid; i < S * (kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+    }
+    if (!multi)
+      for (uint32_t b = threadIdx.x; b < M.nbins; b += kT) P.bins[b] = 0;
+    if (grid_wait(a, epoch)) return;
     // ---- sel2: a warp per node ----
     for (uint32_t s = s0; s <= s1; ++s) {
       if (multi) {
         enter_seg(x, s, l, true);
-        level_bins(x, l);
+        level_setup(x, l);
       }
       const uint32_t shift = M.shift;
       const int ax = (a.depth + l) % 3;
@@ -727,11 +769,14 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
   // ---- F: final children, counted per segment and part of the chunk ----
   const uint32_t half = 1u << (K - 1);
   for (uint32_t s = s0; s <= s1; ++s) {
-    enter_seg(x, s, K, multi);
-    tie_lists(x, half);
+    Step step;
+    const Pass pf = {a.src[(a.depth + K + 2) % 3], nullptr, half};
+    if (multi) enter_seg(x, s, K, true);
+    first_step<false, true>(x, pf, step);
+    level_setup(x, K);
     for (uint32_t b = threadIdx.x; b < kSplitParts * kW * kNodes; b += kT) P.bins[b] = 0;
     __syncthreads();
-    run_a<false, true>(x, a.src[(a.depth + K + 2) % 3], nullptr, half);
+    run_a<false, true>(x, pf, step);
     for (uint32_t i = threadIdx.x; i < kSplitParts * kNodes; i += kT) {
       const uint32_t q = i / kNodes, b = i % kNodes;
       if (q < part_of(a, M.b0) || q > part_of(a, M.b1 - 1) || b >= 2 * half) continue;
