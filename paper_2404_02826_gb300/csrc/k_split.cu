@@ -201,6 +201,18 @@ __device__ __forceinline__ void keep_seg(const Ctx &x, uint32_t s) {
   for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
 }
 
+constexpr int kPerLane = int(kHalf) / 32;  // nodes of a lane
+
+__device__ __forceinline__ uint32_t warp_excl(uint32_t v, int lane) {
+  uint32_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  return incl - v;
+}
+
 // Level l of the segment, by different warps: the smallest shift whose bins fit
 // and every node's offset (warp 0); the tie list of the level above, a run of
 // `mine` places per node with an odd plane (warp 1); the nodes' places in the
@@ -209,46 +221,54 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
   if (x.warp == 0 && l < x.a.levels) {
     const int ax = (x.a.depth + l) % 3, p = l & 1;
     const uint32_t nodes = 1u << l;
-    const uint32_t j0 = 2 * x.lane, j1 = j0 + 1;
-    const bool v0 = j0 < nodes, v1 = j1 < nodes;
-    const uint32_t l0 = v0 ? x.N.blo[p][ax][j0] : 0, h0 = v0 ? x.N.bhi[p][ax][j0] : 0;
-    const uint32_t l1 = v1 ? x.N.blo[p][ax][j1] : 0, h1 = v1 ? x.N.bhi[p][ax][j1] : 0;
-    uint32_t sh = 0, c0, c1, tot;
+    uint32_t lo[kPerLane], hi[kPerLane], c[kPerLane];
+#pragma unroll
+    for (int i = 0; i < kPerLane; ++i) {
+      const uint32_t j = kPerLane * x.lane + i;
+      lo[i] = j < nodes ? x.N.blo[p][ax][j] : 1;
+      hi[i] = j < nodes ? x.N.bhi[p][ax][j] : 0;
+    }
+    uint32_t sh = 0, sum, tot;
     for (;; ++sh) {
-      c0 = v0 ? (h0 >> sh) - (l0 >> sh) + 1u : 0u;
-      c1 = v1 ? (h1 >> sh) - (l1 >> sh) + 1u : 0u;
-      tot = __reduce_add_sync(0xffffffffu, c0 + c1);
+      sum = 0;
+#pragma unroll
+      for (int i = 0; i < kPerLane; ++i) {
+        c[i] = kPerLane * x.lane + i < nodes ? (hi[i] >> sh) - (lo[i] >> sh) + 1u : 0u;
+        sum += c[i];
+      }
+      tot = __reduce_add_sync(0xffffffffu, sum);
       if (tot <= kBins || sh >= 16) break;
     }
-    uint32_t incl = c0 + c1;
+    uint32_t ex = warp_excl(sum, x.lane);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (x.lane >= o) incl += y;
+    for (int i = 0; i < kPerLane; ++i) {
+      const uint32_t j = kPerLane * x.lane + i;
+      if (j < nodes) x.N.off[j] = int32_t(ex) - int32_t(lo[i] >> sh);
+      ex += c[i];
     }
-    const uint32_t ex = incl - c0 - c1;
-    if (v0) x.N.off[j0] = int32_t(ex) - int32_t(l0 >> sh);
-    if (v1) x.N.off[j1] = int32_t(ex + c0) - int32_t(l1 >> sh);
     if (x.lane == 0) {
       x.M.shift = sh;
       x.M.nbins = min(tot, kBins);
     }
   } else if (x.warp == 1) {
-    const uint32_t half = (1u << l) >> 1, j0 = 2 * x.lane, j1 = j0 + 1;
-    const uint32_t t0 = j0 < half && (x.N.plane[j0] & 1u) ? x.N.mine[j0] : 0u;
-    const uint32_t t1 = j1 < half && (x.N.plane[j1] & 1u) ? x.N.mine[j1] : 0u;
-    uint32_t incl = t0 + t1;
+    const uint32_t half = (1u << l) >> 1;
+    uint32_t t[kPerLane], sum = 0, most = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (x.lane >= o) incl += y;
+    for (int i = 0; i < kPerLane; ++i) {
+      const uint32_t j = kPerLane * x.lane + i;
+      t[i] = j < half && (x.N.plane[j] & 1u) ? x.N.mine[j] : 0u;
+      sum += t[i];
+      most = max(most, t[i]);
     }
-    const uint32_t ex = incl - t0 - t1;
-    x.N.lbase[j0] = x.N.cursor[j0] = ex;
-    x.N.lbase[j1] = x.N.cursor[j1] = ex + t0;
-    const bool many = __any_sync(0xffffffffu, max(t0, t1) > kTieWarp);
+    uint32_t ex = warp_excl(sum, x.lane);
+#pragma unroll
+    for (int i = 0; i < kPerLane; ++i) {
+      x.N.lbase[kPerLane * x.lane + i] = x.N.cursor[kPerLane * x.lane + i] = ex;
+      ex += t[i];
+    }
+    const bool many = __any_sync(0xffffffffu, most > kTieWarp);
     if (x.lane == 31) {
-      x.M.ties = incl;
+      x.M.ties = ex;
       x.M.many = many;
     }
   } else if (l < x.a.levels && threadIdx.x >= 64 && threadIdx.x - 64 < (1u << l)) {
@@ -658,7 +678,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
         }
         __syncthreads();
       }
-      const uint32_t nlow = min(nodes << shift, kLow);
+      const uint32_t nlow = min(nodes << shift, a.low_cap);
       uint32_t *const sl = a.seglow + c + s;  // counter i of this segment: sl[i * segs]
       const uint64_t segs = gridDim.x + S;
       if (shift == 0) {  // A's counters hold the ties of every node
@@ -722,7 +742,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
           }
         }
         const uint32_t v = (N.bk[j] << shift) | vlow;
-        const uint32_t tleft = target - less, slot = ((j << shift) | vlow) & (kLow - 1);
+        const uint32_t tleft = target - less, slot = min((j << shift) | vlow, a.low_cap - 1u);
         uint32_t before = 0;
         const uint32_t *const row = a.seglow + uint64_t(slot) * (gridDim.x + S) + s;
         const uint32_t mine = __ldcg(row + c);
@@ -832,19 +852,21 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
 constexpr int kMT = 512;
 constexpr int kMW = kMT / 32;
 
-template <bool IDX>
+template <bool IDX, int BITS>
 struct MoveSmem {
-  static constexpr int kRows = IDX ? 8 : 16;                // rows of 32 particles per warp and tile
+  static constexpr uint32_t kCh = 1u << BITS;                   // children, at most
+  static constexpr int kRows = IDX || BITS > 7 ? 8 : 16;        // rows of 32 particles per warp and tile
+  static constexpr int kRankBits = kRows == 16 ? 9 : 8;         // a warp's particles of a tile
   static constexpr uint32_t kTile = uint32_t(kRows) * kMT;
-  static constexpr uint32_t kStage = kTile + kNodes * 14u;  // every child's run padded to whole groups of 8
+  static constexpr uint32_t kStage = kTile + kCh * 14u;         // every child's run padded to whole groups of 8
   alignas(16) uint2 st[kStage];  // x | y << 16, z; place p at stage_slot(p)
-  // per warp: first the nodes of its particles, then child << 9 | rank of every particle
+  // per warp: first the nodes of its particles, then child << kRankBits | rank of every particle
   alignas(16) uint16_t code[kMW][32 * kRows];
   alignas(16) uint32_t sti[IDX ? kStage : 4];
   // counts of a child by warp, then the place in the stage of the warp's first one; 16 bits, so
   // that the counts of 64 children span the 32 banks once
-  uint16_t wcnt[kMW][kNodes + 2];
-  uint32_t tot[kNodes], lst[kNodes], lend[kNodes], gof[kNodes], run[kNodes];
+  uint16_t wcnt[kMW][kCh + 2];
+  uint32_t tot[kCh], lst[kCh], lend[kCh], gof[kCh], run[kCh];
   uint8_t grp[kStage / 8 + 8];
   uint32_t s0, s1, b0, b1, ngroups;
 };
@@ -857,9 +879,9 @@ __device__ __forceinline__ uint32_t stage_slot(uint32_t p) { return p ^ ((p >> 3
 // the segment.  A warp ranks rows of 32 consecutive particles: the lanes with
 // the same child, and the warp's count of that child so far from shared memory.
 template <bool IDX, int BITS, bool WHOLE>
-__device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T, uint4 nodes, uint32_t t0, uint32_t b0,
+__device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX, BITS> &T, uint4 nodes, uint32_t t0, uint32_t b0,
                                           uint32_t b1, uint32_t NB, int lane, int warp) {
-  using V = MoveSmem<IDX>;
+  using V = MoveSmem<IDX, BITS>;
   constexpr int kRows = V::kRows;
   const uint32_t ltm = (1u << lane) - 1u;
   const uint32_t w0 = t0 + uint32_t(warp) * (32 * kRows);  // the warp's first particle
@@ -896,7 +918,7 @@ __device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T
       const uint32_t b = nd[r] & 0xffu, old = wc[b];
       __syncwarp();
       if (inside(w0 + 32 * r + lane)) wc[b] = uint16_t(old + (nd[r] >> 16));  // every lane of the child: the same
-      cb[32 * r + lane] = uint16_t((b << 9) | (old + ((nd[r] >> 8) & 0xffu)));
+      cb[32 * r + lane] = uint16_t((b << V::kRankBits) | (old + ((nd[r] >> 8) & 0xffu)));
       __syncwarp();
     }
   }
@@ -933,7 +955,7 @@ __device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T
   __syncthreads();
   // the children's runs in the stage: whole groups of 8, aligned as their destinations
   if (warp == 0) {
-    constexpr int kPer = int(kNodes) / 32;
+    constexpr int kPer = int(V::kCh + 31) / 32;
     uint32_t sz[kPer], sum = 0;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
@@ -977,7 +999,8 @@ __device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       if (inside(w0 + 256u * i + 8u * lane + e)) {
-        const uint32_t c = half_of(cd, e), at = wc[c >> 9] + (c & 511u);
+        const uint32_t c = half_of(cd, e);
+        const uint32_t at = wc[c >> V::kRankBits] + (c & ((1u << V::kRankBits) - 1u));
         const uint32_t xw = word_of(x[i], e >> 1), yw = word_of(y[i], e >> 1), zw = word_of(z[i], e >> 1);
         T.st[stage_slot(at)] = make_uint2(__byte_perm(xw, yw, (e & 1) ? 0x7632 : 0x5410), (e & 1) ? zw >> 16 : zw);
         if (IDX) T.sti[at] = word_of(ix[2 * i + (e >> 2)], e & 3);
@@ -995,7 +1018,7 @@ __device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX> &T
 template <bool IDX, int BITS>
 __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLaunch a) {
   extern __shared__ __align__(128) unsigned char sm[];
-  using V = MoveSmem<IDX>;
+  using V = MoveSmem<IDX, BITS>;
   V &T = *reinterpret_cast<V *>(sm);
   constexpr uint32_t kTile = V::kTile;
   if (call_failed(a.err)) return;
@@ -1100,7 +1123,7 @@ __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLa
 
 template <bool IDX, int BITS>
 cudaError_t move_launch(const SplitLaunch &a, cudaStream_t st) {
-  constexpr size_t smem = sizeof(MoveSmem<IDX>);
+  constexpr size_t smem = sizeof(MoveSmem<IDX, BITS>);
   int per_sm = 0;
   cudaError_t e = resident_blocks<k_move<IDX, BITS>>(kMT, smem, &per_sm);
   if (e != cudaSuccess) return e;
@@ -1113,7 +1136,8 @@ template <bool IDX>
 cudaError_t move_dispatch(const SplitLaunch &a, cudaStream_t st) {
   if (a.levels <= 4) return move_launch<IDX, 4>(a, st);
   if (a.levels == 5) return move_launch<IDX, 5>(a, st);
-  return a.levels == 6 ? move_launch<IDX, 6>(a, st) : move_launch<IDX, 7>(a, st);
+  if (a.levels == 6) return move_launch<IDX, 6>(a, st);
+  return a.levels == 7 ? move_launch<IDX, 7>(a, st) : move_launch<IDX, 8>(a, st);
 }
 
 }  // namespace

@@ -291,10 +291,16 @@ uint32_t digit_bits_for(int level) {
 
 // Several levels per launch (k_split.cu).  A launch below depth 0 needs subroots
 // of at least kSplitMinRoot particles, so that their histograms stay small
-// beside the data, and its levels are limited by the codes' bits: at level l of
-// a launch the 2^l nodes share kSplitBins bins and the codes of their median
-// bins kSplitLow counters, which holds for every data while
-// bits <= 26 - 2 l, i.e. 7 levels up to 14 bits, else 6.
+// beside the data, and its levels are limited by the codes' bits: level l's 2^l
+// nodes share kSplitBins = 2^14 bins, so a bin spans at most 2^(bits + l - 14)
+// codes, and the codes of the nodes' median bins need 2^l times as many of the
+// kSplitLow counters.  That holds for every data with 8 levels up to 13 bits, 7
+// up to 15, else 6.
+int split_max_levels(int bits) { return bits <= 13 ? 8 : (bits <= 15 ? 7 : 6); }
+uint32_t split_low_cap(int bits, int levels) {
+  const int shift = bits + levels - 1 - 14;
+  return (1u << (levels - 1)) << (shift > 0 ? shift : 0);
+}
 constexpr uint64_t kSplitMinRoot = 1u << 17;
 constexpr uint64_t kSplitMinChunk = 4096;  // particles of a CTA: fewer CTAs for small inputs
 constexpr int kSplitLaunches = 16;         // barrier words
@@ -876,7 +882,11 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
          ++launches) {
       // even shares of what is left, or as many as one launch takes where a second one's
       // subroots would be too small
-      const int max_levels = bit_length(qmax) <= 14 ? 7 : 6, left = split_to - src_depth;
+      // eight levels save a launch where a call is alone (3,000,017 particles: 343 us against
+      // 391 with four and four), but the move works less well with 256 children: a batch
+      // of 48 snapshots takes 5.17 ms with at most seven, 5.24 with eight
+      const int most_levels = split_max_levels(int(bit_length(qmax))), left = split_to - src_depth;
+      const int max_levels = share > 1 ? std::min(most_levels, 7) : most_levels;
       const int parts = (left + max_levels - 1) / max_levels;
       SplitLaunch sl = {};
       sl.n = n;
@@ -898,7 +908,8 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
         return reinterpret_cast<uint32_t *>(q);
       };
       sl.node = reinterpret_cast<uint8_t *>(take(n + 64));
-      sl.seglow = take(segs * kSplitLow * 4);
+      sl.low_cap = split_low_cap(int(bit_length(qmax)), sl.levels);
+      sl.seglow = take(segs * sl.low_cap * 4);
       sl.segcnt = take((kSplitParts * uint64_t(sl.grid) + roots) * 4 << kSplitMaxLevels);
       sl.ties = take(4 * n);
       if (sl.depth > 0) {

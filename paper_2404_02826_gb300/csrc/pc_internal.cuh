@@ -190,9 +190,9 @@ cudaError_t launch_level(const LevelLaunch &a, cudaStream_t st);
 cudaError_t launch_scatter(const LevelLaunch &a, cudaStream_t st);
 // Several levels in one cooperative launch (k_split.cu): 16-bit codes, split
 // axis depth mod 3, every node above depth + levels larger than a leaf.
-constexpr int kSplitMaxLevels = 7;         // a particle's node below its subroot fits a byte
+constexpr int kSplitMaxLevels = 8;         // a particle's node below its subroot fits a byte
 constexpr uint32_t kSplitBins = 16384;     // counters of one level's histogram, shared by its nodes
-constexpr uint32_t kSplitLow = 4096;       // counters of the codes in the nodes' median bins
+constexpr uint32_t kSplitLow = 8192;       // counters of the codes in the nodes' median bins, at most
 constexpr uint32_t kSplitStateWords = 17u << (kSplitMaxLevels - 1);
 constexpr int kSplitParts = 2;             // parts of a CTA's positions, one per CTA of the move
 constexpr uint32_t kSplitMaxRoots = 512;   // subroots of one launch
@@ -213,7 +213,8 @@ struct SplitLaunch {
   uint32_t *low;              // [2][2^depth][kSplitLow], zero on entry
   uint32_t part;              // positions per CTA of the move (set by launch_split)
   // scratch; a segment is what a CTA holds of a subroot (at most grid + 2^depth of them)
-  uint32_t *seglow;           // [kSplitLow][grid + 2^depth] codes in the median bins, by segment
+  uint32_t *seglow;           // [low_cap][grid + 2^depth] codes in the median bins, by segment
+  uint32_t low_cap;           // at least 2^l << shift of every level l, whatever the codes
   uint32_t *segcnt;           // [2^kSplitMaxLevels][kSplitParts grid + 2^depth] children, by part of a segment
   uint32_t *ties;             // [n] positions of ties
   uint32_t *state;            // [grid + 2^depth][kSplitStateWords] (depth > 0)

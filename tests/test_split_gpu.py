@@ -1,6 +1,6 @@
 """Several k-d levels per launch (csrc/k_split.cu) where it can go wrong: inputs a
-particle past a CTA's positions or a tile of the move, one to seven levels in a
-launch, 16-bit codes (six levels, median bins of several codes), two launches
+particle past a CTA's positions or a tile of the move, one to eight levels in a
+launch, 15 and 16-bit codes (seven and six levels, median bins of several codes), two launches
 with subroots cut by the CTAs' positions, and ties - few, thousands and more
 than the shared-memory list holds - on the split planes.  Streams and
 permutations equal the oracle's byte for byte.
@@ -29,6 +29,8 @@ CASES = [
     ("five levels", lambda: synth.cosmology(152 * 4096 + 1, seed=3), 1e-4, 4096),
     ("seven levels", lambda: synth.cosmology(524_289, seed=4), 1e-3, 700),
     ("seven levels, a chunk of 16", lambda: synth.uniform(1_048_559, seed=5), 1e-2, 4096),
+    ("eight levels", lambda: synth.cosmology(1_100_003, seed=14), 1e-4, 2048),
+    ("eight levels, one child each tile", lambda: synth.fluid(1_300_000, seed=15, dtype=np.float32), 1e-4, 4096),
     ("fifteen bits", lambda: synth.uniform(300_007, seed=6), 2e-5, 512),
     ("sixteen bits", lambda: synth.cosmology(400_001, seed=7), 8e-6, 512),
     ("two launches", lambda: synth.cosmology(2_200_003, seed=8), 1e-4, 4096),
