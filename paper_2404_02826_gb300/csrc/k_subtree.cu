@@ -4,11 +4,16 @@
 // Once every node of a level fits in shared memory, a CTA takes one node (in
 // ticket order), copies its code arrays in with bulk copies and finishes its
 // subtree on chip, without returning to HBM:
-//   - every remaining level: per subnode a radix select of the median code on
-//     its split axis (histograms in shared memory), then a stable two-way
-//     partition of every subnode (the median rule of Sec. 4.1: code < v, then
-//     the first `tleft` codes equal to v in index order, go left), from warp
-//     ballots and one block-wide scan, moved in place through registers;
+//   - every remaining level (the median rule of Sec. 4.1: code < v, then the
+//     first `tleft` codes equal to v in index order, go left).  With 16-bit
+//     codes and the depth-mod-3 axis nothing moves until the last level is
+//     split: a thread keeps its particles' subnodes beside their codes, a histogram
+//     of the split axis over all subnodes gives every median, and one stable
+//     partition then takes the particles to their leaves (Multi).
+//     Otherwise (32-bit codes, widest-cell axis, the leaf-size search's pass,
+//     which needs the arrangement of every level): per level and subnode a
+//     radix select, then a stable two-way partition in place through tensor
+//     memory;
 //   - the leaves' bit boxes (AABB, the particle closest to its centre, Eq. 2);
 //   - the CTA's first payload word, from the payload sizes of the CTAs before
 //     it (decoupled look-back over one status word per node, bounded waits);
@@ -31,6 +36,7 @@ constexpr int kLgWarps = 5;
 constexpr int kWarps = 1 << kLgWarps;
 constexpr int kSubMaxLevels = kLgWarps + 1;  // splits inside a CTA: at least one warp per splitting subnode
 constexpr uint32_t kSubBins = 2048;  // radix bins of a level, shared by its subnodes
+constexpr uint32_t kMultiBins = 3072;  // the same where levels are split without moving
 constexpr uint32_t kLookSpin = 1u << 20;  // polls of a predecessor's status before giving up
 constexpr uint32_t kTmemCols = 512;       // tensor-memory columns of a CTA (one CTA per SM)
 
@@ -53,6 +59,7 @@ struct SubLeaf {
 };
 
 struct SubMisc {
+  uint32_t shift, narrow;       // bins of a level; whether codes outside the subnodes' ranges are skipped
   unsigned long long bar;
   unsigned long long prefix;    // payload words of the nodes before this one
   unsigned long long wd[kWarps][2];
@@ -83,6 +90,21 @@ __device__ __forceinline__ LeafSlots leaf_slots(uint32_t nl, int warp, int lane)
   return q;
 }
 
+constexpr uint32_t kTiesLeft = 0xffffffffu, kTiesRight = 0xfffffffeu;
+
+// Tables of the levels split without moving (an entry per subnode).
+struct MultiTab {
+  union {
+    uint32_t tc[kWarps][kWarps];            // by warp: ties of its particles, then where they go: all
+                                            // left, all right, or the subnode's ties before them
+    uint16_t wcnt[kWarps][2 * kWarps + 2];  // the move: a warp's particles of a child, then its first place
+  };
+  uint32_t plane[kWarps];  // right if 2 code + 1 >= plane
+  int32_t off[kWarps];     // bin of code x: off + (x >> shift)
+  uint32_t range[kWarps];  // codes that can hold the median: lowest | how many << 16 (none: a leaf)
+  uint32_t tleft[kWarps];  // ties that go left
+};
+
 __host__ __device__ constexpr uint32_t al128(uint32_t x) { return (x + 127u) & ~127u; }
 
 // Shared-memory layout of one CTA: the code arrays of a node of up to
@@ -90,20 +112,24 @@ __host__ __device__ constexpr uint32_t al128(uint32_t x) { return (x + 127u) & ~
 // aligned window), the optional index array, the radix bins, the partition's
 // masks and scan (reused as the packing's word staging), the subnode and leaf
 // records.  All offsets are compile-time constants.
-template <typename C, bool IDX>
+// MULTI: the levels are split without moving, and with input indices the
+// particles' places in the node are kept (16 bits) instead of the indices, so
+// that a CTA holds half as many more.
+template <typename C, bool IDX, bool MULTI>
 struct SubL {
-  static constexpr int R = sizeof(C) == 2 ? (IDX ? 16 : 32) : (IDX ? 12 : 16);  // positions per thread
+  static constexpr int R =
+      sizeof(C) == 2 ? (IDX ? (MULTI ? 24 : 16) : 32) : (IDX ? 12 : 16);  // positions per thread
   // tensor-memory columns of one thread: every array's values of its positions, 32 bits per column
   static constexpr int kCodeCols = sizeof(C) == 2 ? R / 2 : R;
-  static constexpr int kCols = 3 * kCodeCols + (IDX ? R : 0);
+  static constexpr int kCols = 3 * kCodeCols + (MULTI ? R / 2 : (IDX ? R : 0));
   static_assert(kCodeCols % 4 == 0 && (kWarps / 4) * kCols <= 512, "tensor-memory columns");
   static constexpr uint32_t kCap = uint32_t(R) * kT;
   static constexpr uint32_t kSlots = kCap + 16;
   static constexpr uint32_t kCodeStride = al128(kSlots * uint32_t(sizeof(C)));
   static constexpr uint32_t kIdx = 3 * kCodeStride;
-  static constexpr uint32_t kBins = kIdx + (IDX ? al128(kSlots * 4) : 0u);
-  static constexpr uint32_t kStage = kBins + al128(kSubBins * 4);
-  static constexpr uint32_t kPart = uint32_t(R) * kWarps * 16, kPack = kWarps * 96u * 4;
+  static constexpr uint32_t kBins = kIdx + (IDX ? al128(kSlots * (MULTI ? 2 : 4)) : 0u);
+  static constexpr uint32_t kStage = kBins + al128((MULTI ? kMultiBins : kSubBins) * 4);
+  static constexpr uint32_t kPart = MULTI ? sizeof(MultiTab) : uint32_t(R) * kWarps * 16, kPack = kWarps * 96u * 4;
   static constexpr uint32_t kSn0 = kStage + al128(kPart > kPack ? kPart : kPack);
   static constexpr uint32_t kSn1 = kSn0 + al128(kWarps * sizeof(SubNode));
   static constexpr uint32_t kLeaf = kSn1 + al128(kWarps * sizeof(SubNode));
@@ -128,6 +154,17 @@ __device__ __forceinline__ uint32_t widest_axis(const uint32_t *blo, const uint3
   for (uint32_t d = 1; d < 3; ++d)
     if (bhi[d] - blo[d] > bhi[ax] - blo[ax]) ax = d;
   return ax;
+}
+
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
 }
 
 // Radix-select state of a splitting subnode from its cell (k_prep's rule):
@@ -205,6 +242,31 @@ __device__ __forceinline__ void tmem_ld4x3(uint32_t t0, uint32_t t1, uint32_t t2
       : "r"(t0), "r"(t1), "r"(t2)
       : "memory");
 }
+// 4 columns from one place and 2 from another, one wait
+__device__ __forceinline__ void tmem_ld4_2(uint32_t t0, uint32_t t1, uint32_t *v, uint32_t *n) {
+  __syncwarp();
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%6];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4, %5}, [%7];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(n[0]), "=r"(n[1])
+      : "r"(t0), "r"(t1)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld2(uint32_t t, uint32_t *v) {
+  __syncwarp();
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(v[0]), "=r"(v[1])
+      : "r"(t)
+      : "memory");
+}
+// 2 consecutive columns; complete by tmem_wait_st()
+__device__ __forceinline__ void tmem_st2(uint32_t t, uint32_t a, uint32_t b) {
+  __syncwarp();
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(t), "r"(a), "r"(b) : "memory");
+}
 __device__ __forceinline__ void tmem_ld4(uint32_t t, uint32_t *v) {
   __syncwarp();
   asm volatile(
@@ -257,13 +319,417 @@ __device__ __forceinline__ void load_rows(const E *A, uint32_t nv, uint32_t Tg, 
   }
 }
 
+// All levels of a CTA's node, then one move (16-bit codes, depth-mod-3 axis).
+// Warp w owns the positions [w Rn 32, (w + 1) Rn 32) in rows of 32.  A thread's
+// rows stay in its tensor-memory columns, 8 rows a chunk: the codes of array d
+// from tcol + d NC, from kRk on first a byte per row with 4 x its subnode (the
+// byte offset into the tables), at the end child << 10 | rank.  On entry cur[0]
+// is the node; on exit X0 (and, with IDX, the places P) are in leaf order and
+// cur holds the subnodes of the last level.  bins: zero on entry and on exit.
+// Chunks whose rows all hold particles take unguarded code: with a guard per
+// row the guards cost more than the work.
+// A CTA of 32768 particles and three levels takes 119 K cycles (2^27 particles:
+// 1.58 ms a launch, 1.94 with a move per level and a particle per lane in the
+// packing, 148 K): copy 5, rows into tensor memory 4, per level histogram 6
+// (bound by the shared-memory atomics), search 1.5, split 7, ties 3, then ranks 9,
+// move 10, boxes 11, look-back 10 (waiting for the slowest node before), packing 15.
+template <bool IDX, typename L>
+struct Multi {
+  static constexpr int R = L::R, NC = L::kCodeCols;
+  static constexpr uint32_t kRk = 3u * NC, kNid = kRk + R / 4;  // rank columns: R / 2; nodes: their second half
+  static constexpr uint32_t S = L::kCodeStride / 2;
+  const SubtreeLaunch &a;
+  uint16_t *const X0, *const P;
+  uint32_t *const bins;
+  MultiTab &T;
+  SubMisc &M;
+  const uint32_t tcol;
+  const int lane, warp;
+  uint32_t cnt, Rn, w0, nv, nvw, chunks;  // nv: this thread's rows, nvw: the least of the warp
+
+  template <typename V>
+  static __device__ __forceinline__ V at4(const V *t, uint32_t byte) {
+    return *reinterpret_cast<const V *>(reinterpret_cast<const char *>(t) + byte);
+  }
+  static __device__ __forceinline__ uint32_t byte_at(const uint32_t *n, int i) {
+    return __byte_perm(n[i >> 2], 0u, 0x4440u | uint32_t(i & 3));
+  }
+
+  // NARROW: only codes that can hold their subnode's median
+  template <bool FULL, bool NARROW>
+  __device__ __forceinline__ void hist_chunk(uint32_t ch, uint32_t ax, uint32_t shift) {
+    uint32_t v[4], n[2];
+    tmem_ld4_2(tcol + ax * NC + 4u * ch, tcol + kNid + 2u * ch, v, n);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t c = row_of<uint16_t>(v, i), j4 = byte_at(n, i);
+      const uint32_t b = min(uint32_t(int32_t(c >> shift) + at4(T.off, j4)), kMultiBins - 1u);
+      bool in = FULL || 8u * ch + i < nv;
+      if (NARROW) {
+        const uint32_t rg = at4(T.range, j4);
+        in = in && c - (rg & 0xffffu) < (rg >> 16);
+      }
+      if (in) atomicAdd(&bins[b], 1u);
+    }
+  }
+  // to the children, ties right; the ties are counted by warp and subnode, their rows kept
+  template <bool FULL>
+  __device__ __forceinline__ uint32_t split_chunk(uint32_t ch, uint32_t ax) {
+    uint32_t v[4], n[2], o[2] = {0, 0}, hit = 0;
+    tmem_ld4_2(tcol + ax * NC + 4u * ch, tcol + kNid + 2u * ch, v, n);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t t = 2u * row_of<uint16_t>(v, i) + 1u, j4 = byte_at(n, i);
+      const uint32_t p = at4(T.plane, j4);
+      o[i >> 2] |= (2u * j4 + (t >= p ? 4u : 0u)) << (8 * (i & 3));
+      if (t == p && (FULL || 8u * ch + i < nv)) hit |= 1u << i;
+    }
+    tmem_st2(tcol + kNid + 2u * ch, o[0], o[1]);
+    if (__any_sync(0xffffffffu, hit != 0)) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if ((hit >> i) & 1u) atomicAdd(&T.tc[warp][byte_at(n, i) >> 2], 1u);
+    }
+    return hit;
+  }
+  // the ties of a chunk whose subnode's ties in this warp all go left
+  __device__ __forceinline__ void left_chunk(uint32_t ch, uint32_t hit) {
+    uint32_t n[2];
+    tmem_ld2(tcol + kNid + 2u * ch, n);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t how = T.tc[warp][(byte_at(n, i) >> 3) & 31u];  // 4 x child = 8 x node + 4
+      if (((hit >> i) & 1u) && how == kTiesLeft) n[i >> 2] -= 4u << (8 * (i & 3));
+    }
+    tmem_st2(tcol + kNid + 2u * ch, n[0], n[1]);
+  }
+  // the first `quota` ties of subnode j in position order
+  __device__ __forceinline__ void cut_node(uint32_t j, uint32_t quota, uint32_t hits) {
+    const uint32_t ltm = (1u << lane) - 1u;
+    uint32_t seen = 0;
+    for (uint32_t ch = 0; ch < chunks && seen < quota; ++ch) {
+      const uint32_t hit = (hits >> (8u * ch)) & 0xffu;
+      if (!__any_sync(0xffffffffu, hit != 0)) continue;
+      uint32_t n[2];
+      tmem_ld2(tcol + kNid + 2u * ch, n);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const bool mine = ((hit >> i) & 1u) && ((byte_at(n, i) >> 3) & 31u) == j;
+        const uint32_t m = __ballot_sync(0xffffffffu, mine);
+        if (mine && seen + __popc(m & ltm) < quota) n[i >> 2] -= 4u << (8 * (i & 3));
+        seen += __popc(m);
+      }
+      tmem_st2(tcol + kNid + 2u * ch, n[0], n[1]);
+    }
+  }
+  // ranks among the warp's particles of the same child
+  template <bool FULL, int BITS>
+  __device__ __forceinline__ void rank_chunk(uint32_t ch) {
+    const uint32_t ltm = (1u << lane) - 1u;
+    uint16_t *const wc = T.wcnt[warp];
+    uint32_t n[2], rk[4];
+    tmem_ld2(tcol + kNid + 2u * ch, n);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t b = byte_at(n, i) >> 2;
+      uint32_t peers = FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, 8u * ch + i < nv);
+#pragma unroll
+      for (int q = 0; q < BITS; ++q) {
+        uint32_t m;  // the lanes whose bit q is this lane's
+        asm(
+            "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t"
+            "vote.sync.ballot.b32 %0, p, 0xffffffff;\n\t@!p not.b32 %0, %0;\n\t}"
+            : "=r"(m)
+            : "r"(b), "r"(1u << q));
+        peers &= m;
+      }
+      const uint32_t old = wc[b];
+      __syncwarp();
+      if (FULL || 8u * ch + i < nv) wc[b] = uint16_t(old + __popc(peers));  // the same from every lane of the child
+      __syncwarp();
+      const uint32_t cd = (b << 10) | (old + __popc(peers & ltm));
+      if (i & 1) rk[i >> 1] |= cd << 16;
+      else rk[i >> 1] = cd;
+    }
+    tmem_st4(tcol + kRk + 4u * ch, rk[0], rk[1], rk[2], rk[3]);
+  }
+  template <bool FULL>
+  __device__ __forceinline__ void move_chunk(uint32_t ch) {
+    const uint16_t *const wc = T.wcnt[warp];
+    uint32_t v[12], rk[4];
+    tmem_ld4x3(tcol + 4u * ch, tcol + NC + 4u * ch, tcol + 2 * NC + 4u * ch, v);
+    tmem_ld4(tcol + kRk + 4u * ch, rk);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t cd = row_of<uint16_t>(rk, i);
+      const uint32_t dst = min(uint32_t(wc[cd >> 10]) + (cd & 1023u), uint32_t(L::kCap) - 1u);
+      if (FULL || 8u * ch + i < nv) {
+        X0[dst] = uint16_t(row_of<uint16_t>(v, i));
+        X0[S + dst] = uint16_t(row_of<uint16_t>(v + 4, i));
+        X0[2 * S + dst] = uint16_t(row_of<uint16_t>(v + 8, i));
+        if (IDX) P[dst] = uint16_t(w0 + 32u * (8u * ch + i));
+      }
+    }
+  }
+
+  __device__ __forceinline__ void run(SubNode *&cur, SubNode *&nxt) {
+    cnt = cur[0].cnt;
+    Rn = (cnt + kT - 1u) / kT;
+    chunks = (Rn + 7u) / 8u;
+    w0 = uint32_t(warp) * Rn * 32u + uint32_t(lane);
+    nv = w0 < cnt ? min((cnt - w0 + 31u) / 32u, Rn) : 0u;
+    nvw = __reduce_min_sync(0xffffffffu, nv);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) load_rows<R>(X0 + d * S + uint32_t(warp) * Rn * 32u, nv, 32u, uint32_t(lane), tcol + d * NC);
+    for (uint32_t ch = 0; ch < chunks; ++ch) tmem_st2(tcol + kNid + 2u * ch, 0u, 0u);
+    tmem_wait_st();
+
+    for (int k = 0; k < a.levels; ++k) {
+      const uint32_t G = 1u << k, ax = uint32_t(a.depth + k) % 3u;
+      if (threadIdx.x < G) {
+        SubNode &u = cur[threadIdx.x];
+        u.lo = u.blo[ax];
+        u.prefix = u.bhi[ax];  // the codes that can hold the median: lo .. prefix
+        u.below = 0;
+      }
+      __syncthreads();
+      // the medians: bins of 2^shift codes over all subnodes' ranges, narrowed until shift is 0
+      for (bool first = true;; first = false) {
+        if (warp == 0) {
+          const bool in = uint32_t(lane) < G && cur[lane].split;
+          const uint32_t lo = in ? cur[lane].lo : 1u, hi = in ? cur[lane].prefix : 0u;
+          uint32_t sh = 0, nb, tot;
+          for (;; ++sh) {
+            nb = in ? (hi >> sh) - (lo >> sh) + 1u : 0u;
+            tot = __reduce_add_sync(0xffffffffu, nb);
+            if (tot <= kMultiBins || sh >= 16) break;
+          }
+          uint32_t incl = nb;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          T.off[lane] = int32_t(incl - nb) - int32_t(lo >> sh);
+          T.range[lane] = in ? (lo & 0xffffu) | (min(hi - lo + 1u, 0xffffu) << 16) : 0u;
+          const bool all = __all_sync(0xffffffffu, in || uint32_t(lane) >= G);
+          if (lane == 0) {
+            M.shift = sh;
+            M.narrow = !(first && all);
+          }
+        }
+        __syncthreads();
+        const uint32_t shift = M.shift;
+        const bool narrow = M.narrow != 0;
+        for (uint32_t ch = 0; ch < chunks; ++ch) {
+          const bool full = 8u * ch + 8u <= nvw;
+          if (!narrow) {
+            if (full) hist_chunk<true, false>(ch, ax, shift);
+            else hist_chunk<false, false>(ch, ax, shift);
+          } else {
+            if (full) hist_chunk<true, true>(ch, ax, shift);
+            else hist_chunk<false, true>(ch, ax, shift);
+          }
+        }
+        __syncthreads();
+        {  // exclusive prefixes in place, three bins per thread
+          static_assert(kMultiBins == 3 * kT, "bins per thread");
+          const uint32_t b = 3u * threadIdx.x, h0 = bins[b], h1 = bins[b + 1], h2 = bins[b + 2];
+          uint32_t incl = h0 + h1 + h2;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          if (lane == 31) M.wt[warp] = incl;
+          __syncthreads();
+          const uint32_t t = M.wt[lane];
+          const uint32_t ex = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u) + incl - h0 - h1 - h2;
+          bins[b] = ex;
+          bins[b + 1] = ex + h0;
+          bins[b + 2] = ex + h0 + h1;
+        }
+        __syncthreads();
+        if (uint32_t(warp) < G && cur[warp].split) {  // a warp per subnode: its last bin whose prefix is not above the rank
+          SubNode &u = cur[warp];
+          const int32_t off = T.off[warp];
+          uint32_t lo = uint32_t(int32_t(u.lo >> shift) + off);
+          uint32_t hi = min(uint32_t(int32_t(u.prefix >> shift) + off), kMultiBins - 1u);
+          const uint32_t s0 = bins[min(lo, kMultiBins - 1u)], target = (u.cnt >> 1) - u.below + s0;
+          while (lo < hi) {
+            const uint32_t by = (hi - lo) / 32u + 1u, at = lo + by * lane;
+            const uint32_t m = __ballot_sync(0xffffffffu, at <= hi && bins[min(at, kMultiBins - 1u)] <= target);
+            lo += by * (m ? 31u - uint32_t(__clz(m)) : 0u);
+            hi = min(hi, lo + by - 1u);
+          }
+          __syncwarp();
+          if (lane == 0) {
+            const uint32_t q = uint32_t(int32_t(lo) - off);  // the bin's codes: q << shift ..
+            u.below += bins[min(lo, kMultiBins - 1u)] - s0;
+            u.lo = max(u.lo, q << shift);
+            u.prefix = min(u.prefix, ((q + 1u) << shift) - 1u);
+          }
+        }
+        __syncthreads();
+        for (uint32_t b = threadIdx.x; b < kMultiBins; b += kT) bins[b] = 0;
+        if (shift == 0) break;
+      }
+      // the planes (an odd one: 2 v + 1, its ties are listed) and the children
+      T.tc[warp][lane] = 0;
+      if (threadIdx.x < G) {
+        SubNode &u = cur[threadIdx.x];
+        const uint32_t v = u.lo, kk = u.cnt >> 1;
+        u.v = v;
+        u.tleft = kk - u.below;
+        T.plane[threadIdx.x] = u.split ? 2u * v + 1u : 0x7ffffffeu;
+        if (k + 1 < a.levels) {
+          if (!u.split) atomicOr(a.err, kErrInternal);
+          for (uint32_t h = 0; h < 2; ++h) {
+            SubNode &w = nxt[2 * threadIdx.x + h];
+            for (int d = 0; d < 3; ++d) {
+              w.blo[d] = u.blo[d];
+              w.bhi[d] = u.bhi[d];
+            }
+            if (h) w.blo[ax] = v;
+            else w.bhi[ax] = v;
+            w.off = u.off + (h ? kk : 0u);
+            w.cnt = h ? u.cnt - kk : kk;
+            w.axis = uint32_t(a.depth + k + 1) % 3u;
+            w.split = w.cnt > a.leaf_size;
+          }
+        }
+      }
+      __syncthreads();
+      uint32_t hits = 0;  // a bit per row
+      for (uint32_t ch = 0; ch < chunks; ++ch) {
+        const uint32_t h = 8u * ch + 8u <= nvw ? split_chunk<true>(ch, ax) : split_chunk<false>(ch, ax);
+        hits |= h << (8u * ch);
+      }
+      tmem_wait_st();
+      __syncthreads();
+      // where each warp's ties start among its subnode's: the first `tleft` of all go left
+      if (uint32_t(warp) < G) {
+        const uint32_t mine = T.tc[lane][warp];
+        uint32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const uint32_t tleft = cur[warp].split ? cur[warp].tleft : 0u;
+        T.tc[lane][warp] = incl <= tleft ? kTiesLeft : (incl - mine >= tleft ? kTiesRight : incl - mine);
+        if (lane == 0) T.tleft[warp] = tleft;
+      }
+      __syncthreads();
+      {
+        const uint32_t how = uint32_t(lane) < G ? T.tc[warp][lane] : kTiesRight;
+        if (__any_sync(0xffffffffu, how == kTiesLeft)) {
+          for (uint32_t ch = 0; ch < chunks; ++ch) {
+            const uint32_t h = (hits >> (8u * ch)) & 0xffu;
+            if (__any_sync(0xffffffffu, h != 0)) left_chunk(ch, h);
+          }
+          tmem_wait_st();
+        }
+        for (uint32_t cut = __ballot_sync(0xffffffffu, how < kTiesRight); cut; cut &= cut - 1u) {
+          const uint32_t j = uint32_t(__ffs(cut)) - 1u;
+          cut_node(j, T.tleft[j] - __shfl_sync(0xffffffffu, how, j), hits);
+          tmem_wait_st();
+        }
+        tmem_wait_st();
+      }
+      if (k + 1 < a.levels) {
+        SubNode *t = cur;
+        cur = nxt;
+        nxt = t;
+      }
+      __syncthreads();
+    }
+
+    // ---- the move ----
+    const uint32_t NB = 1u << a.levels;
+    uint16_t *const wc = T.wcnt[warp];
+    for (uint32_t b = lane; b < 2u * kWarps; b += 32) wc[b] = 0;
+    __syncwarp();
+    for (uint32_t ch = 0; ch < chunks; ++ch) {
+      const bool full = 8u * ch + 8u <= nvw;
+      if (a.levels <= 3) {
+        if (full) rank_chunk<true, 3>(ch);
+        else rank_chunk<false, 3>(ch);
+      } else {
+        if (full) rank_chunk<true, 6>(ch);
+        else rank_chunk<false, 6>(ch);
+      }
+    }
+    tmem_wait_st();
+    __syncthreads();
+    // first place of every warp's particles of a child: the child's place from the median rule
+    for (uint32_t b = warp; b < NB; b += kWarps) {
+      const SubNode &u = cur[b >> 1];
+      const uint32_t base = u.off + ((b & 1u) ? (u.split ? u.cnt >> 1 : u.cnt) : 0u);
+      const uint32_t v = T.wcnt[lane][b];
+      uint32_t incl = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      T.wcnt[lane][b] = uint16_t(base + incl - v);
+    }
+    __syncthreads();
+    for (uint32_t ch = 0; ch < chunks; ++ch) {
+      if (8u * ch + 8u <= nvw) move_chunk<true>(ch);
+      else move_chunk<false>(ch);
+    }
+    __syncthreads();
+  }
+};
+
+// 128 particles of a leaf (block `blk` of its non-centre particles) packed by a
+// warp, 8 <= w <= 32: a lane forms 4 consecutive particles' 4 w bits, shifted to
+// their place in the words, and takes the word it shares with the next lane's
+// first bits.  128 particles fill 4 w whole words.  24 instructions per 32
+// particles, against 80 with a particle per lane whose words are put together
+// by shuffles.
+template <typename C>
+__device__ __forceinline__ void pack_block(const C *x0, const C *x1, const C *x2, uint32_t b0, uint32_t b1, uint32_t b2,
+                                           uint32_t m0, uint32_t m1, uint32_t w, uint32_t blk, uint32_t centre,
+                                           uint32_t nsl, uint32_t words, uint32_t *payload, int lane) {
+  uint32_t v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t sl = blk * 128u + 4u * lane + i;
+    const uint32_t p = min(sl, nsl - 1u) + (sl >= centre ? 1u : 0u);
+    const uint32_t q = min(p, nsl);  // nsl + 1 particles with the centre
+    const uint32_t y = uint32_t(x0[q]) - b0 | ((uint32_t(x1[q]) - b1) << (m0 & 31u)) |
+                       ((uint32_t(x2[q]) - b2) << ((m0 + m1) & 31u));
+    v[i] = sl < nsl ? y : 0u;
+  }
+  const unsigned long long lo = v[0] | ((unsigned long long)v[1] << w), hi = v[2] | ((unsigned long long)v[3] << w);
+  const unsigned long long a0 = w < 32u ? lo | (hi << (2u * w)) : lo, a1 = w < 32u ? hi >> (64u - 2u * w) : hi;
+  const uint32_t bit = 4u * w * uint32_t(lane), k0 = bit >> 5, sh = bit & 31u, end = sh + 4u * w;
+  const uint32_t t0 = uint32_t(a0), t1 = uint32_t(a0 >> 32), t2 = uint32_t(a1), t3 = uint32_t(a1 >> 32);
+  uint32_t W[5] = {t0 << sh, __funnelshift_l(t0, t1, sh), __funnelshift_l(t1, t2, sh), __funnelshift_l(t2, t3, sh),
+                   __funnelshift_l(t3, 0u, sh)};
+  const uint32_t nx = __shfl_down_sync(0xffffffffu, W[0], 1);
+  const uint32_t last = (end - 1u) >> 5, gw0 = blk * 4u * w + k0;
+#pragma unroll
+  for (uint32_t i = 0; i < 5; ++i) {
+    if ((i > 0 || sh == 0) && i <= last && gw0 + i < words) {
+      uint32_t word = W[i];
+      if (i == last && (end & 31u) != 0) word |= nx;
+      __stcs(payload + gw0 + i, word);
+    }
+  }
+}
+
 // COST: the leaf-size search's pass.  Every subnode splits at every level;
 // before the first level and after each one the leaves at that depth get their
 // bit boxes, and their payload words are added to cost_words[level]; nothing
 // is written to the stream.
 template <typename C, bool IDX, bool WIDEST, bool COST>
-__global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
-  using L = SubL<C, IDX>;
+__global__ void __launch_bounds__(kT, 1) k_subtree(const __grid_constant__ SubtreeLaunch a) {
+  constexpr bool MULTI = sizeof(C) == 2 && !WIDEST && !COST;
+  using L = SubL<C, IDX, MULTI>;
   constexpr int R = L::R;
   extern __shared__ __align__(128) unsigned char sm[];
   uint32_t *bins = reinterpret_cast<uint32_t *>(sm + L::kBins);
@@ -298,14 +764,14 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
     const bool dead = *reinterpret_cast<const volatile uint32_t *>(a.err) != 0u;
     M.skip = dead ? 1u : 0u;
     const bool ok = ncnt <= L::kCap && !dead;
-    const uint32_t bytes = ok ? 3 * nwin * uint32_t(sizeof(C)) + (IDX ? 4 * niw : 0u) : 0u;
+    const uint32_t bytes = ok ? 3 * nwin * uint32_t(sizeof(C)) + (IDX && !MULTI ? 4 * niw : 0u) : 0u;
     if (!ok && !dead) atomicOr(a.err, kErrInternal);
     mbar_expect_tx(&M.bar, bytes);
     if (bytes) {
       for (int d = 0; d < 3; ++d)
         bulk_g2s(sm + d * L::kCodeStride, static_cast<const C *>(a.codes[d]) + (noff - lead),
                  nwin * uint32_t(sizeof(C)), &M.bar);
-      if (IDX) bulk_g2s(sm + L::kIdx, a.idx + (noff - ilead), 4 * niw, &M.bar);
+      if (IDX && !MULTI) bulk_g2s(sm + L::kIdx, a.idx + (noff - ilead), 4 * niw, &M.bar);
     }
     // the root of the subtree: its cell from the parent's split (k_prep's rule);
     // in a failed call the parents' records were never written and are not read
@@ -332,7 +798,7 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
     s.split = s.cnt > a.leaf_size;
   }
   // the radix bins start at zero (every select pass leaves them zero again)
-  for (uint32_t b = threadIdx.x; b < kSubBins; b += kT) bins[b] = 0;
+  for (uint32_t b = threadIdx.x; b < (MULTI ? kMultiBins : kSubBins); b += kT) bins[b] = 0;
   if (warp == 0) tmem_alloc(&M.tmem, kTmemCols);
   tmem_fence_before();
   __syncthreads();
@@ -361,7 +827,7 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
   constexpr int RPC = sizeof(C) == 2 ? 2 : 1;      // rows per column
   constexpr uint32_t S = L::kCodeStride / sizeof(C);
   uint32_t *const XI = reinterpret_cast<uint32_t *>(sm + L::kIdx) + M.ilead;
-  if (a.levels > 0) {  // the root's rows into TMEM (level 0: one group of all warps)
+  if (!MULTI && a.levels > 0) {  // the root's rows into TMEM (level 0: one group of all warps)
     const uint32_t cnt0 = cur[0].cnt;
     const uint32_t nv0 = cnt0 > threadIdx.x ? (cnt0 - threadIdx.x + kT - 1u) / kT : 0u;
     load_rows<R>(X0, nv0, kT, threadIdx.x, tcol);
@@ -408,14 +874,43 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
     for (uint32_t f = uint32_t(warp) >> lgwl; f < nl; f += slots) {
       const uint32_t off = LF[f].off, cnt = LF[f].cnt;
       uint32_t mn0 = 0xffffffffu, mn1 = 0xffffffffu, mn2 = 0xffffffffu, mx0 = 0, mx1 = 0, mx2 = 0;
-      for (uint32_t i = lt; i < cnt; i += lstep) {
-        const uint32_t c0 = Y0[off + i], c1 = Y1[off + i], c2 = Y2[off + i];
-        mn0 = min(mn0, c0);
-        mx0 = max(mx0, c0);
-        mn1 = min(mn1, c1);
-        mx1 = max(mx1, c1);
-        mn2 = min(mn2, c2);
-        mx2 = max(mx2, c2);
+      if (sizeof(C) == 2) {  // eight codes a load, two a minimum; the ends one by one
+        const uint32_t e0 = uint32_t(X0 - reinterpret_cast<C *>(sm)) + off, e1 = e0 + cnt;  // slots of the leaf
+        const uint32_t g0 = min((e0 + 7u) & ~7u, e1), g1 = max(g0, e1 & ~7u);
+        uint32_t n2[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, x2[3] = {0, 0, 0};
+        for (uint32_t g = g0 + 8u * lt; g < g1; g += 8u * lstep) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(sm + d * L::kCodeStride + 2u * g);
+            n2[d] = min_u16x2(n2[d], min_u16x2(min_u16x2(q.x, q.y), min_u16x2(q.z, q.w)));
+            x2[d] = max_u16x2(x2[d], max_u16x2(max_u16x2(q.x, q.y), max_u16x2(q.z, q.w)));
+          }
+        }
+        const uint32_t e = lt < 8u ? (e0 + lt < g0 ? e0 + lt : e1) : (lt < 16u ? g1 + lt - 8u : e1);
+        if (e < e1) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const uint32_t c = *reinterpret_cast<const C *>(sm + d * L::kCodeStride + 2u * e) * 0x10001u;
+            n2[d] = min_u16x2(n2[d], c);
+            x2[d] = max_u16x2(x2[d], c);
+          }
+        }
+        mn0 = min(n2[0] & 0xffffu, n2[0] >> 16);
+        mn1 = min(n2[1] & 0xffffu, n2[1] >> 16);
+        mn2 = min(n2[2] & 0xffffu, n2[2] >> 16);
+        mx0 = max(x2[0] & 0xffffu, x2[0] >> 16);
+        mx1 = max(x2[1] & 0xffffu, x2[1] >> 16);
+        mx2 = max(x2[2] & 0xffffu, x2[2] >> 16);
+      } else {
+        for (uint32_t i = lt; i < cnt; i += lstep) {
+          const uint32_t c0 = Y0[off + i], c1 = Y1[off + i], c2 = Y2[off + i];
+          mn0 = min(mn0, c0);
+          mx0 = max(mx0, c0);
+          mn1 = min(mn1, c1);
+          mx1 = max(mx1, c1);
+          mn2 = min(mn2, c2);
+          mx2 = max(mx2, c2);
+        }
       }
       mn0 = __reduce_min_sync(0xffffffffu, mn0);
       mn1 = __reduce_min_sync(0xffffffffu, mn1);
@@ -529,7 +1024,14 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
     }
   };
   if (COST) add_cost(leaf_boxes(1, false), 0);  // the node itself as one leaf
-  for (int k = 0; k < a.levels; ++k) {
+  uint16_t *const PL = reinterpret_cast<uint16_t *>(sm + L::kIdx);  // MULTI: places of the input indices in the node
+  if constexpr (MULTI) {
+    if (a.levels > 0)
+      Multi<IDX, L>{a, X0, PL, bins, *reinterpret_cast<MultiTab *>(sm + L::kStage), M, tcol, lane, warp}.run(cur, nxt);
+    else if (IDX)
+      for (uint32_t i = threadIdx.x; i < cur[0].cnt; i += kT) PL[i] = uint16_t(i);
+  }
+  for (int k = 0; !MULTI && k < a.levels; ++k) {
     const int lgW = kLgWarps - k;  // log2 of the warps per group
     const uint32_t G = 1u << k;
     const int g = warp >> lgW;
@@ -892,7 +1394,8 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
       const uint32_t *XI = reinterpret_cast<const uint32_t *>(sm + L::kIdx) + M.ilead + foff;
       for (uint32_t i = lt; i < fcnt; i += lstep) {
         const uint32_t src = i == 0 ? centre : (i - 1 < centre ? i - 1 : i);
-        a.perm[goff + i] = XI[src];
+        if (MULTI) a.perm[goff + i] = __ldg(a.idx + off64 + PL[foff + src]);
+        else a.perm[goff + i] = XI[src];
       }
     }
     const uint32_t m0 = fm & 0xffu, m1 = (fm >> 8) & 0xffu, m2 = (fm >> 16) & 0xffu;
@@ -903,6 +1406,12 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
     const uint32_t h1 = m1 ? (1u << (m1 - 1)) - 1u : 0u;
     const uint32_t h2 = m2 ? (1u << (m2 - 1)) - 1u : 0u;
     const uint32_t nsl = fcnt - 1, chunks = (nsl + 31) / 32;
+    if (w >= 8 && w <= 32) {
+      const C *x0 = Y0 + foff, *x1 = Y1 + foff, *x2 = Y2 + foff;
+      for (uint32_t blk = lw; blk * 128u < nsl; blk += WL)
+        pack_block(x0, x1, x2, r0 - h0, r1 - h1, r2 - h2, m0, m1, w, blk, centre, nsl, words, payload, lane);
+      continue;
+    }
     // w <= 32: word k of a chunk takes bits from lanes i0 = 32k / w on (at most nit of them)
     const uint32_t i0 = w <= 32 ? (32u * lane) / w : 0u;
     const int sh0 = int(i0 * w) - int(32u * lane);
@@ -972,7 +1481,7 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(SubtreeLaunch a) {
 
 template <typename C, bool IDX, bool WIDEST, bool COST>
 cudaError_t subtree_launch_as(const SubtreeLaunch &a, cudaStream_t st) {
-  const uint32_t smem = SubL<C, IDX>::kTotal;
+  const uint32_t smem = SubL<C, IDX, sizeof(C) == 2 && !WIDEST && !COST>::kTotal;
   int per_sm = 0;
   cudaError_t e = resident_blocks<k_subtree<C, IDX, WIDEST, COST>>(kT, smem, &per_sm);
   if (e != cudaSuccess) return e;
@@ -988,9 +1497,11 @@ cudaError_t subtree_launch(const SubtreeLaunch &a, cudaStream_t st) {
 
 }  // namespace
 
-uint32_t subtree_capacity(int code_bytes, bool with_idx) {
-  return code_bytes == 2 ? (with_idx ? SubL<uint16_t, true>::kCap : SubL<uint16_t, false>::kCap)
-                         : (with_idx ? SubL<uint32_t, true>::kCap : SubL<uint32_t, false>::kCap);
+uint32_t subtree_capacity(int code_bytes, bool with_idx, bool multi) {
+  if (code_bytes == 2 && multi)
+    return with_idx ? SubL<uint16_t, true, true>::kCap : SubL<uint16_t, false, true>::kCap;
+  return code_bytes == 2 ? (with_idx ? SubL<uint16_t, true, false>::kCap : SubL<uint16_t, false, false>::kCap)
+                         : (with_idx ? SubL<uint32_t, true, false>::kCap : SubL<uint32_t, false, false>::kCap);
 }
 
 cudaError_t launch_subtree(const SubtreeLaunch &a, cudaStream_t st) {

@@ -238,9 +238,9 @@ uint64_t subtree_status_entries(int levels) {
   return 1ull << d;
 }
 
-int subtree_depth(uint64_t n, uint32_t r, int levels, int code_bytes, bool idx, int sms) {
+int subtree_depth(uint64_t n, uint32_t r, int levels, int code_bytes, bool idx, bool widest, int sms) {
   if (n == 0) return -1;
-  const uint64_t cap = subtree_capacity(code_bytes, idx);
+  const uint64_t cap = subtree_capacity(code_bytes, idx, !widest);
   const int hi = levels >= 1 ? levels - 1 : 0;
   int lo = levels - kSubMaxLevels > 0 ? levels - kSubMaxLevels : 0;
   while (lo <= hi && ((n + (1ull << lo) - 1) >> lo) > cap) ++lo;
@@ -265,7 +265,7 @@ int subtree_depth(uint64_t n, uint32_t r, int levels, int code_bytes, bool idx, 
 // search stays on the levels over HBM.
 int tune_subtree_depth(uint64_t n, int tune_first, int tune_last, int code_bytes, bool idx) {
   if (n == 0 || tune_last < 1) return -1;
-  const uint64_t cap = subtree_capacity(code_bytes, idx);
+  const uint64_t cap = subtree_capacity(code_bytes, idx, false);
   int d = 0;
   while (d < tune_last && ((n + (1ull << d) - 1) >> d) > cap) ++d;
   if (d >= tune_last || d > kSubMaxDepth || d + kSubMaxLevels < tune_first) return -1;
@@ -690,7 +690,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     const int levels = p.tune ? p.tune_last : p.levels;
     const int sub_depth = (p.tune || p.reduce || p.reorder || sweep || L.raw)
                               ? -1
-                              : subtree_depth(n, p.r, p.levels, cb, use_idx, device_sm_count());
+                              : subtree_depth(n, p.r, p.levels, cb, use_idx, p.widest, device_sm_count());
     // the leaf-size search over the plain stream: levels over HBM down to tune_depth, then
     // the candidates below it costed on chip (the depth-mod-3 rule: a resumed level takes the
     // root's cell, which the widest-cell rule could not)

@@ -287,7 +287,9 @@ struct SubtreeLaunch {
   LevelNode *wb_nodes;
 };
 cudaError_t launch_subtree(const SubtreeLaunch &a, cudaStream_t st);
-uint32_t subtree_capacity(int code_bytes, bool with_idx);  // largest node of one CTA
+// Largest node of one CTA; `plain`: the packing pass on the depth-mod-3 axis (else the widest-cell
+// axis or the leaf-size search's pass).
+uint32_t subtree_capacity(int code_bytes, bool with_idx, bool plain);
 
 struct HeaderLaunch {
   uint8_t *out;
