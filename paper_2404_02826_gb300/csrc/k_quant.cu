@@ -294,6 +294,25 @@ __device__ __forceinline__ uint32_t quant_fast64(double p, double o, double s, d
   return quant_exact_call64(p, o, s);
 }
 
+// Same result in 64-bit integers.  p in units u of 2^-61 of the power of two
+// above every |p| (truncated), less the origin in them, times fw: the quotient
+// with fs (24 .. 60) fraction bits in the product's high word.  Truncations put it
+// within 2^-23 of the exact quotient ((p - o) / s with s / u >= 2^26: two units
+// are 2^-25), the double quotient of the definition lies within 2^-21 of that
+// (codes below 2^30); unless it is within 2^-20 of a half-integer, both round alike.
+__device__ __forceinline__ uint32_t quant_fixed64(double p, int d, const QuantParams &qp) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(p);
+  const uint32_t hi = uint32_t(b >> 32);
+  const int r = qp.fe - int((hi >> 20) & 0x7ffu);
+  const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+  const long long v = r < 64 ? (long long)((m << 8) >> r) : 0ll;
+  const long long t = (int32_t(hi) < 0 ? -v : v) - qp.fo[d];
+  const unsigned long long x = __umul64hi((unsigned long long)(t < 0 ? 0 : t), qp.fw) + (1ull << (qp.fs - 1));
+  const uint32_t f = uint32_t(x >> (qp.fs - 24)) & 0xffffffu;  // fraction of x + 1/2 in 2^-24
+  if (__builtin_expect(f - 16u < 0xffffffu - 32u, 1)) return uint32_t(x >> qp.fs);
+  return quant_exact_call64(p, qp.o[d], qp.s);
+}
+
 template <typename C>
 struct CodeVec;
 template <>
@@ -353,15 +372,18 @@ __global__ void __launch_bounds__(kThreads) k_quant_f32(const float *__restrict_
   }
 }
 
-template <typename C, bool VEC, bool FAST>
-__global__ void __launch_bounds__(kThreads) k_quant_f64(const double *__restrict__ pos, uint64_t n, QuantParams qp,
+// MODE: 0 the definition, 1 two double operations, 2 fixed point.
+template <typename C, bool VEC, int MODE>
+__global__ void __launch_bounds__(kThreads) k_quant_f64(const double *__restrict__ pos, uint64_t n,
+                                                        const __grid_constant__ QuantParams qp,
                                                         C *__restrict__ qx, C *__restrict__ qy, C *__restrict__ qz,
                                                         uint32_t *__restrict__ idx) {
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  auto quant_exact = [&](double p, double o, double s) -> uint32_t {
-    if (FAST) return quant_fast64(p, o, s, qp.inv);
-    return pcx::quant_exact(p, o, s);
+  auto Q = [&](double p, int d) -> uint32_t {
+    if (MODE == 2) return quant_fixed64(p, d, qp);
+    if (MODE == 1) return quant_fast64(p, qp.o[d], qp.s, qp.inv);
+    return quant_exact(p, qp.o[d], qp.s);
   };
   uint64_t done = 0;
   if (VEC) {
@@ -369,17 +391,17 @@ __global__ void __launch_bounds__(kThreads) k_quant_f64(const double *__restrict
     const uint64_t groups = n / 2;
     for (uint64_t g = tid; g < groups; g += stride) {
       double2 a = __ldcs(p2 + 3 * g), b = __ldcs(p2 + 3 * g + 1), c = __ldcs(p2 + 3 * g + 2);
-      CodeVec<C>::put2(qx, 2 * g, quant_exact(a.x, qp.o[0], qp.s), quant_exact(b.y, qp.o[0], qp.s));
-      CodeVec<C>::put2(qy, 2 * g, quant_exact(a.y, qp.o[1], qp.s), quant_exact(c.x, qp.o[1], qp.s));
-      CodeVec<C>::put2(qz, 2 * g, quant_exact(b.x, qp.o[2], qp.s), quant_exact(c.y, qp.o[2], qp.s));
+      CodeVec<C>::put2(qx, 2 * g, Q(a.x, 0), Q(b.y, 0));
+      CodeVec<C>::put2(qy, 2 * g, Q(a.y, 1), Q(c.x, 1));
+      CodeVec<C>::put2(qz, 2 * g, Q(b.x, 2), Q(c.y, 2));
       if (idx) __stcs(reinterpret_cast<uint2 *>(idx + 2 * g), make_uint2(uint32_t(2 * g), uint32_t(2 * g + 1)));
     }
     done = groups * 2;
   }
   for (uint64_t i = done + tid; i < n; i += stride) {
-    qx[i] = (C)quant_exact(pos[3 * i + 0], qp.o[0], qp.s);
-    qy[i] = (C)quant_exact(pos[3 * i + 1], qp.o[1], qp.s);
-    qz[i] = (C)quant_exact(pos[3 * i + 2], qp.o[2], qp.s);
+    qx[i] = (C)Q(pos[3 * i + 0], 0);
+    qy[i] = (C)Q(pos[3 * i + 1], 1);
+    qz[i] = (C)Q(pos[3 * i + 2], 2);
     if (idx) idx[i] = uint32_t(i);
   }
 }
@@ -425,13 +447,11 @@ cudaError_t quant_dispatch(const QuantLaunch &a, cudaStream_t st) {
     else k_quant_f32<C, false, false><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx);
   } else {
     const double *p = static_cast<const double *>(a.pos);
-    if (a.fast) {
-      if (a.vec) k_quant_f64<C, true, true><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx);
-      else k_quant_f64<C, false, true><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx);
-    } else {
-      if (a.vec) k_quant_f64<C, true, false><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx);
-      else k_quant_f64<C, false, false><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx);
-    }
+    const int mode = a.fixed ? 2 : (a.fast ? 1 : 0);
+    auto run = [&](auto kernel) { kernel<<<a.blocks, kThreads, 0, st>>>(p, a.n, a.qp, qx, qy, qz, a.idx); };
+    if (mode == 2) a.vec ? run(k_quant_f64<C, true, 2>) : run(k_quant_f64<C, false, 2>);
+    else if (mode == 1) a.vec ? run(k_quant_f64<C, true, 1>) : run(k_quant_f64<C, false, 1>);
+    else a.vec ? run(k_quant_f64<C, true, 0>) : run(k_quant_f64<C, false, 0>);
   }
   return cudaGetLastError();
 }

@@ -542,6 +542,30 @@ int lattice_from_range(const RangeResult &rr, int dtype, int mode, double eb, La
   return PC_OK;
 }
 
+// Parameters of the fixed-point quantizer (k_quant.cu); false where the step is too
+// fine beside the coordinates for it.
+bool fixed_point(const RangeResult &rr, const Lattice &L, QuantParams &q) {
+  double m = 0.0;
+  for (int d = 0; d < 3; ++d) m = std::max(m, std::max(std::fabs(rr.lo[d]), std::fabs(rr.hi[d])));
+  int e = 0;
+  std::frexp(m, &e);  // m < 2^e
+  if (!(m > 0.0) || e < -900 || e > 900) return false;
+  const double units = std::ldexp(L.s, 61 - e);  // s / u
+  int es = 0;
+  std::frexp(units, &es);  // units in [2^(es - 1), 2^es)
+  if (es - 1 < 26 || es > 62) return false;
+  q.fe = 1022 + e;         // biased exponent of the largest coordinates
+  q.fs = es - 2;           // fw in (2^62, 2^63]
+  const double w = std::ldexp(1.0, 64 + q.fs) / units;
+  if (!(w <= 0x1p63)) return false;
+  q.fw = (unsigned long long)w;
+  for (int d = 0; d < 3; ++d) {
+    q.fo[d] = (long long)std::ldexp(std::fabs(L.o[d]), 61 - e);
+    if (L.o[d] < 0.0) q.fo[d] = -q.fo[d];
+  }
+  return true;
+}
+
 #define PC_TRY(x)                        \
   do {                                   \
     cudaError_t e_ = (x);                \
@@ -676,6 +700,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     qa.qp.inv = inv;
     qa.fast = dtype == PC_F32 ? (qmax < (1u << 22) && inv > 0x1p-100 && inv < 0x1p100)
                               : (inv > 0x1p-1000 && inv < 0x1p1000);
+    qa.fixed = dtype == PC_F64 && !L.raw && fixed_point(rr, L, qa.qp);
     qa.qp.raw = L.raw;
     for (int d = 0; d < 3; ++d) {
       qa.qp.lo[d] = L.lo[d];

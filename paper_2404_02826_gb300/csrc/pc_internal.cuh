@@ -51,6 +51,12 @@ struct QuantParams {
   float of[3];   // origin as float (exact for float input)
   float rh, rl;  // 1/s as an unevaluated float sum rh + rl
   double inv;    // fl(1/s)
+  // double input in fixed point (QuantLaunch.fixed): p = +-m 2^(e - 1075) is +-(m << 8) >> (fe - e)
+  // in units u = 2^-61 of the power of two above every |p|; fo: the origin in them; the code with
+  // fs fraction bits is the high word of (p - o) fw, fw = 2^(64 + fs) / (s / u)
+  long long fo[3];
+  unsigned long long fw;
+  int32_t fe, fs;
   uint32_t raw;      // bit d: axis d stored losslessly; its code is the split key
   double lo[3];      //   floor((p - lo) / span * 2^29) (span = hi - lo; 0 when span is 0)
   double span[3];
@@ -148,6 +154,7 @@ struct QuantLaunch {
   int code_bytes;  // 2 or 4
   bool vec;
   bool fast;
+  bool fixed;  // double input: the fixed-point quantizer
   QuantParams qp;
   void *q[3];
   uint32_t *idx;  // optional identity permutation

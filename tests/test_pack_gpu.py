@@ -32,6 +32,20 @@ def test_widths_and_leaf_sizes(pc, oracle_mod, n, r, eb):
     _check(pc, oracle_mod, synth.uniform(n, seed=n + r, dtype=np.float64), eb, r)
 
 
+# float64 positions and bounds on both sides of the fixed-point quantizer's rule (s >= 2^-35 of
+# the power of two above the coordinates), on lattice midpoints, with both signs and zeros
+@pytest.mark.parametrize("offset,span", [(0.0, 1.0), (-0.5, 1.0), (1e6, 3.0), (-1e9, 0.25), (-3e4, 7e4), (1e-3, 1e-6)])
+@pytest.mark.parametrize("eb", [1e-1, 1e-3, 1e-5, 1e-8])
+def test_float64_quantizer(pc, oracle_mod, offset, span, eb):
+    rng = np.random.default_rng(17)
+    pos = offset + span * rng.random((6_000, 3))
+    pos[::7] = offset + span * np.round(rng.random((858, 3)) * 64) / 64
+    pos[::50] = np.where(rng.random((120, 3)) < 0.5, 0.0 if offset <= 0.0 <= offset + span else offset, pos[::50])
+    s = 2 * eb * span
+    pos[::11] = np.minimum(offset + s * (rng.integers(0, int(0.5 / eb) - 1, (546, 3)) + 0.5), offset + span)
+    _check(pc, oracle_mod, pos, eb, 512)
+
+
 def _uneven(n, seed):
     """Half the particles in a corner of a thousandth of the box, half spread over it."""
     rng = np.random.default_rng(seed)
