@@ -22,13 +22,13 @@
  *     naturally aligned (4 or 8 bytes); 16-byte alignment selects vector loads.
  *   - Every call returns a pc_status.  After an error no output is valid.
  *   - Calls are synchronous with respect to the host where stated: compress
- *     and decompress each read a few bytes back (the value range, then the
+ *     and decompress each wait for a few bytes (the value range, then the
  *     final size or the error word) and so return with their work finished.
- *     Those bytes pass through page-locked host blocks of 4 KB that the
- *     library allocates on first use, sixteen at a time, and keeps for the
- *     life of the process (one block per call in flight; decompression also
- *     keeps one CUDA event per call in flight); pc_compress_noalloc allocates
- *     none (it uses blocks that exist, else plain copies).
+ *     The kernels write those bytes into page-locked host blocks of 4 KB, where
+ *     the calling thread watches for them; the library allocates the blocks on
+ *     first use, sixteen at a time, and keeps them for the life of the process
+ *     (one block per call in flight); pc_compress_noalloc allocates none (it
+ *     uses blocks that exist, else plain copies).
  *
  * Stream format (little-endian), version 1:
  *   header, 96 bytes:

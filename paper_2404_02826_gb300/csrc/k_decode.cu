@@ -197,6 +197,9 @@ __global__ void k_decode_start(const uint8_t *stream, uint32_t *ws64, uint8_t *h
   if (t < 16) ws64[t] = 0u;
   if (t < kHeaderBytes / 16)
     reinterpret_cast<uint4 *>(host_header)[t] = __ldg(reinterpret_cast<const uint4 *>(stream) + t);
+  __threadfence_system();
+  __syncwarp();
+  if (t == 0) reinterpret_cast<volatile uint32_t *>(host_header)[kHeaderBytes / 4 + 1] = 1u;
 }
 
 // k_validate with the header read on the device: a fixed grid strides over the
@@ -694,7 +697,15 @@ __global__ void k_header(HeaderLaunch a) {
   uint4 *dst = reinterpret_cast<uint4 *>(a.out);
   const uint4 *src = reinterpret_cast<const uint4 *>(h);
   for (int i = 0; i < int(kHeaderBytes / 16); ++i) dst[i] = src[i];
-  *a.total_bytes = uint64_t(kHeaderBytes) + uint64_t(kLeafBytes) * a.num_leaves + 4ull * words;
+  const uint64_t total = uint64_t(kHeaderBytes) + uint64_t(kLeafBytes) * a.num_leaves + 4ull * words;
+  *a.total_bytes = total;
+  if (a.host_end) {
+    volatile CallEnd *const end = a.host_end;
+    end->total = total;
+    end->err = *reinterpret_cast<volatile uint32_t *>(a.err);
+    __threadfence_system();
+    end->done = 1u;
+  }
 }
 
 template <typename T, bool FAST, bool VEC>

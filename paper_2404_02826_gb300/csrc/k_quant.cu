@@ -77,9 +77,78 @@ struct F64Acc {
   }
 };
 
+// The last block to finish folds the per-block partials (one launch instead of
+// two).  Comparisons go through the same order-preserving integer keys, so no
+// FP64 arithmetic is involved.  Every thread of every block calls it, after its
+// block's partial is written by thread 0.
+__device__ __forceinline__ void range_final(const double *partial, RangeResult *res, uint32_t *ticket,
+                                            RangeResult *host_res, uint32_t *host_flag) {
+  __shared__ unsigned long long kmn[3][kThreads / 32], kmx[3][kThreads / 32];
+  __shared__ int fbad;
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    fbad = 0;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) + 1u == gridDim.x;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  unsigned long long mn[3], mx[3];
+  bool bad = false;
+  for (int d = 0; d < 3; ++d) {
+    mn[d] = ~0ull;
+    mx[d] = 0;
+  }
+  for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    const double *p = partial + 8 * b;
+    for (int d = 0; d < 3; ++d) {
+      const unsigned long long a = f64_key(__ldcg(p + d)), c = f64_key(__ldcg(p + 3 + d));
+      mn[d] = a < mn[d] ? a : mn[d];
+      mx[d] = c > mx[d] ? c : mx[d];
+    }
+    bad |= __ldcg(p + 6) != 0.0;
+  }
+  for (int d = 0; d < 3; ++d) {
+    unsigned long long a = mn[d], b = mx[d];
+    for (int o = 16; o; o >>= 1) {
+      const unsigned long long x = __shfl_xor_sync(0xffffffffu, a, o), y = __shfl_xor_sync(0xffffffffu, b, o);
+      a = x < a ? x : a;
+      b = y > b ? y : b;
+    }
+    if ((threadIdx.x & 31) == 0) {
+      kmn[d][threadIdx.x >> 5] = a;
+      kmx[d][threadIdx.x >> 5] = b;
+    }
+  }
+  if (bad) fbad = 1;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    RangeResult r;
+    for (int d = 0; d < 3; ++d) {
+      unsigned long long a = kmn[d][0], b = kmx[d][0];
+      for (int w = 1; w < kThreads / 32; ++w) {
+        a = kmn[d][w] < a ? kmn[d][w] : a;
+        b = kmx[d][w] > b ? kmx[d][w] : b;
+      }
+      r.lo[d] = f64_from_key(a);
+      r.hi[d] = f64_from_key(b);
+    }
+    r.nonfinite = fbad ? 1u : 0u;
+    r.pad = 0;
+    *res = r;
+    if (host_res) {
+      *host_res = r;
+      __threadfence_system();
+      *reinterpret_cast<volatile uint32_t *>(host_flag) = 1u;
+    }
+  }
+}
+
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) k_range_f32(const float *__restrict__ pos, uint64_t n,
-                                                        double *__restrict__ partial) {
+                                                        double *partial, RangeResult *res, uint32_t *ticket,
+                                                        RangeResult *host_res, uint32_t *host_flag) {
   F32Acc acc;
   acc.init();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
@@ -129,11 +198,13 @@ __global__ void __launch_bounds__(kThreads) k_range_f32(const float *__restrict_
     }
     out[6] = sbad ? 1.0 : 0.0;
   }
+  range_final(partial, res, ticket, host_res, host_flag);
 }
 
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) k_range_f64(const double *__restrict__ pos, uint64_t n,
-                                                        double *__restrict__ partial) {
+                                                        double *partial, RangeResult *res, uint32_t *ticket,
+                                                        RangeResult *host_res, uint32_t *host_flag) {
   F64Acc acc;
   acc.init();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
@@ -183,58 +254,7 @@ __global__ void __launch_bounds__(kThreads) k_range_f64(const double *__restrict
     }
     out[6] = sbad ? 1.0 : 0.0;
   }
-}
-
-// One block folds the per-block partials.  Comparisons go through the same
-// order-preserving integer keys, so no FP64 arithmetic is involved.
-__global__ void k_range_final(const double *__restrict__ partial, int blocks, RangeResult *__restrict__ res) {
-  __shared__ unsigned long long smn[3][32], smx[3][32];
-  __shared__ int sbad;
-  if (threadIdx.x == 0) sbad = 0;
-  __syncthreads();
-  unsigned long long mn[3], mx[3];
-  bool bad = false;
-  for (int d = 0; d < 3; ++d) {
-    mn[d] = ~0ull;
-    mx[d] = 0;
-  }
-  for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
-    const double *p = partial + 8 * b;
-    for (int d = 0; d < 3; ++d) {
-      unsigned long long a = f64_key(p[d]), c = f64_key(p[3 + d]);
-      mn[d] = a < mn[d] ? a : mn[d];
-      mx[d] = c > mx[d] ? c : mx[d];
-    }
-    bad |= p[6] != 0.0;
-  }
-  for (int d = 0; d < 3; ++d) {
-    unsigned long long a = mn[d], b = mx[d];
-    for (int o = 16; o; o >>= 1) {
-      unsigned long long x = __shfl_xor_sync(0xffffffffu, a, o), y = __shfl_xor_sync(0xffffffffu, b, o);
-      a = x < a ? x : a;
-      b = y > b ? y : b;
-    }
-    if ((threadIdx.x & 31) == 0) {
-      smn[d][threadIdx.x >> 5] = a;
-      smx[d][threadIdx.x >> 5] = b;
-    }
-  }
-  if (bad) sbad = 1;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int warps = blockDim.x / 32;
-    for (int d = 0; d < 3; ++d) {
-      unsigned long long a = smn[d][0], b = smx[d][0];
-      for (int w = 1; w < warps; ++w) {
-        a = smn[d][w] < a ? smn[d][w] : a;
-        b = smx[d][w] > b ? smx[d][w] : b;
-      }
-      res->lo[d] = f64_from_key(a);
-      res->hi[d] = f64_from_key(b);
-    }
-    res->nonfinite = sbad ? 1u : 0u;
-    res->pad = 0;
-  }
+  range_final(partial, res, ticket, host_res, host_flag);
 }
 
 // -------------------------------------------------------------------------
@@ -460,16 +480,16 @@ cudaError_t quant_dispatch(const QuantLaunch &a, cudaStream_t st) {
 
 cudaError_t launch_range(const RangeLaunch &a, cudaStream_t st) {
   TraceScope ts("k_range", st);
+  auto run = [&](auto kernel, auto p) {
+    kernel<<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial, a.result, a.ticket, a.host_result, a.host_flag);
+  };
   if (a.dtype == 0) {
     const float *p = static_cast<const float *>(a.pos);
-    if (a.vec) k_range_f32<true><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial);
-    else k_range_f32<false><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial);
+    a.vec ? run(k_range_f32<true>, p) : run(k_range_f32<false>, p);
   } else {
     const double *p = static_cast<const double *>(a.pos);
-    if (a.vec) k_range_f64<true><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial);
-    else k_range_f64<false><<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial);
+    a.vec ? run(k_range_f64<true>, p) : run(k_range_f64<false>, p);
   }
-  k_range_final<<<1, 1024, 0, st>>>(a.partial, a.blocks, a.result);
   return cudaGetLastError();
 }
 

@@ -54,69 +54,58 @@ void pinned_give(void *p) {
   g_pinned_free.push_back(p);
 }
 
-// Events without timing, per device, kept for the life of the process.
-std::vector<cudaEvent_t> g_events[64];
-
-cudaEvent_t event_take(int dev) {
-  {
-    std::lock_guard<std::mutex> g(g_pinned_mu);
-    std::vector<cudaEvent_t> &v = g_events[dev & 63];
-    if (!v.empty()) {
-      cudaEvent_t e = v.back();
-      v.pop_back();
-      return e;
-    }
-  }
-  cudaEvent_t e = nullptr;
-  if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return e;
-}
-
-void event_give(int dev, cudaEvent_t e) {
-  std::lock_guard<std::mutex> g(g_pinned_mu);
-  g_events[dev & 63].push_back(e);
-}
 }  // namespace
 
-HeaderCopy::~HeaderCopy() {
-  if (!done) return;  // a copy that may still be in flight keeps its block and event
-  if (blk) pinned_give(blk);
-  if (ev) event_give(dev, ev);
+cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st) {
+  for (uint32_t spins = 0;; ++spins) {
+    if (*word != unset) break;
+    if ((spins & 4095u) != 4095u) continue;
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaSuccess) break;  // done, the word as the kernels left it
+    if (e != cudaErrorNotReady) return e;
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  return cudaSuccess;
 }
 
-cudaError_t HeaderCopy::start(const void *src, uint32_t *ws64, cudaStream_t st) {
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  blk = pinned_take();
-  ev = blk ? event_take(dev) : nullptr;
-  if (ev && cudaHostGetDevicePointer(&dblk, blk, 0) != cudaSuccess) {
+HostBlock::HostBlock() {
+  if (trace_enabled()) return;
+  void *h = pinned_take(), *d = nullptr;
+  if (!h) return;
+  if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
     cudaGetLastError();
-    dblk = nullptr;
+    pinned_give(h);
+    return;
   }
-  if (!dblk) {  // no staging: plain calls, waited for here
-    if (ev) event_give(dev, ev);
-    if (blk) pinned_give(blk);
-    ev = nullptr;
-    blk = nullptr;
-    dblk = nullptr;
+  host = static_cast<uint8_t *>(h);
+  dev = static_cast<uint8_t *>(d);
+}
+
+HostBlock::~HostBlock() {
+  if (host && !pending) pinned_give(host);
+}
+
+cudaError_t HeaderCopy::start(const void *src, uint32_t *ws64, cudaStream_t stream) {
+  st = stream;
+  if (!b.host) {  // no staging: plain calls, waited for here
     done = true;
-    e = cudaMemsetAsync(ws64, 0, 64, st);
+    cudaError_t e = cudaMemsetAsync(ws64, 0, 64, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, src, kHeaderBytes, cudaMemcpyDefault, st);
     return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
   }
-  e = launch_decode_start(static_cast<const uint8_t *>(src), ws64, static_cast<uint8_t *>(dblk), st);
-  if (e == cudaSuccess) e = cudaEventRecord(ev, st);
-  return e;
+  *reinterpret_cast<volatile uint32_t *>(b.host + kHeaderBytes + 4) = 0u;
+  b.pending = true;
+  return launch_decode_start(static_cast<const uint8_t *>(src), ws64, b.dev, st);
 }
 
 cudaError_t HeaderCopy::finish() {
   if (done) return cudaSuccess;
-  const cudaError_t e = cudaEventSynchronize(ev);
+  const volatile uint32_t *flag = reinterpret_cast<volatile uint32_t *>(b.host + kHeaderBytes + 4);
+  const cudaError_t e = wait_word(flag, 0u, st);
   if (e != cudaSuccess) return e;
-  std::memcpy(h, blk, kHeaderBytes);
+  if (*flag == 0u) return cudaErrorUnknown;
+  std::memcpy(h, b.host, kHeaderBytes);
+  b.pending = false;
   done = true;
   return cudaSuccess;
 }
@@ -442,8 +431,8 @@ int make_plan(uint64_t n, int dtype, const pc_config *cfg, bool idx, int sm_coun
   o = align_up(o + 4 * (hist_bins ? hist_bins : 1));
   p.off_tiles = o;
   o = align_up(o + 8 * (tiles ? tiles : 1));
-  p.off_tickets = o;  // one per level over HBM, the subtree's, the leaf-size search pass's
-  o = align_up(o + 4 * (p.levels + 2));
+  p.off_tickets = o;  // one per level over HBM, the subtree's, the leaf-size search pass's, the range's
+  o = align_up(o + 4 * (p.levels + 3));
   p.off_tunecost = o;
   o = align_up(o + 8 * (kSubMaxLevels + 1));
   p.off_split = o;
@@ -628,6 +617,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   uint32_t *err = reinterpret_cast<uint32_t *>(ws + p.off_err);
   uint64_t *total_dev = reinterpret_cast<uint64_t *>(ws + p.off_total);
+  HostBlock hb;  // the value range, then the call's end
   PC_TRY(cudaMemsetAsync(ws + p.off_zero, 0, p.zero_bytes, st));
 
   HeaderLaunch hl = {};
@@ -653,10 +643,25 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     ra.vec = reinterpret_cast<uintptr_t>(positions) % 16 == 0;
     ra.partial = reinterpret_cast<double *>(ws + p.off_partial);
     ra.result = reinterpret_cast<RangeResult *>(ws + p.off_range);
-    ra.blocks = p.range_blocks;
+    ra.ticket = reinterpret_cast<uint32_t *>(ws + p.off_tickets) + p.levels + 2;
+    ra.blocks = int(std::min<uint64_t>(uint64_t(p.range_blocks), (n + 1023) / 1024));
+    volatile uint32_t *const flag = reinterpret_cast<volatile uint32_t *>(hb.host + 128);
+    if (hb.host) {
+      *flag = 0u;
+      hb.pending = true;
+      ra.host_result = reinterpret_cast<RangeResult *>(hb.dev);
+      ra.host_flag = reinterpret_cast<uint32_t *>(hb.dev + 128);
+    }
     PC_TRY(launch_range(ra, st));
     RangeResult rr;
-    PC_TRY(read_back(&rr, ra.result, sizeof(rr), st));
+    if (hb.host) {
+      PC_TRY(wait_word(flag, 0u, st));
+      if (*flag == 0u) return PC_ERR_CUDA;
+      std::memcpy(&rr, hb.host, sizeof(rr));
+      hb.pending = false;
+    } else {
+      PC_TRY(read_back(&rr, ra.result, sizeof(rr), st));
+    }
     rc = lattice_from_range(rr, dtype, eb_mode, eb, L);
     if (rc) return rc;
     // lossless axes (Sec. 4.1, m_d > M): the plain stream only; the reduction,
@@ -707,7 +712,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       qa.qp.span[d] = L.span[d];
     }
     qa.idx = idx_a;
-    qa.blocks = 8 * device_sm_count();
+    qa.blocks = int(std::min<uint64_t>(8 * uint64_t(device_sm_count()), (n + 1023) / 1024));
     PC_TRY(launch_quantize(qa, st));
 
     // a3: the k-d levels, down to the leaves (autotuning: down to the deepest candidate at most);
@@ -1174,13 +1179,23 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
   hl.eps = L.eps;
   hl.s = L.s;
   for (int d = 0; d < 3; ++d) hl.o[d] = L.o[d];
-  PC_TRY(launch_header(hl, st));
-  struct {
-    uint64_t total;
-    uint32_t err;
-  } back = {0, 0};
-  const ReadBack rb[2] = {{&back.total, total_dev, 8}, {&back.err, err, 4}};
-  PC_TRY(read_back(rb, 2, st));
+  CallEnd back = {};
+  if (hb.host) {
+    volatile CallEnd *const end = reinterpret_cast<volatile CallEnd *>(hb.host + 192);
+    end->done = 0u;
+    hb.pending = true;
+    hl.host_end = reinterpret_cast<CallEnd *>(hb.dev + 192);
+    PC_TRY(launch_header(hl, st));
+    PC_TRY(wait_word(&end->done, 0u, st));
+    if (end->done == 0u) return PC_ERR_CUDA;
+    back.total = end->total;
+    back.err = end->err;
+    hb.pending = false;
+  } else {
+    PC_TRY(launch_header(hl, st));
+    const ReadBack rb[2] = {{&back.total, total_dev, 8}, {&back.err, err, 4}};
+    PC_TRY(read_back(rb, 2, st));
+  }
   trace_flush();
   if (back.err & kErrTimeout) return PC_ERR_TIMEOUT;
   if (back.err) return PC_ERR_CUDA;
@@ -1289,16 +1304,16 @@ int decompress_impl(const void *stream_data, uint64_t stream_bytes, void *out_po
   // mark that stays when a block returned early (then the word is read back here)
   constexpr uint32_t kUnset = 0xffffffffu;
   da.host_err = da.raw ? nullptr : hc.host_err_dev();
-  if (da.host_err) *hc.host_err() = kUnset;
+  if (da.host_err) {
+    *hc.host_err() = kUnset;
+    hc.b.pending = true;
+  }
   PC_TRY(launch_decode(da, st));
   uint32_t e = kUnset;
   if (da.host_err) {
-    const cudaError_t se = cudaStreamSynchronize(st);
-    if (se != cudaSuccess) {
-      hc.done = false;  // the decoder may still write into the staging block: it is not reused
-      return PC_ERR_CUDA;
-    }
+    PC_TRY(wait_word(hc.host_err(), kUnset, st));
     e = *hc.host_err();
+    hc.b.pending = false;
   }
   if (e == kUnset) PC_TRY(read_back(&e, err, 4, st));
   trace_flush();

@@ -143,6 +143,9 @@ struct RangeLaunch {
   bool vec;
   double *partial;  // [blocks][7]
   RangeResult *result;
+  uint32_t *ticket;       // zero on entry
+  RangeResult *host_result;  // optional, page-locked host memory: the result once more, then
+  uint32_t *host_flag;       // a 1 here
   int blocks;
 };
 cudaError_t launch_range(const RangeLaunch &a, cudaStream_t st);
@@ -298,6 +301,13 @@ cudaError_t launch_subtree(const SubtreeLaunch &a, cudaStream_t st);
 // axis or the leaf-size search's pass).
 uint32_t subtree_capacity(int code_bytes, bool with_idx, bool plain);
 
+// What a compression leaves for the host.
+struct CallEnd {
+  uint64_t total;  // stream bytes
+  uint32_t err;
+  uint32_t done;
+};
+
 struct HeaderLaunch {
   uint8_t *out;
   uint64_t n;
@@ -309,6 +319,7 @@ struct HeaderLaunch {
   uint64_t *total_bytes;        // device slot read back by the host
   uint32_t *err;
   uint32_t raw;                 // lossless-axis mask (header byte 84)
+  CallEnd *host_end;            // optional, page-locked host memory: the call's end, `done` last
 };
 cudaError_t launch_header(const HeaderLaunch &a, cudaStream_t st);
 
@@ -344,7 +355,7 @@ cudaError_t launch_decode_prologue(const uint8_t *stream, uint64_t stream_bytes,
                                    int32_t *qb, void *tab, void *chunks, cudaStream_t st);
 // The first launch of a decompression: clears the workspace's first 64 bytes (error
 // word, block count, code bounds) and copies the stream's header into page-locked
-// host memory (`host_header`, 16-byte aligned).
+// host memory (`host_header`, 16-byte aligned), then a 1 into its 26th word.
 cudaError_t launch_decode_start(const uint8_t *stream, uint32_t *ws64, uint8_t *host_header, cudaStream_t st);
 
 // Many streams decoded by one set of launches: each stream's plain launch
@@ -394,29 +405,40 @@ inline cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStrea
   return read_back(&r, 1, st);
 }
 
+// Waits until the word, in page-locked host memory that a kernel of `st` writes,
+// is no longer `unset`, or the stream is done.  The word is watched by the
+// calling thread: a result arrives 1 to 2 us after it is written, a copy and a
+// synchronisation of the stream take 8.
+cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st);
+
+// A page-locked staging block for the results that kernels write to host memory
+// (null without one, and while kernels are traced: each then needs its events).
+// A block that a kernel may still write into is not reused.
+struct HostBlock {
+  uint8_t *host = nullptr, *dev = nullptr;
+  bool pending = false;  // a kernel that writes into it is queued and has not been waited for
+  HostBlock();
+  ~HostBlock();
+  HostBlock(const HostBlock &) = delete;
+  HostBlock &operator=(const HostBlock &) = delete;
+};
+
 // A stream header on its way to host memory: written into a page-locked block
 // by launch_decode_start (which also clears the workspace's first 64 bytes) and
-// waited for on an event (finish), so that what is queued on the stream after
-// start runs meanwhile; the block's word after the header then receives the
-// decoder's error word.  Without a block or an event, start clears and copies
-// with plain calls and waits for them.
+// waited for there (finish), so that what is queued on the stream after start
+// runs meanwhile; the block's word after the header then receives the decoder's
+// error word.  Without a block, start clears and copies with plain calls and
+// waits for them.
 struct HeaderCopy {
   uint8_t h[kHeaderBytes];
-  void *blk = nullptr;   // the staging block, host address
-  void *dblk = nullptr;  // and device address
-  cudaEvent_t ev = nullptr;
-  int dev = 0;
+  HostBlock b;
+  cudaStream_t st = nullptr;
   bool done = false;  // h holds the header (or the copy failed before it was queued)
-  cudaError_t start(const void *src, uint32_t *ws64, cudaStream_t st);
+  cudaError_t start(const void *src, uint32_t *ws64, cudaStream_t stream);
   cudaError_t finish();
   // the word after the header in the staging block (null without one): host, device address
-  volatile uint32_t *host_err() const {
-    return blk ? reinterpret_cast<volatile uint32_t *>(static_cast<uint8_t *>(blk) + kHeaderBytes) : nullptr;
-  }
-  uint32_t *host_err_dev() const {
-    return dblk ? reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(dblk) + kHeaderBytes) : nullptr;
-  }
-  ~HeaderCopy();
+  volatile uint32_t *host_err() const { return b.host ? reinterpret_cast<volatile uint32_t *>(b.host + kHeaderBytes) : nullptr; }
+  uint32_t *host_err_dev() const { return b.dev ? reinterpret_cast<uint32_t *>(b.dev + kHeaderBytes) : nullptr; }
 };
 
 // Blocks of kernel F resident per SM with `smem` bytes of dynamic shared
