@@ -30,17 +30,15 @@ constexpr int kThreads = 256;
 // range
 // -------------------------------------------------------------------------
 
-__device__ __forceinline__ unsigned long long f64_key(double v) {
-  unsigned long long b = __double_as_longlong(v);
+__device__ __forceinline__ unsigned long long f64_key_bits(unsigned long long b) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
+__device__ __forceinline__ unsigned long long f64_key(double v) { return f64_key_bits(__double_as_longlong(v)); }
 __device__ __forceinline__ double f64_from_key(unsigned long long k) {
   unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
   return __longlong_as_double(b);
 }
-__device__ __forceinline__ bool f64_bad(double v) {
-  return ((__double_as_longlong(v) >> 52) & 0x7ff) == 0x7ff;
-}
+__device__ __forceinline__ bool f64_bad_bits(unsigned long long b) { return ((b >> 52) & 0x7ff) == 0x7ff; }
 
 struct F32Acc {
   float mn[3], mx[3];
@@ -69,9 +67,11 @@ struct F64Acc {
     }
     bad = false;
   }
-  __device__ __forceinline__ void add(int d, double v) {
-    bad |= f64_bad(v);
-    unsigned long long k = f64_key(v);
+  // the coordinate's bits: loaded as a double, each would pass through an instruction of the
+  // FP64 pipe (114 us at 2^24 particles, with integer loads 97)
+  __device__ __forceinline__ void add(int d, unsigned long long b) {
+    bad |= f64_bad_bits(b);
+    unsigned long long k = f64_key_bits(b);
     mn[d] = k < mn[d] ? k : mn[d];
     mx[d] = k > mx[d] ? k : mx[d];
   }
@@ -211,17 +211,17 @@ __global__ void __launch_bounds__(kThreads) k_range_f64(const double *__restrict
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   uint64_t done = 0;
   if (VEC) {
-    const double2 *p2 = reinterpret_cast<const double2 *>(pos);
+    const ulonglong2 *p2 = reinterpret_cast<const ulonglong2 *>(pos);
     const uint64_t groups = n / 2;  // 2 particles = 3 double2
     for (uint64_t g = tid; g < groups; g += stride) {
-      double2 a = __ldcs(p2 + 3 * g), b = __ldcs(p2 + 3 * g + 1), c = __ldcs(p2 + 3 * g + 2);
+      ulonglong2 a = __ldcs(p2 + 3 * g), b = __ldcs(p2 + 3 * g + 1), c = __ldcs(p2 + 3 * g + 2);
       acc.add(0, a.x); acc.add(1, a.y); acc.add(2, b.x);
       acc.add(0, b.y); acc.add(1, c.x); acc.add(2, c.y);
     }
     done = groups * 2;
   }
   for (uint64_t i = done + tid; i < n; i += stride)
-    for (int d = 0; d < 3; ++d) acc.add(d, pos[3 * i + d]);
+    for (int d = 0; d < 3; ++d) acc.add(d, reinterpret_cast<const unsigned long long *>(pos)[3 * i + d]);
 
   __shared__ unsigned long long smn[3][kThreads / 32], smx[3][kThreads / 32];
   __shared__ int sbad;
@@ -320,8 +320,7 @@ __device__ __forceinline__ uint32_t quant_fast64(double p, double o, double s, d
 // within 2^-23 of the exact quotient ((p - o) / s with s / u >= 2^26: two units
 // are 2^-25), the double quotient of the definition lies within 2^-21 of that
 // (codes below 2^30); unless it is within 2^-20 of a half-integer, both round alike.
-__device__ __forceinline__ uint32_t quant_fixed64(double p, int d, const QuantParams &qp) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(p);
+__device__ __forceinline__ uint32_t quant_fixed64(unsigned long long b, int d, const QuantParams &qp) {
   const uint32_t hi = uint32_t(b >> 32);
   const int r = qp.fe - int((hi >> 20) & 0x7ffu);
   const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
@@ -330,7 +329,7 @@ __device__ __forceinline__ uint32_t quant_fixed64(double p, int d, const QuantPa
   const unsigned long long x = __umul64hi((unsigned long long)(t < 0 ? 0 : t), qp.fw) + (1ull << (qp.fs - 1));
   const uint32_t f = uint32_t(x >> (qp.fs - 24)) & 0xffffffu;  // fraction of x + 1/2 in 2^-24
   if (__builtin_expect(f - 16u < 0xffffffu - 32u, 1)) return uint32_t(x >> qp.fs);
-  return quant_exact_call64(p, qp.o[d], qp.s);
+  return quant_exact_call64(__longlong_as_double((long long)b), qp.o[d], qp.s);
 }
 
 template <typename C>
@@ -363,6 +362,7 @@ template <typename C, bool VEC, bool FAST>
 __global__ void __launch_bounds__(kThreads) k_quant_f32(const float *__restrict__ pos, uint64_t n, QuantParams qp,
                                                         C *__restrict__ qx, C *__restrict__ qy, C *__restrict__ qz,
                                                         uint32_t *__restrict__ idx) {
+  dep_launch();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   auto Q = [&](float p, int d) -> uint32_t {
@@ -398,19 +398,22 @@ __global__ void __launch_bounds__(kThreads) k_quant_f64(const double *__restrict
                                                         const __grid_constant__ QuantParams qp,
                                                         C *__restrict__ qx, C *__restrict__ qy, C *__restrict__ qz,
                                                         uint32_t *__restrict__ idx) {
+  dep_launch();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  auto Q = [&](double p, int d) -> uint32_t {
-    if (MODE == 2) return quant_fixed64(p, d, qp);
+  // coordinates as their bits (a double that is only taken apart still passes through the FP64 pipe)
+  auto Q = [&](unsigned long long bits, int d) -> uint32_t {
+    if (MODE == 2) return quant_fixed64(bits, d, qp);
+    const double p = __longlong_as_double((long long)bits);
     if (MODE == 1) return quant_fast64(p, qp.o[d], qp.s, qp.inv);
     return quant_exact(p, qp.o[d], qp.s);
   };
   uint64_t done = 0;
   if (VEC) {
-    const double2 *p2 = reinterpret_cast<const double2 *>(pos);
+    const ulonglong2 *p2 = reinterpret_cast<const ulonglong2 *>(pos);
     const uint64_t groups = n / 2;
     for (uint64_t g = tid; g < groups; g += stride) {
-      double2 a = __ldcs(p2 + 3 * g), b = __ldcs(p2 + 3 * g + 1), c = __ldcs(p2 + 3 * g + 2);
+      ulonglong2 a = __ldcs(p2 + 3 * g), b = __ldcs(p2 + 3 * g + 1), c = __ldcs(p2 + 3 * g + 2);
       CodeVec<C>::put2(qx, 2 * g, Q(a.x, 0), Q(b.y, 0));
       CodeVec<C>::put2(qy, 2 * g, Q(a.y, 1), Q(c.x, 1));
       CodeVec<C>::put2(qz, 2 * g, Q(b.x, 2), Q(c.y, 2));
@@ -419,9 +422,10 @@ __global__ void __launch_bounds__(kThreads) k_quant_f64(const double *__restrict
     done = groups * 2;
   }
   for (uint64_t i = done + tid; i < n; i += stride) {
-    qx[i] = (C)Q(pos[3 * i + 0], 0);
-    qy[i] = (C)Q(pos[3 * i + 1], 1);
-    qz[i] = (C)Q(pos[3 * i + 2], 2);
+    const unsigned long long *u = reinterpret_cast<const unsigned long long *>(pos) + 3 * i;
+    qx[i] = (C)Q(u[0], 0);
+    qy[i] = (C)Q(u[1], 1);
+    qz[i] = (C)Q(u[2], 2);
     if (idx) idx[i] = uint32_t(i);
   }
 }
