@@ -193,6 +193,7 @@ __device__ __forceinline__ DevHeader read_header(const uint8_t *stream, uint64_t
 // (error word, the decoder's block count, code bounds) and copies the header
 // into page-locked host memory.
 __global__ void k_decode_start(const uint8_t *stream, uint32_t *ws64, uint8_t *host_header) {
+  dep_launch();
   const uint32_t t = threadIdx.x;
   if (t < 16) ws64[t] = 0u;
   if (t < kHeaderBytes / 16)
@@ -208,6 +209,8 @@ __global__ void k_decode_start(const uint8_t *stream, uint32_t *ws64, uint8_t *h
 // `chunk_cap` entries the workspace holds (the host then returns the error).
 __global__ void __launch_bounds__(256) k_validate_dev(const uint8_t *stream, uint64_t stream_bytes, uint64_t chunk_cap,
                                                       ChunkInfo *info, uint32_t *err, int32_t *qb) {
+  dep_launch();
+  dep_wait();
   const DevHeader H = read_header(stream, stream_bytes);
   if (!H.ok) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, kErrCorrupt);
@@ -359,7 +362,7 @@ __device__ __forceinline__ void fill_table(const DecodeLaunch &a) {
 // tables' completion (griddepcontrol.wait) before they read anything.
 template <typename T, bool FAST>
 __global__ void k_dtable(DecodeLaunch a) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dep_launch();
   if (*a.err) return;
   fill_table<T, FAST>(a);
 }
@@ -368,7 +371,8 @@ __global__ void k_dtable(DecodeLaunch a) {
 // 2^-100 .. 2^100).  Nothing for a failed validation or lossless axes.
 __global__ void k_dtable_dev(const uint8_t *stream, uint64_t stream_bytes, const uint32_t *err, int32_t *qb,
                              void *tab) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dep_launch();
+  dep_wait();
   if (*reinterpret_cast<const volatile uint32_t *>(err)) return;
   const DevHeader H = read_header(stream, stream_bytes);
   if (!H.ok || H.raw || H.n == 0) return;
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(kDecThreads) k_decode(DecodeLaunch a) {
   __shared__ __align__(16) DecSmem S;
   // launched as the tables' programmatic dependent: they (and the validation before
   // them) are complete and visible after this wait
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  dep_wait();
   if (call_failed(a.err)) return;  // validation failed: write nothing
   const uint64_t nchunks = (a.n + kChunk - 1) / kChunk;
   uint64_t chunk = blockIdx.x;
@@ -671,6 +675,7 @@ __global__ void __launch_bounds__(kDecThreads) k_decode_lossless(DecodeLaunch a)
 }
 
 __global__ void k_header(HeaderLaunch a) {
+  dep_wait();
   const uint64_t words = a.total_words ? *a.total_words : 0;
   __align__(16) uint8_t h[kHeaderBytes];
   for (int i = 0; i < int(kHeaderBytes); ++i) h[i] = 0;
@@ -722,17 +727,7 @@ cudaError_t decode_launch(const DecodeLaunch &a, cudaStream_t st, bool tables) {
   if (grid > decode_chunks(a.n)) grid = decode_chunks(a.n);
   TraceScope ts("k_decode", st);
   // a programmatic dependent of the tables: its blocks are placed while they are filled
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(kDecThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_decode<T, FAST, VEC>, a);
+  return launch_dependent(true, k_decode<T, FAST, VEC>, dim3(unsigned(grid)), dim3(kDecThreads), 0, st, a);
 }
 
 template <typename T, bool FAST>
@@ -1036,8 +1031,7 @@ uint64_t decode_chunk_bytes(uint64_t n) { return decode_chunks(n) * sizeof(Chunk
 
 cudaError_t launch_header(const HeaderLaunch &a, cudaStream_t st) {
   TraceScope ts("k_header", st);
-  k_header<<<1, 1, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(true, k_header, dim3(1), dim3(1), 0, st, a);
 }
 
 cudaError_t launch_gather_headers(const uint8_t *const *streams, uint32_t count, uint8_t *dst, cudaStream_t st) {
@@ -1119,12 +1113,13 @@ cudaError_t launch_decode_prologue(const uint8_t *stream, uint64_t stream_bytes,
                                    int32_t *qb, void *tab, void *chunks, cudaStream_t st) {
   {
     TraceScope ts("k_validate", st);
-    k_validate_dev<<<unsigned(4 * device_sm_count()), 256, 0, st>>>(stream, stream_bytes, chunk_cap,
-                                                                    static_cast<ChunkInfo *>(chunks), err, qb);
+    const cudaError_t e = launch_dependent(true, k_validate_dev, dim3(unsigned(4 * device_sm_count())), dim3(256), 0, st, stream,
+                                           stream_bytes, chunk_cap, static_cast<ChunkInfo *>(chunks), err, qb);
+    if (e != cudaSuccess) return e;
   }
   TraceScope ts("k_dtable", st);
-  k_dtable_dev<<<unsigned((kTabEntries + 255) / 256), 256, 0, st>>>(stream, stream_bytes, err, qb, tab);
-  return cudaGetLastError();
+  return launch_dependent(true, k_dtable_dev, dim3(unsigned((kTabEntries + 255) / 256)), dim3(256), 0, st, stream, stream_bytes,
+                          err, qb, tab);
 }
 
 cudaError_t launch_decode(const DecodeLaunch &a, cudaStream_t st) {

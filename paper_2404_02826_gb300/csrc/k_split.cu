@@ -284,6 +284,13 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
 // one warp, 5 bits at a time.
 __device__ __forceinline__ uint32_t select_warp(const uint32_t *list, uint32_t m, uint32_t rank, uint32_t b0, int bits,
                                                 uint32_t *h, int lane) {
+  if (m <= 32) {  // few: every lane counts the positions below its own
+    const uint32_t v = uint32_t(lane) < m ? list[lane] : 0xffffffffu;
+    uint32_t below = 0;
+    for (uint32_t i = 0; i < m; ++i) below += __shfl_sync(0xffffffffu, v, int(i)) < v;
+    const uint32_t hit = __ballot_sync(0xffffffffu, uint32_t(lane) < m && below == rank);
+    return __shfl_sync(0xffffffffu, v, hit ? __ffs(hit) - 1 : 0);
+  }
   uint32_t prefix = 0;
   for (int sh = (bits + 4) / 5 * 5 - 5; sh >= 0; sh -= 5) {
     h[lane] = 0;
@@ -807,6 +814,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     }
   }
   if (grid_sync(a, epoch)) return;
+  dep_launch();
   // first place of every child for every part: exclusive sums along the parts of a
   // subroot, in place, a warp per subroot and child
   const uint64_t msegs = uint64_t(gridDim.x) * kSplitParts + S;
@@ -852,10 +860,10 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
 constexpr int kMT = 512;
 constexpr int kMW = kMT / 32;
 
-template <bool IDX, int BITS>
+template <bool IDX, int BITS, int ROWS>
 struct MoveSmem {
   static constexpr uint32_t kCh = 1u << BITS;                   // children, at most
-  static constexpr int kRows = IDX || BITS > 7 ? 8 : 16;        // rows of 32 particles per warp and tile
+  static constexpr int kRows = ROWS;                            // rows of 32 particles per warp and tile
   static constexpr int kRankBits = kRows == 16 ? 9 : 8;         // a warp's particles of a tile
   static constexpr uint32_t kTile = uint32_t(kRows) * kMT;
   static constexpr uint32_t kStage = kTile + kCh * 14u;         // every child's run padded to whole groups of 8
@@ -878,10 +886,10 @@ __device__ __forceinline__ uint32_t stage_slot(uint32_t p) { return p ^ ((p >> 3
 // One tile, up to its particles in the stage by child.  WHOLE: the tile lies in
 // the segment.  A warp ranks rows of 32 consecutive particles: the lanes with
 // the same child, and the warp's count of that child so far from shared memory.
-template <bool IDX, int BITS, bool WHOLE>
-__device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX, BITS> &T, uint4 nodes, uint32_t t0, uint32_t b0,
+template <bool IDX, int BITS, int ROWS, bool WHOLE>
+__device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX, BITS, ROWS> &T, uint4 nodes, uint32_t t0, uint32_t b0,
                                           uint32_t b1, uint32_t NB, int lane, int warp) {
-  using V = MoveSmem<IDX, BITS>;
+  using V = MoveSmem<IDX, BITS, ROWS>;
   constexpr int kRows = V::kRows;
   const uint32_t ltm = (1u << lane) - 1u;
   const uint32_t w0 = t0 + uint32_t(warp) * (32 * kRows);  // the warp's first particle
@@ -1015,12 +1023,14 @@ __device__ __forceinline__ void move_tile(const SplitLaunch &a, MoveSmem<IDX, BI
 // every child's run starting at the same offset modulo 8 as its destination,
 // so that whole groups of 8 leave as 16-byte stores.  BITS: at least `levels`,
 // the bits of a child.
-template <bool IDX, int BITS>
+template <bool IDX, int BITS, int ROWS>
 __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLaunch a) {
   extern __shared__ __align__(128) unsigned char sm[];
-  using V = MoveSmem<IDX, BITS>;
+  using V = MoveSmem<IDX, BITS, ROWS>;
   V &T = *reinterpret_cast<V *>(sm);
   constexpr uint32_t kTile = V::kTile;
+  dep_launch();
+  dep_wait();
   if (call_failed(a.err)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t m = blockIdx.x, S = 1u << a.depth;
@@ -1064,8 +1074,8 @@ __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLa
     };
     load_nodes(b0 & ~31u);
     for (uint32_t t0 = b0 & ~31u; t0 < b1; t0 += kTile) {
-      if (t0 >= b0 && t0 + kTile <= b1) move_tile<IDX, BITS, true>(a, T, nodes, t0, b0, b1, NB, lane, warp);
-      else move_tile<IDX, BITS, false>(a, T, nodes, t0, b0, b1, NB, lane, warp);
+      if (t0 >= b0 && t0 + kTile <= b1) move_tile<IDX, BITS, ROWS, true>(a, T, nodes, t0, b0, b1, NB, lane, warp);
+      else move_tile<IDX, BITS, ROWS, false>(a, T, nodes, t0, b0, b1, NB, lane, warp);
       if (t0 + kTile < b1) load_nodes(t0 + kTile);
       const uint32_t ngroups = T.ngroups;
       for (uint32_t g = threadIdx.x; g < ngroups; g += kMT) {
@@ -1121,23 +1131,32 @@ __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLa
   }
 }
 
-template <bool IDX, int BITS>
+template <bool IDX, int BITS, int ROWS>
 cudaError_t move_launch(const SplitLaunch &a, cudaStream_t st) {
-  constexpr size_t smem = sizeof(MoveSmem<IDX, BITS>);
+  constexpr size_t smem = sizeof(MoveSmem<IDX, BITS, ROWS>);
   int per_sm = 0;
-  cudaError_t e = resident_blocks<k_move<IDX, BITS>>(kMT, smem, &per_sm);
+  cudaError_t e = resident_blocks<k_move<IDX, BITS, ROWS>>(kMT, smem, &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   TraceScope ts("k_move", st);
-  k_move<IDX, BITS><<<unsigned(a.grid) * kSplitParts, kMT, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(a.alone, k_move<IDX, BITS, ROWS>, dim3(unsigned(a.grid) * kSplitParts), dim3(kMT), smem, st, a);
+}
+// Tiles of 8192 particles (16 rows a warp) carry their fixed work over twice as many
+// (its barriers, scans and tables are half of the instructions with 8); of 4096 where a CTA holds no more, since then
+// every warp has rows, and with indices or 256 children, whose stages fill the SM.
+template <bool IDX, int BITS>
+cudaError_t move_rows(const SplitLaunch &a, cudaStream_t st) {
+  if constexpr (!IDX && BITS <= 7) {
+    if (a.part > 8u * kMT) return move_launch<IDX, BITS, 16>(a, st);
+  }
+  return move_launch<IDX, BITS, 8>(a, st);
 }
 template <bool IDX>
 cudaError_t move_dispatch(const SplitLaunch &a, cudaStream_t st) {
-  if (a.levels <= 4) return move_launch<IDX, 4>(a, st);
-  if (a.levels == 5) return move_launch<IDX, 5>(a, st);
-  if (a.levels == 6) return move_launch<IDX, 6>(a, st);
-  return a.levels == 7 ? move_launch<IDX, 7>(a, st) : move_launch<IDX, 8>(a, st);
+  if (a.levels <= 4) return move_rows<IDX, 4>(a, st);
+  if (a.levels == 5) return move_rows<IDX, 5>(a, st);
+  if (a.levels == 6) return move_rows<IDX, 6>(a, st);
+  return a.levels == 7 ? move_rows<IDX, 7>(a, st) : move_rows<IDX, 8>(a, st);
 }
 
 }  // namespace

@@ -742,6 +742,8 @@ __global__ void __launch_bounds__(kT, 1) k_subtree(const __grid_constant__ Subtr
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t ltm = (1u << lane) - 1u;
 
+  dep_launch();
+  dep_wait();
   // ---- the node: ticket order, so every node before it has started ----
   if (threadIdx.x == 0) {
     M.j = atomicAdd(a.ticket, 1u);
@@ -1487,8 +1489,7 @@ cudaError_t subtree_launch_as(const SubtreeLaunch &a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   TraceScope ts(COST ? "k_subtree_cost" : "k_subtree", st);
-  k_subtree<C, IDX, WIDEST, COST><<<unsigned(1ull << a.depth), kT, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(a.alone, k_subtree<C, IDX, WIDEST, COST>, dim3(unsigned(1ull << a.depth)), dim3(kT), smem, st, a);
 }
 template <typename C, bool IDX, bool WIDEST>
 cudaError_t subtree_launch(const SubtreeLaunch &a, cudaStream_t st) {

@@ -960,6 +960,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.parents = sl.depth > 0 ? nodes + ((1ull << (sl.depth - 1)) - 1) : nullptr;
       sl.out_nodes = nodes + ((1ull << (sl.depth + sl.levels - 1)) - 1);
       sl.clear = sl.levels < left;
+      sl.alone = share <= 1;
       sl.err = err;
       PC_TRY(launch_split(sl, st));
       if (facts)
@@ -1062,6 +1063,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sa.total_words = reinterpret_cast<uint64_t *>(ws + p.off_words);
       sa.payload_cap = payload_words(out_capacity, num_leaves);
       sa.err = err;
+      sa.alone = share <= 1;
       return sa;
     };
     // a4-a5: bit boxes, payload offsets, packing
