@@ -20,11 +20,12 @@
 //            smaller (key, index) meets its bit box (the box found blocking it
 //            in an earlier round is checked first).  Taken boxes are pairwise
 //            disjoint, so no particle lies in two of them.
-//   take     a block per taken box: ranks in its sequence for its centre, its
-//            other live particles in slot order, then, for every alive box c
-//            that is not taken and meets it, the live particles of c inside
-//            its bit box, by c and slot (counted first, then ranked); boxes
-//            that lost particles are listed.
+//   take     a cluster of blocks per taken box (a round takes a few boxes, so
+//            that what bounds it is the time of one): ranks in its sequence
+//            for its centre, its other live particles in slot order, then, for
+//            every alive box c that is not taken and meets it, the live
+//            particles of c inside its bit box, by c and slot (counted first,
+//            then ranked); boxes that lost particles are listed.
 //   scan     one block: each taken box's sequence index and first output
 //            position, in box order, after the sequences of earlier rounds.
 //   rebuild  a block per listed box: the bit box of what it keeps (the leaf
@@ -33,6 +34,8 @@
 // The host reads the alive count back every few rounds; rounds issued after
 // the last box died return at once.  A final pass moves codes and input
 // indices to their output positions for the packing kernels.
+#include <cooperative_groups.h>
+
 #include <climits>
 #include <cstdint>
 
@@ -346,6 +349,8 @@ __device__ __forceinline__ Box6 box6(const RBox &b) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_rd_select(State S) {
+  dep_launch();
+  dep_wait();
   if (S.ctr->alive == 0) return;
   const uint32_t a = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   if (a >= S.nl) return;
@@ -388,6 +393,7 @@ __global__ void __launch_bounds__(kThreads) k_rd_select(State S) {
 // ---- count and place ------------------------------------------------------
 
 constexpr int kTakeThreads = 1024;
+constexpr uint32_t kTakeCluster = 4;  // blocks per taken box
 constexpr int kTakeWarps = kTakeThreads / 32;
 static_assert(kTakeWarps >= 2 && kTakeWarps <= 32, "take: a search warp and an own-particle warp, one scan warp");
 
@@ -551,12 +557,18 @@ __device__ __forceinline__ uint32_t warp_pick_inside(const State &S, const C *q0
 // the taken box's own particles.
 __device__ __forceinline__ void search_sync(int nthreads) { asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory"); }
 
-// A block per taken box: the ranks of its sequence, its length into seq_cnt.
-// The last warp ranks the box's own particles while the others search the
-// tree breadth first (one level per step, all nodes of a level at once; a
-// level of more than kListCap boxes falls back to a depth-first search in
-// batches by warp 0).  Then every warp counts, and after a scan ranks, pieces
-// of the boxes met.
+// A cluster of blocks per taken box: the ranks of its sequence, its length into
+// seq_cnt.  The last warp of every block ranks its share of the box's own
+// particles while the others search the tree breadth first (one level per
+// step, all nodes of a level at once; a level of more than kListCap boxes falls
+// back to a depth-first search in batches by warp 0), every block for itself.
+// Then every warp of the cluster counts, and after a scan (the blocks' sums
+// through distributed shared memory) ranks, pieces of the boxes met.
+//
+// Bound by latency: a round has few boxes for 152 SMs, and each is a chain of
+// dependent steps on one box's data.  2^21 clustered particles, 64 rounds, a
+// launch with 1, 2, 4, 8 blocks per box: 27.3, 20.5, 17.5, 17.5 us; four leave
+// twice as many clusters as eight for rounds of many boxes.
 template <typename C>
 __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__restrict__ q0,
                                                           const C *__restrict__ q1, const C *__restrict__ q2) {
@@ -564,11 +576,19 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
   __shared__ uint32_t fr[2][kListCap];  // search frontiers; the boxes met end in one of them
   __shared__ uint32_t fmask[kListCap];
   __shared__ uint32_t lpos[kListCap];
-  __shared__ uint32_t s_nf, s_over, s_cur, s_n, s_done, s_sum;
+  __shared__ uint32_t s_nf, s_over, s_cur, s_n, s_done;
+  __shared__ uint32_t s_sum[2][kTakeCluster], s_own[kTakeCluster];  // by block of the cluster
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();  // every block of the cluster runs before one writes to another's shared memory
+  dep_launch();
+  dep_wait();
   if (S.ctr->alive == 0) return;
+  const uint32_t rank = cluster.block_rank();
   const uint32_t ntaken = S.ctr->taken;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t i = blockIdx.x; i < ntaken; i += gridDim.x) {
+  uint32_t turn = 0;  // which of the sums is in use
+  for (uint32_t i = blockIdx.x / kTakeCluster; i < ntaken; i += gridDim.x / kTakeCluster) {
     const uint32_t a = S.taken[i];
     const RBox A = S.t.box[a];
     const Box6 bx = box6(A);
@@ -577,17 +597,16 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
     auto bok = [&](uint32_t, const int4 &p, const int4 &q) {
       return (uint32_t(q.w) & (kAlive | kTaken)) == kAlive && meets(bx, p, q);
     };
-    if (warp == kTakeWarps - 1) {  // the centre, then the box's other live particles in slot order
+    // this block's share of the box's own slots, whole groups of four
+    const uint32_t og = IA.off >> 2, on = ((IA.off + IA.cnt + 3) >> 2) - og;
+    const uint32_t o0 = max(IA.off, 4 * (og + on * rank / kTakeCluster));
+    const uint32_t o1 = max(o0, min(IA.off + IA.cnt, 4 * (og + on * (rank + 1) / kTakeCluster)));
+    Picks own;
+    if (warp == kTakeWarps - 1) {  // the box's live particles but the centre, in slot order
       const uint32_t centre = IA.centre;
-      Picks rec;
-      warp_pick<C, false>(S, q0, q1, q2, IA.off, IA.off + IA.cnt,
-                          [=](uint32_t s, uint32_t, uint32_t, uint32_t) { return s != centre; }, rec);
-      warp_place(S, a, IA.off, IA.off + IA.cnt, 1, rec, kPickUnroll<C>);
-      if (lane == 0) {
-        atomicAnd(S.live + (centre >> 5), ~(1u << (centre & 31)));
-        S.dest[centre] = a;
-        S.rank[centre] = 0;
-      }
+      const uint32_t k = warp_pick<C, false>(S, q0, q1, q2, o0, o1,
+                                             [=](uint32_t s, uint32_t, uint32_t, uint32_t) { return s != centre; }, own);
+      if (uint32_t(lane) < kTakeCluster) *cluster.map_shared_rank(&s_own[rank], lane) = k;
     } else {
       const Tree &t = S.t;
       int cur = 0;
@@ -635,15 +654,26 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
       }
       if (threadIdx.x == 0) s_cur = uint32_t(cur);
     }
-    __syncthreads();
+    cluster.sync();
+    if (warp == kTakeWarps - 1) {
+      uint32_t p = 1;
+      for (uint32_t b = 0; b < rank; ++b) p += s_own[b];
+      warp_place(S, a, o0, o1, p, own, kPickUnroll<C>);
+      if (rank == 0 && lane == 0) {
+        atomicAnd(S.live + (IA.centre >> 5), ~(1u << (IA.centre & 31)));
+        S.dest[IA.centre] = a;
+        S.rank[IA.centre] = 0;
+      }
+    }
     uint32_t pos = IA.live;
     // counts, then ranks, of `parts` pieces of each of the nlist boxes in list,
     // at most one piece per warp at a time (its picks stay in the warp's registers)
     auto batch = [&](const uint32_t *list, uint32_t nlist) {
-      const uint32_t parts = nlist ? max(1u, min(16u, uint32_t(kTakeWarps) / nlist)) : 1u;
+      constexpr uint32_t kAll = kTakeCluster * uint32_t(kTakeWarps);
+      const uint32_t parts = nlist ? max(1u, min(16u, kAll / nlist)) : 1u;
       const uint32_t items = nlist * parts;
-      for (uint32_t i0 = 0; i0 < items; i0 += kTakeWarps) {
-        const uint32_t it = i0 + uint32_t(warp);
+      for (uint32_t i0 = 0; i0 < items; i0 += kAll) {
+        const uint32_t it = i0 + rank * uint32_t(kTakeWarps) + uint32_t(warp);
         uint32_t c = 0, off = 0, end = 0, k = 0;
         Picks rec;
         if (it < items) {
@@ -662,18 +692,25 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
             if (lane >= o) incl += y;
           }
           lpos[lane] = incl - x;
-          if (lane == 31) s_sum = incl;
+          const uint32_t sum = __shfl_sync(0xffffffffu, incl, 31);
+          if (uint32_t(lane) < kTakeCluster) *cluster.map_shared_rank(&s_sum[turn][rank], lane) = sum;
         }
-        __syncthreads();
+        cluster.sync();
+        uint32_t before = 0, total = 0;
+        for (uint32_t b = 0; b < kTakeCluster; ++b) {
+          before += b < rank ? s_sum[turn][b] : 0u;
+          total += s_sum[turn][b];
+        }
+        turn ^= 1u;  // the other sums are written next; these again only after one more barrier
         if (k) {
-          warp_place(S, a, off, end, pos + lpos[warp], rec, kPickUnroll<C>);
+          warp_place(S, a, off, end, pos + before + lpos[warp], rec, kPickUnroll<C>);
           if (lane == 0 && atomicExch(&S.info[c].lost, 1u) == 0u) {
             S.lost[atomicAdd(&S.ctr->nlost, 1u)] = c;
             mark_dirty(S.t, c);
           }
         }
-        pos += s_sum;
-        __syncthreads();  // lpos and s_sum are reused
+        pos += total;
+        __syncthreads();  // lpos is reused
       }
     };
     if (!s_over) {
@@ -702,8 +739,8 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
         if (done) break;
       }
     }
-    if (threadIdx.x == 0) S.seq_cnt[a] = pos;
-    __syncthreads();
+    if (rank == 0 && threadIdx.x == 0) S.seq_cnt[a] = pos;
+    cluster.sync();  // s_own and the frontiers are reused
   }
 }
 
@@ -713,6 +750,8 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
 // block over the bitmap of taken boxes, which it clears for the next round.
 __global__ void __launch_bounds__(1024) k_rd_scan(State S, LeafRec *seqs) {
   __shared__ uint32_t ws[32], wc[32];
+  dep_launch();
+  dep_wait();
   if (S.ctr->alive == 0) return;
   const uint32_t filled = S.ctr->filled, nseq = S.ctr->nseq;
   const uint32_t nw = (S.nl + 31) / 32;
@@ -789,7 +828,7 @@ __global__ void __launch_bounds__(1024) k_rd_scan(State S, LeafRec *seqs) {
 
 // ---- rebuild --------------------------------------------------------------
 
-constexpr int kBoxThreads = 128;
+constexpr int kBoxThreads = 256;  // a launch of 2^21 particles' rounds with 128, 256, 512: 12.8, 11.7, 12.1 us
 constexpr int kBoxWarps = kBoxThreads / 32;
 
 // The block's threads visit the live slots of [off, end) (every slot when
@@ -837,6 +876,10 @@ __global__ void __launch_bounds__(kBoxThreads) k_rd_rebuild(State S, const C *__
   __shared__ uint32_t red[7][kBoxWarps];
   __shared__ unsigned long long rd[kBoxWarps];
   __shared__ uint32_t rp[kBoxWarps];
+  if (!INIT) {
+    dep_launch();
+    dep_wait();
+  }
   if (INIT) {
     if (blockIdx.x == 0 && threadIdx.x == 0) S.ctr->alive = S.nl;  // the rest starts zeroed
   } else if (S.ctr->alive == 0) {
@@ -1065,7 +1108,8 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
 
   const uint32_t sms = uint32_t(device_sm_count());
   const unsigned box_blocks = unsigned(a.num_leaves < 16ull * sms ? a.num_leaves : 16ull * sms);
-  const unsigned take_blocks = unsigned(a.num_leaves < 2ull * sms ? a.num_leaves : 2ull * sms);
+  const uint64_t most_clusters = 2ull * sms / kTakeCluster;  // one wave
+  const unsigned take_blocks = unsigned(a.num_leaves < most_clusters ? a.num_leaves : most_clusters) * kTakeCluster;
   const unsigned refit_blocks = unsigned((uint64_t(L.count[1]) + kWarps - 1) / kWarps);
   const unsigned select_blocks = unsigned((a.num_leaves + kWarps - 1) / kWarps);
   {
@@ -1076,24 +1120,43 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
     TraceScope ts("k_rd_refit", st);
     k_rd_refit<<<refit_blocks, kThreads, 0, st>>>(S);
   }
-  // kRoundsPerCheck rounds: the same launches with the same arguments every time
+  // kRoundsPerCheck rounds: the same launches with the same arguments every time, each the
+  // programmatic dependent of the one before it where the call is alone
+  cudaError_t le = cudaSuccess;
   auto issue_rounds = [&](cudaStream_t s) {
+    auto ok = [&](cudaError_t r) {
+      if (le == cudaSuccess) le = r;
+    };
     for (int k = 0; k < kRoundsPerCheck; ++k) {
       {
         TraceScope ts("k_rd_select", s);
-        k_rd_select<<<select_blocks, kThreads, 0, s>>>(S);
+        ok(launch_dependent(a.alone, k_rd_select, dim3(select_blocks), dim3(kThreads), 0, s, S));
       }
       {
         TraceScope ts("k_rd_take", s);
-        k_rd_take<C><<<take_blocks, kTakeThreads, 0, s>>>(S, q0, q1, q2);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(take_blocks);
+        cfg.blockDim = dim3(kTakeThreads);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kTakeCluster;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = a.alone ? 2 : 1;
+        ok(cudaLaunchKernelEx(&cfg, k_rd_take<C>, S, q0, q1, q2));
       }
       {
         TraceScope ts("k_rd_scan", s);
-        k_rd_scan<<<1, 1024, 0, s>>>(S, a.seqs);
+        ok(launch_dependent(a.alone, k_rd_scan, dim3(1), dim3(1024), 0, s, S, a.seqs));
       }
       {
         TraceScope ts("k_rd_rebuild", s);
-        k_rd_rebuild<C, false><<<box_blocks, kBoxThreads, 0, s>>>(S, q0, q1, q2, a.leafs);
+        ok(launch_dependent(a.alone, k_rd_rebuild<C, false>, dim3(box_blocks), dim3(kBoxThreads), 0, s, S, q0, q1, q2,
+                            a.leafs));
       }
     }
   };
@@ -1105,6 +1168,11 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
   // they for a caller that may not allocate (no graph is instantiated).
   RoundGraph graph;
   if (!trace_enabled() && !no_host_alloc()) graph.capture(issue_rounds);
+  if (le != cudaSuccess) {  // a launch missing from the graph: they are issued one by one
+    if (graph.exec) cudaGraphExecDestroy(graph.exec);
+    graph.exec = nullptr;
+    le = cudaSuccess;
+  }
   uint64_t issued = 0;
   for (;;) {
     if (graph.exec) {
@@ -1112,6 +1180,7 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
       if (e != cudaSuccess) return e;
     } else {
       issue_rounds(st);
+      if (le != cudaSuccess) return le;
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

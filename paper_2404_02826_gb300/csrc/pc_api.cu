@@ -1022,6 +1022,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       rl.seqs = reinterpret_cast<LeafRec *>(ws + p.off_seqrec);
       rl.scratch = ws + p.off_reduce;
       rl.err = err;
+      rl.alone = share <= 1;
       uint64_t num_seq = 0, rounds = 0;
       PC_TRY(launch_reduce(rl, st, &num_seq, &rounds));
       hl.num_leaves = num_seq;

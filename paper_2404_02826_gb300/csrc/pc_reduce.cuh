@@ -21,6 +21,7 @@ struct ReduceLaunch {
   LeafRec *seqs;            // [num_leaves] the sequences: off, cnt, centre = 0, m, q_ref, words
   void *scratch;            // reduce_scratch_bytes(n, num_leaves), 256-byte aligned
   uint32_t *err;
+  bool alone;               // no other call shares the GPU: the rounds' kernels are programmatic dependents
 };
 uint64_t reduce_scratch_bytes(uint64_t n, uint64_t num_leaves);
 // Runs the rounds (reading a counter back every few rounds); on success
