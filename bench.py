@@ -225,6 +225,10 @@ def algorithmic_bytes(kernel, n, esz, cb, stream_bytes, with_idx=False, launches
         "k_median": cb * n,
         "k_count": cb * n,
         "k_scatter": 2 * (3 * cb + idx) * n,
+        # up to eight levels in two launches: the planes (every code read once, a byte per particle
+        # written), then the one move of every particle to its node
+        "k_split": 3 * cb * n + n,
+        "k_move": 2 * (3 * cb + idx) * n + n,
         "k_leafbox": 3 * cb * n,
         "k_leafpack": 3 * cb * n + stream_bytes,
         "k_decode": stream_bytes + 3 * esz * n,

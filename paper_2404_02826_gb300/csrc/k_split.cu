@@ -37,11 +37,12 @@
 // pass A reads two code arrays and the node bytes and writes those, 6 bytes a
 // particle, in 115 us (7.0 TB/s, the copy rate of the memory and what L2
 // keeps); level 0 reads one array in 70 us, bound by the shared-memory atomics;
-// B 80 us where a level needs it.  A launch takes 1.25 ms; the move 0.61 ms
-// (13 bytes a particle, 2.9 TB/s), bound by its instructions (78 a row of 32
-// particles) and shared-memory passes (18 a row).  Twelve levels: 3.7 ms, against
-// 5.9 ms level by level (96 launches).  At 2^20 particles the seven levels take
-// 0.13 ms in two launches, against 0.28 ms in 42.
+// B 80 us where a level needs it.  A launch takes 1.25 to 1.35 ms from board to
+// board; the move 0.53 ms (13 bytes a particle, 3.3 TB/s), bound by its
+// instructions (77 a row of 32 particles) and shared-memory passes (18 a row).
+// Twelve levels: 3.6 to 3.8 ms, against 5.9 ms level by level (96 launches).  At
+// 2^20 particles the seven levels take 0.11 ms in two launches, against 0.28 ms
+// in 42.
 #include <cstddef>
 #include <cstdint>
 

@@ -898,9 +898,9 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     };
     // several levels per launch while every node is larger than a leaf and than what a
     // warp splits (k_split.cu; u16 codes, depth mod 3); the leaf-size search needs the
-    // arrangement of every candidate depth.  Two launches for up to seven levels against
+    // arrangement of every candidate depth.  Two launches for up to eight levels against
     // eight a level: faster at every size measured (one level of 10,007 particles 30 us
-    // against 39; seven of 2^20 130 us against 280; twelve of 2^27 3.7 ms against 5.9)
+    // against 39; seven of 2^20 110 us against 280; twelve of 2^27 3.6 ms against 5.9)
     int split_to = 0;
     if (cb == 2 && !p.widest && !t_drop_tile_copies) {
       const int most = p.tune && first_depth < global_levels ? first_depth : global_levels;
