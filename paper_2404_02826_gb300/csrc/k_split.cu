@@ -283,7 +283,9 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
 
 // The value of rank `rank` among list[0 .. m), positions in [b0, 2^bits + b0): by
 // one warp, 5 bits at a time.
-__device__ __forceinline__ uint32_t select_warp(const uint32_t *list, uint32_t m, uint32_t rank, uint32_t b0, int bits,
+// Not inlined: inside the kernel it lengthened the passes' loops (2^27 particles 6030 us a call
+// inlined, 5965 so; 2^20 167 and 166).
+__device__ __noinline__ uint32_t select_warp(const uint32_t *list, uint32_t m, uint32_t rank, uint32_t b0, int bits,
                                                 uint32_t *h, int lane) {
   if (m <= 32) {  // few: every lane counts the positions below its own
     const uint32_t v = uint32_t(lane) < m ? list[lane] : 0xffffffffu;
