@@ -616,15 +616,17 @@ __global__ void __launch_bounds__(kDecThreads) k_decode(DecodeLaunch a) {
     }
   }
   // with host_err: the last block to get here leaves the error word there (a block that
-  // returned early does not count, and the host then reads the word itself)
+  // returned early does not count, and the host then reads the word itself).  The host
+  // returns to its caller on that word, and the output may lie in memory that the host reads:
+  // the blocks' output precedes their counts on the device, and the last block's fence, of
+  // system scope and ahead of its store, puts all of it before the word for the host too.
   if (a.host_err) {
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
       if (atomicAdd(a.err + 1, 1u) == gridDim.x - 1) {
-        __threadfence();
-        *reinterpret_cast<volatile uint32_t *>(a.host_err) = *reinterpret_cast<volatile uint32_t *>(a.err);
         __threadfence_system();
+        *reinterpret_cast<volatile uint32_t *>(a.host_err) = *reinterpret_cast<volatile uint32_t *>(a.err);
       }
     }
   }
