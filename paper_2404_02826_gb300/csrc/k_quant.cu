@@ -148,11 +148,13 @@ __device__ __forceinline__ void range_final(const double *partial, RangeResult *
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) k_range_f32(const float *__restrict__ pos, uint64_t n,
                                                         double *partial, RangeResult *res, uint32_t *ticket,
-                                                        RangeResult *host_res, uint32_t *host_flag) {
+                                                        RangeResult *host_res, uint32_t *host_flag, uint4 *zero,
+                                                        uint64_t zero_n) {
   F32Acc acc;
   acc.init();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (uint64_t i = tid; i < zero_n; i += stride) zero[i] = make_uint4(0, 0, 0, 0);
   uint64_t done = 0;
   if (VEC) {
     const float4 *p4 = reinterpret_cast<const float4 *>(pos);
@@ -204,11 +206,13 @@ __global__ void __launch_bounds__(kThreads) k_range_f32(const float *__restrict_
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) k_range_f64(const double *__restrict__ pos, uint64_t n,
                                                         double *partial, RangeResult *res, uint32_t *ticket,
-                                                        RangeResult *host_res, uint32_t *host_flag) {
+                                                        RangeResult *host_res, uint32_t *host_flag, uint4 *zero,
+                                                        uint64_t zero_n) {
   F64Acc acc;
   acc.init();
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   const uint64_t tid = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (uint64_t i = tid; i < zero_n; i += stride) zero[i] = make_uint4(0, 0, 0, 0);
   uint64_t done = 0;
   if (VEC) {
     const ulonglong2 *p2 = reinterpret_cast<const ulonglong2 *>(pos);
@@ -485,7 +489,8 @@ cudaError_t quant_dispatch(const QuantLaunch &a, cudaStream_t st) {
 cudaError_t launch_range(const RangeLaunch &a, cudaStream_t st) {
   TraceScope ts("k_range", st);
   auto run = [&](auto kernel, auto p) {
-    kernel<<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial, a.result, a.ticket, a.host_result, a.host_flag);
+    kernel<<<a.blocks, kThreads, 0, st>>>(p, a.n, a.partial, a.result, a.ticket, a.host_result, a.host_flag,
+                                            a.zero, a.zero_n);
   };
   if (a.dtype == 0) {
     const float *p = static_cast<const float *>(a.pos);

@@ -14,7 +14,8 @@
 //   A     every particle takes its child of the level above (code against the
 //         split plane) and is counted in a shared histogram of its code on the
 //         level's axis, one run of bins per node; the bins of all nodes share
-//         16384 counters, so a bin spans 2^shift codes with the smallest shift
+//         16384 counters (fewer where a small input has no room for them), so
+//         a bin spans 2^shift codes with the smallest shift
 //         that fits the nodes' real code ranges (0 for most of them);
 //   sel1  every CTA scans the summed histogram: the bin of every node's median;
 //   B     only with shift > 0: the particles of those bins are counted per code
@@ -238,7 +239,7 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
         sum += c[i];
       }
       tot = __reduce_add_sync(0xffffffffu, sum);
-      if (tot <= kBins || sh >= 16) break;
+      if (tot <= x.a.bins || sh >= 16) break;
     }
     uint32_t ex = warp_excl(sum, x.lane);
 #pragma unroll
@@ -249,7 +250,7 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
     }
     if (x.lane == 0) {
       x.M.shift = sh;
-      x.M.nbins = min(tot, kBins);
+      x.M.nbins = min(tot, x.a.bins);
     }
   } else if (x.warp == 1) {
     const uint32_t half = (1u << l) >> 1;
@@ -587,8 +588,8 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     const uint32_t nodes = 1u << l, half = nodes >> 1;
     const uint16_t *const cur = a.src[(a.depth + l) % 3];
     const uint16_t *const prev = a.src[(a.depth + l + 2) % 3];
-    uint32_t *const hist = a.hist + uint64_t(l & 1) * S * kBins;
-    uint32_t *const low = a.low + uint64_t(l & 1) * S * kLow;
+    uint32_t *const hist = a.hist + uint64_t(l & 1) * S * a.bins;
+    uint32_t *const low = a.low + uint64_t(l & 1) * S * a.low_cap;
     // ---- A ----
     Step step;
     const Pass pa = {prev, cur, half};
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       }
       if (l == 0) run_a<true, false>(x, pa, step);
       else run_a<false, false>(x, pa, step);
-      uint32_t *const h = hist + uint64_t(s) * kBins;
+      uint32_t *const h = hist + uint64_t(s) * a.bins;
       uint32_t *const own = a.seghist + uint64_t(2 * s + (c != M.clo)) * kBins;
       for (uint32_t b = threadIdx.x; b < nbins; b += kT) {
         const uint32_t v = P.bins[b];
@@ -616,8 +617,8 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     }
     grid_arrive(a);
     if (l > 0) {  // the other histogram was read by every CTA before the last barrier
-      uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * kBins);
-      for (uint32_t i = gtid; i < S * (kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+      uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * a.bins);
+      for (uint32_t i = gtid; i < S * (a.bins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
     }
     if (grid_wait(a, epoch)) return;
     // ---- sel1 and B ----
@@ -628,7 +629,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       }
       const uint32_t nbins = M.nbins, shift = M.shift;
       {  // exclusive prefixes within each warp's 512 bins, and the warps' totals
-        const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + uint64_t(s) * kBins);
+        const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + uint64_t(s) * a.bins);
         constexpr uint32_t kPer = kBins / kW;
         uint4 v[kPer / 128];
 #pragma unroll
@@ -705,15 +706,15 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
         for (uint32_t i = threadIdx.x; i < nlow; i += kT) {
           const uint32_t v = P.sum[i];
           sl[i * segs] = v;
-          if (v) atomicAdd(low + uint64_t(s) * kLow + i, v);
+          if (v) atomicAdd(low + uint64_t(s) * a.low_cap + i, v);
         }
       }
       if (multi) keep_seg(x, s);
     }
     grid_arrive(a);
     if (l > 0) {  // read by every CTA before the barrier before
-      uint4 *z = reinterpret_cast<uint4 *>(a.low + uint64_t((l + 1) & 1) * S * kLow);
-      for (uint32_t i = gtid; i < S * (kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
+      uint4 *z = reinterpret_cast<uint4 *>(a.low + uint64_t((l + 1) & 1) * S * a.low_cap);
+      for (uint32_t i = gtid; i < S * (a.low_cap / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
     }
     if (!multi)
       for (uint32_t b = threadIdx.x; b < M.nbins; b += kT) P.bins[b] = 0;
@@ -731,7 +732,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
         const uint32_t target = (N.rcnt[j] >> 1) - N.below[j];
         uint32_t vlow = 0, less = 0;
         if (shift) {
-          const uint32_t *lw = low + uint64_t(s) * kLow + (j << shift);
+          const uint32_t *lw = low + uint64_t(s) * a.low_cap + (j << shift);
           uint32_t run = 0;
           for (uint32_t i0 = 0; i0 < (1u << shift); i0 += 32) {
             const uint32_t v = i0 + lane < (1u << shift) ? __ldcg(lw + i0 + lane) : 0u;
@@ -850,12 +851,8 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       }
     }
   }
-  if (a.clear) {  // another launch follows: the histograms are left zero
-    uint4 *z = reinterpret_cast<uint4 *>(a.hist);
-    for (uint64_t i = gtid; i < uint64_t(S) * (2 * kBins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
-    z = reinterpret_cast<uint4 *>(a.low);
-    for (uint64_t i = gtid; i < uint64_t(S) * (2 * kLow / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
-  }
+  uint4 *const z = reinterpret_cast<uint4 *>(a.hist);
+  for (uint64_t i = gtid; i < a.zero_next; i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
 }
 
 // ---- the move ----

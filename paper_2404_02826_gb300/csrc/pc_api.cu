@@ -196,6 +196,7 @@ struct Plan {
   uint64_t off_nodes = 0, off_leafrec = 0, off_words = 0;
   uint64_t off_zero = 0, zero_bytes = 0;  // zeroed at every call:
   uint64_t off_hist = 0, off_tiles = 0, off_tickets = 0, off_err = 0, off_total = 0;
+  uint64_t hist_bytes = 0;
   uint64_t off_status = 0;  // look-back words of the on-chip subtree kernel
   uint64_t off_groups = 0, off_slices = 0;
   uint64_t off_reduce = 0, off_seqrec = 0;  // bit-box reduction: its scratch and the sequence records
@@ -206,7 +207,6 @@ struct Plan {
   bool tune = false;  // leaf size chosen by descending from r_hi while the stream shrinks (sized for r)
   uint32_t r_hi = 0;
   int tune_first = 0, tune_last = 0;  // candidate depths
-  uint64_t off_split = 0;             // several levels per launch (k_split.cu): histograms and barriers (zeroed)
   uint64_t off_tunecost = 0;          // leaf-size search: payload words per in-CTA depth (zeroed)
   uint64_t total = 0;
   int range_blocks = 0;
@@ -281,29 +281,115 @@ uint32_t digit_bits_for(int level) {
 // Several levels per launch (k_split.cu).  A launch below depth 0 needs subroots
 // of at least kSplitMinRoot particles, so that their histograms stay small
 // beside the data, and its levels are limited by the codes' bits: level l's 2^l
-// nodes share kSplitBins = 2^14 bins, so a bin spans at most 2^(bits + l - 14)
-// codes, and the codes of the nodes' median bins need 2^l times as many of the
-// kSplitLow counters.  That holds for every data with 8 levels up to 13 bits, 7
-// up to 15, else 6.
-int split_max_levels(int bits) { return bits <= 13 ? 8 : (bits <= 15 ? 7 : 6); }
-uint32_t split_low_cap(int bits, int levels) {
-  const int shift = bits + levels - 1 - 14;
+// nodes share 2^b bins, so a bin spans at most 2^(bits + l - b) codes, and the
+// codes of the nodes' median bins need 2^l times as many of the kSplitLow
+// counters.  With all kSplitBins = 2^14 bins that holds for every data with 8
+// levels up to 13 bits, 7 up to 15, else 6.
+uint32_t split_low_cap(int bits, int levels, int b) {
+  const int shift = bits + levels - 1 - b;
   return (1u << (levels - 1)) << (shift > 0 ? shift : 0);
+}
+int split_max_levels(int bits, int b) {
+  int l = kSplitMaxLevels;
+  while (l > 1 && split_low_cap(bits, l, b) > kSplitLow) --l;
+  return l;
 }
 constexpr uint64_t kSplitMinRoot = 1u << 17;
 constexpr uint64_t kSplitMinChunk = 4096;  // particles of a CTA: fewer CTAs for small inputs
-constexpr int kSplitLaunches = 16;         // barrier words
+constexpr uint64_t kSplitOwnTies = 4 * kSplitBins;  // up to here a CTA's ties always fit its shared memory
+constexpr int kSplitLaunches = 16;         // one barrier word each
+constexpr uint64_t kBarrierAt = 128;       // their place after the error word, a cache line of its own
 
 bool split_roots_ok(uint64_t n, int depth) {
   return depth == 0 || ((1ull << depth) <= kSplitMaxRoots && (n >> depth) >= kSplitMinRoot);
 }
-uint64_t split_roots_max(uint64_t n) {
-  int d = 0;
-  while (split_roots_ok(n, d + 1)) ++d;
-  return 1ull << d;
+
+// CTAs of a launch: one per SM of the call's `cap`, fewer for small inputs.
+uint64_t split_grid(uint64_t n, uint64_t cap) {
+  const uint64_t g = std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap));
+  return n <= kSplitOwnTies ? std::max(g, (n + kSplitBins - 1) / kSplitBins) : g;
 }
-uint64_t split_zero_bytes(uint64_t n) {
-  return 4 * kSplitLaunches * 32 + split_roots_max(n) * 2 * 4 * uint64_t(kSplitBins + kSplitLow);
+
+// Scratch of a launch of `grid` CTAs, in the order in which it is laid out.
+struct SplitScratch {
+  uint64_t node, seglow, segcnt, ties, state, seghist, total;
+};
+SplitScratch split_scratch(uint64_t n, int depth, uint32_t low_cap, uint64_t grid) {
+  const uint64_t roots = 1ull << depth, segs = grid + roots;
+  SplitScratch s = {};
+  uint64_t o = 0;
+  auto take = [&](uint64_t bytes) {
+    const uint64_t at = o;
+    o = align_up(o + bytes);
+    return at;
+  };
+  s.node = take(n + 64);
+  s.seglow = take(segs * low_cap * 4);
+  s.segcnt = take((kSplitParts * grid + roots) * 4 << kSplitMaxLevels);
+  s.ties = take(n > kSplitOwnTies ? 4 * n : 0);
+  if (depth > 0) {
+    s.state = take(segs * kSplitStateWords * 4);
+    s.seghist = take(2 * roots * kSplitBins * 4);
+  }
+  s.total = o;
+  return s;
+}
+
+// Bytes of a launch's zeroed counters.
+uint64_t split_counters(int depth, uint32_t bins, uint32_t low_cap) {
+  return (2ull << depth) * 4 * (uint64_t(bins) + low_cap);
+}
+
+// The launches that take the levels 0 .. split_to - 1, as far as they go, and where their
+// zeroed counters lie.
+struct SplitPlan {
+  int count = 0, depth[kSplitLaunches], levels[kSplitLaunches];
+  uint32_t bins = 0, low_cap = 0;  // counters per subroot and parity
+  uint64_t room = 0;               // bytes of the launch with the most subroots
+  bool in_spare = false;           // ahead of the launches' scratch (zeroed by the range kernel for the
+                                   // first launch, by each launch for the next), else in the per-level
+                                   // path's histograms (zeroed with those and left zero)
+};
+
+// `spare_bytes`: what the u16 codes leave of the u32 codes' room; `hist_bytes`: the
+// per-level path's histograms.  The counters have no room of their own in the workspace:
+// one that holds the per-level path holds this one (so pc_compress_noalloc's fixed
+// scratch takes the same sizes with either), and what is zeroed is what the launches use,
+// 12.6 MB at 2^27 particles.  An input of some ten thousand particles has less spare room
+// than the 128 KB of one subroot; its counters lie in the histograms where those are as
+// large (four levels or more), else it has fewer bins.
+SplitPlan split_plan(uint64_t n, int split_to, int bits, bool alone, uint64_t sms, uint64_t spare_bytes,
+                     uint64_t hist_bytes) {
+  SplitPlan p;
+  const uint64_t grid = split_grid(n, sms);
+  for (int b = 14; b >= 10 && p.count == 0; b -= 2) {
+    // eight levels save a launch where a call is alone (3,000,017 particles: 343 us against
+    // 391 with four and four), but the move works less well with 256 children: a batch
+    // of 48 snapshots takes 5.17 ms with at most seven, 5.24 with eight
+    const int most = split_max_levels(bits, b), max_levels = alone ? most : std::min(most, 7);
+    // even shares of what is left, or as many as one launch takes where a second one's
+    // subroots would be too small
+    for (int at = 0; at < split_to && split_roots_ok(n, at) && p.count < kSplitLaunches;) {
+      const int left = split_to - at, parts = (left + max_levels - 1) / max_levels;
+      int levels = (left + parts - 1) / parts;
+      if (parts > 1 && !split_roots_ok(n, at + levels)) levels = max_levels;
+      p.depth[p.count] = at;
+      p.levels[p.count++] = levels;
+      at += levels;
+    }
+    p.bins = 1u << b;
+    for (; p.count > 0; --p.count) {  // the last launch has the most subroots: left out without room for it
+      p.low_cap = 4;
+      uint64_t scratch = 0;
+      for (int i = 0; i < p.count; ++i) p.low_cap = std::max(p.low_cap, split_low_cap(bits, p.levels[i], b));
+      for (int i = 0; i < p.count; ++i)
+        scratch = std::max(scratch, split_scratch(n, p.depth[i], p.low_cap, grid).total);
+      p.room = align_up(split_counters(p.depth[p.count - 1], p.bins, p.low_cap));
+      p.in_spare = p.room + scratch <= spare_bytes;
+      if (p.in_spare || (p.room <= hist_bytes && scratch <= spare_bytes)) break;
+    }
+  }
+  return p;
 }
 
 // Bytes of one axis's u16 code array (the same padding).
@@ -312,6 +398,9 @@ inline uint64_t code_stride16(uint64_t n) { return align_up(2 * n + 64); }
 // Bytes of one axis's code array: room for u32 codes and for the 16-byte
 // loads of a tile's last group, which may reach up to 64 bytes past n.
 inline uint64_t code_stride(uint64_t n) { return align_up(4 * n + 64); }
+
+// What the u16 codes of both arrangements leave of the room for u32 codes.
+inline uint64_t spare_room(uint64_t n) { return 6 * (code_stride(n) - code_stride16(n)); }
 
 // Tiles per node at one level: node sizes are floor(n / 2^level) or one more.
 uint64_t tiles_per_node(uint64_t n, int level, uint32_t tile) {
@@ -428,6 +517,7 @@ int make_plan(uint64_t n, int dtype, const pc_config *cfg, bool idx, int sm_coun
     tiles += (1ull << l) * tiles_per_node(n, l, min_scatter_tile(true));
   }
   p.off_hist = o;
+  p.hist_bytes = 4 * hist_bins;
   o = align_up(o + 4 * (hist_bins ? hist_bins : 1));
   p.off_tiles = o;
   o = align_up(o + 8 * (tiles ? tiles : 1));
@@ -435,12 +525,10 @@ int make_plan(uint64_t n, int dtype, const pc_config *cfg, bool idx, int sm_coun
   o = align_up(o + 4 * (p.levels + 3));
   p.off_tunecost = o;
   o = align_up(o + 8 * (kSubMaxLevels + 1));
-  p.off_split = o;
-  if (p.levels > 0) o = align_up(o + split_zero_bytes(n));
   p.off_status = o;
   o = align_up(o + 8 * subtree_status_entries(p.levels));
-  p.off_err = o;
-  o = align_up(o + 4);
+  p.off_err = o;  // the error word; from kBarrierAt on the barrier words of the launches of k_split.cu
+  o = align_up(o + kBarrierAt + 4 * kSplitLaunches);
   p.off_total = o;
   o = align_up(o + 8);
   p.zero_bytes = o - p.off_zero;
@@ -644,6 +732,10 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     ra.partial = reinterpret_cast<double *>(ws + p.off_partial);
     ra.result = reinterpret_cast<RangeResult *>(ws + p.off_range);
     ra.ticket = reinterpret_cast<uint32_t *>(ws + p.off_tickets) + p.levels + 2;
+    if (p.levels > 0 && !p.widest) {  // the counters of a first launch of several levels
+      ra.zero = reinterpret_cast<uint4 *>(ws + p.off_codes_a + 3 * code_stride16(n));
+      ra.zero_n = std::min<uint64_t>(split_counters(0, kSplitBins, kSplitLow), spare_room(n)) / 16;
+    }
     ra.blocks = int(std::min<uint64_t>(uint64_t(p.range_blocks), (n + 1023) / 1024));
     volatile uint32_t *const flag = reinterpret_cast<volatile uint32_t *>(hb.host + 128);
     if (hb.host) {
@@ -674,15 +766,14 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
                                                  : (L.qmax[1] > L.qmax[2] ? L.qmax[1] : L.qmax[2]);
     const int cb = (qmax < 65536u && !L.raw) ? 2 : 4;
     // u16 codes lie at the two ends of the room for u32 codes; what they leave
-    // between them is scratch of the levels
+    // between them is scratch of the levels (`spare`)
     void *codes_a[3], *codes_b[3];
     const uint64_t cstride = cb == 2 ? code_stride16(n) : code_stride(n);
     for (int d = 0; d < 3; ++d) {
       codes_a[d] = ws + p.off_codes_a + uint64_t(d) * cstride;
       codes_b[d] = ws + p.off_codes_b + 3 * code_stride(n) - uint64_t(3 - d) * cstride;
     }
-    uint8_t *const spare = ws + p.off_codes_a + 3 * cstride;
-    const uint64_t spare_bytes = (p.off_codes_b + 3 * code_stride(n) - 3 * cstride) - (p.off_codes_a + 3 * cstride);
+    uint8_t *const spare = ws + p.off_codes_a + 3 * code_stride16(n);
     uint32_t *idx_a = use_idx ? reinterpret_cast<uint32_t *>(ws + p.off_idx_a) : nullptr;
     uint32_t *idx_b = use_idx ? reinterpret_cast<uint32_t *>(ws + p.off_idx_b) : nullptr;
 
@@ -728,6 +819,20 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
                                ? tune_subtree_depth(n, p.tune_first, p.tune_last, cb, use_idx)
                                : -1;
     const int global_levels = sub_depth >= 0 ? sub_depth : (tune_depth >= 0 ? tune_depth : levels);
+    // several levels per launch while every node is larger than a leaf and than what a
+    // warp splits (k_split.cu; u16 codes, depth mod 3); the leaf-size search needs the
+    // arrangement of every candidate depth.  Two launches for up to eight levels against
+    // eight a level: faster at every size measured (one level of 10,007 particles 30 us
+    // against 39; seven of 2^20 110 us against 280; twelve of 2^27 3.6 ms against 5.9)
+    int split_to = 0;
+    if (cb == 2 && !p.widest && !t_drop_tile_copies) {
+      const int most = p.tune && p.tune_first < global_levels ? p.tune_first : global_levels;
+      while (split_to < most && (n >> split_to) > p.r &&
+             ((n + (1ull << split_to) - 1) >> split_to) > p.warp_node_max)
+        ++split_to;
+    }
+    const SplitPlan sp = split_plan(n, split_to, int(bit_length(qmax)), share <= 1, uint64_t(device_sm_count()),
+                                    spare_room(n), p.hist_bytes);
     // a4-a5 on the arrangement at depth `depth` (leaves = its 2^depth nodes when split_level = depth - 1)
     auto leaf_launch = [&](void *const *codes, const uint32_t *idxs, int split_level, uint32_t r,
                            uint64_t num_leaves, bool cost_only, bool box_only = false) {
@@ -896,60 +1001,33 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       if (l > first_depth && bytes >= best_bytes) chosen = l - 1;
       else best_bytes = bytes;
     };
-    // several levels per launch while every node is larger than a leaf and than what a
-    // warp splits (k_split.cu; u16 codes, depth mod 3); the leaf-size search needs the
-    // arrangement of every candidate depth.  Two launches for up to eight levels against
-    // eight a level: faster at every size measured (one level of 10,007 particles 30 us
-    // against 39; seven of 2^20 110 us against 280; twelve of 2^27 3.6 ms against 5.9)
-    int split_to = 0;
-    if (cb == 2 && !p.widest && !t_drop_tile_copies) {
-      const int most = p.tune && first_depth < global_levels ? first_depth : global_levels;
-      while (split_to < most && (n >> split_to) > p.r &&
-             ((n + (1ull << split_to) - 1) >> split_to) > p.warp_node_max)
-        ++split_to;
-    }
-    for (int launches = 0; src_depth < split_to && split_roots_ok(n, src_depth) && launches < kSplitLaunches;
-         ++launches) {
-      // even shares of what is left, or as many as one launch takes where a second one's
-      // subroots would be too small
-      // eight levels save a launch where a call is alone (3,000,017 particles: 343 us against
-      // 391 with four and four), but the move works less well with 256 children: a batch
-      // of 48 snapshots takes 5.17 ms with at most seven, 5.24 with eight
-      const int most_levels = split_max_levels(int(bit_length(qmax))), left = split_to - src_depth;
-      const int max_levels = share > 1 ? std::min(most_levels, 7) : most_levels;
-      const int parts = (left + max_levels - 1) / max_levels;
+    for (int k = 0; k < sp.count; ++k) {
       SplitLaunch sl = {};
       sl.n = n;
-      sl.depth = src_depth;
-      sl.levels = (left + parts - 1) / parts;
-      if (parts > 1 && !split_roots_ok(n, src_depth + sl.levels)) sl.levels = max_levels;
-      // a CTA per SM, fewer for small inputs, and this call's share of them when others run
-      // beside it: 48 snapshots of 10^4 to 10^7 particles on 8 lanes took 8.3 ms when every
-      // launch asked for all SMs, 5.8 with its share
+      sl.depth = sp.depth[k];
+      sl.levels = sp.levels[k];
+      // this call's share of the SMs when others run beside it: 48 snapshots of 10^4 to 10^7
+      // particles on 8 lanes took 8.3 ms when every launch asked for all SMs, 5.8 with its share
       const uint64_t sms = uint64_t(device_sm_count());
       const uint64_t cap = share > 1 ? std::max<uint64_t>(1, sms / uint64_t(share)) : sms;
-      sl.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap)));
+      sl.grid = int(split_grid(n, cap));
       sl.chunk = uint32_t(((n + sl.grid - 1) / sl.grid + 15) & ~15ull);
-      const uint64_t roots = 1ull << sl.depth, segs = uint64_t(sl.grid) + roots;
-      uint64_t used = 0;
-      auto take = [&](uint64_t bytes) {
-        uint8_t *q = spare + used;
-        used += align_up(bytes);
-        return reinterpret_cast<uint32_t *>(q);
-      };
-      sl.node = reinterpret_cast<uint8_t *>(take(n + 64));
-      sl.low_cap = split_low_cap(int(bit_length(qmax)), sl.levels);
-      sl.seglow = take(segs * sl.low_cap * 4);
-      sl.segcnt = take((kSplitParts * uint64_t(sl.grid) + roots) * 4 << kSplitMaxLevels);
-      sl.ties = take(4 * n);
+      uint8_t *const counters = sp.in_spare ? spare : ws + p.off_hist;
+      uint8_t *const scratch = spare + (sp.in_spare ? sp.room : 0);
+      const SplitScratch at = split_scratch(n, sl.depth, sp.low_cap, uint64_t(sl.grid));
+      sl.node = scratch + at.node;
+      sl.bins = sp.bins;
+      sl.low_cap = sp.low_cap;
+      sl.seglow = reinterpret_cast<uint32_t *>(scratch + at.seglow);
+      sl.segcnt = reinterpret_cast<uint32_t *>(scratch + at.segcnt);
+      sl.ties = n > kSplitOwnTies ? reinterpret_cast<uint32_t *>(scratch + at.ties) : nullptr;
       if (sl.depth > 0) {
-        sl.state = take(segs * kSplitStateWords * 4);
-        sl.seghist = take(2 * roots * kSplitBins * 4);
+        sl.state = reinterpret_cast<uint32_t *>(scratch + at.state);
+        sl.seghist = reinterpret_cast<uint32_t *>(scratch + at.seghist);
       }
-      if (used > spare_bytes) break;
-      sl.barrier = reinterpret_cast<uint32_t *>(ws + p.off_split) + 32 * launches;
-      sl.hist = reinterpret_cast<uint32_t *>(ws + p.off_split) + 32 * kSplitLaunches;
-      sl.low = sl.hist + split_roots_max(n) * 2 * kSplitBins;
+      sl.barrier = reinterpret_cast<uint32_t *>(ws + p.off_err + kBarrierAt) + k;
+      sl.hist = reinterpret_cast<uint32_t *>(counters);
+      sl.low = sl.hist + (2ull << sl.depth) * sp.bins;
       for (int d = 0; d < 3; ++d) {
         sl.root_hi[d] = L.qmax[d];
         sl.src[d] = static_cast<const uint16_t *>(src[d]);
@@ -959,7 +1037,8 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.dst_idx = idst;
       sl.parents = sl.depth > 0 ? nodes + ((1ull << (sl.depth - 1)) - 1) : nullptr;
       sl.out_nodes = nodes + ((1ull << (sl.depth + sl.levels - 1)) - 1);
-      sl.clear = sl.levels < left;
+      if (k + 1 < sp.count) sl.zero_next = split_counters(sp.depth[k + 1], sp.bins, sp.low_cap) / 16;
+      else if (!sp.in_spare) sl.zero_next = split_counters(sl.depth, sp.bins, sp.low_cap) / 16;
       sl.alone = share <= 1;
       sl.err = err;
       PC_TRY(launch_split(sl, st));

@@ -144,6 +144,8 @@ struct RangeLaunch {
   double *partial;  // [blocks][7]
   RangeResult *result;
   uint32_t *ticket;       // zero on entry
+  uint4 *zero;            // zeroed by the way: zero_n 16-byte words
+  uint64_t zero_n;
   RangeResult *host_result;  // optional, page-locked host memory: the result once more, then
   uint32_t *host_flag;       // a 1 here
   int blocks;
@@ -201,7 +203,7 @@ cudaError_t launch_scatter(const LevelLaunch &a, cudaStream_t st);
 // Several levels in one cooperative launch (k_split.cu): 16-bit codes, split
 // axis depth mod 3, every node above depth + levels larger than a leaf.
 constexpr int kSplitMaxLevels = 8;         // a particle's node below its subroot fits a byte
-constexpr uint32_t kSplitBins = 16384;     // counters of one level's histogram, shared by its nodes
+constexpr uint32_t kSplitBins = 16384;     // counters of one level's histogram, shared by its nodes, at most
 constexpr uint32_t kSplitLow = 8192;       // counters of the codes in the nodes' median bins, at most
 constexpr uint32_t kSplitStateWords = 17u << (kSplitMaxLevels - 1);
 constexpr int kSplitParts = 2;             // parts of a CTA's positions, one per CTA of the move
@@ -219,17 +221,18 @@ struct SplitLaunch {
   const uint32_t *src_idx;    // optional
   uint32_t *dst_idx;
   uint8_t *node;              // [n + 64] scratch: node below the subroot
-  uint32_t *hist;             // [2][2^depth][kSplitBins], zero on entry
-  uint32_t *low;              // [2][2^depth][kSplitLow], zero on entry
+  uint32_t *hist;             // [2][2^depth][bins], zero on entry
+  uint32_t *low;              // [2][2^depth][low_cap], zero on entry
   uint32_t part;              // positions per CTA of the move (set by launch_split)
   // scratch; a segment is what a CTA holds of a subroot (at most grid + 2^depth of them)
   uint32_t *seglow;           // [low_cap][grid + 2^depth] codes in the median bins, by segment
-  uint32_t low_cap;           // at least 2^l << shift of every level l, whatever the codes
+  uint32_t bins;              // counters of a level's histogram: a power of two, at most kSplitBins
+  uint32_t low_cap;           // at least 2^l << shift of every level l, whatever the codes; a multiple of 4
   uint32_t *segcnt;           // [2^kSplitMaxLevels][kSplitParts grid + 2^depth] children, by part of a segment
-  uint32_t *ties;             // [n] positions of ties
+  uint32_t *ties;             // [n] positions of ties (null with chunks of at most kSplitBins)
   uint32_t *state;            // [grid + 2^depth][kSplitStateWords] (depth > 0)
   uint32_t *seghist;          // [2^(depth + 1)][kSplitBins] (depth > 0)
-  bool clear;                 // leave hist and low zero (another launch uses them)
+  uint64_t zero_next;         // 16-byte words left zero from hist on: what the next launch counts in
   bool alone;                 // no other call shares the GPU
   uint32_t *barrier;          // zero on entry
   uint32_t *err;
