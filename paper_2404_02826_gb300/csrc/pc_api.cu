@@ -1,12 +1,14 @@
 // C ABI (include/pc.h): argument checks, the error-bound arithmetic of Sec. 3
 // on the host, workspace layout, and the launch sequence of the hot path.
 #include <algorithm>
+#include <atomic>
 #include <cfloat>
 #include <chrono>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <optional>
 #include <vector>
 
 #include "../../include/pc.h"
@@ -308,6 +310,33 @@ bool split_roots_ok(uint64_t n, int depth) {
 uint64_t split_grid(uint64_t n, uint64_t cap) {
   const uint64_t g = std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap));
   return n <= kSplitOwnTies ? std::max(g, (n + kSplitBins - 1) / kSplitBins) : g;
+}
+
+// Compressions in flight, by device.
+struct Load {
+  std::atomic<uint32_t> calls{0};
+  std::atomic<uint64_t> particles{0};
+};
+Load g_load[64];
+
+Load &load_of(int dev) { return g_load[dev & 63]; }
+Load &in_flight() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return load_of(dev);
+}
+
+// SMs of a call of n particles for a launch whose CTAs must all be placed at once: its part
+// of the particles in flight, and one left to every other call; all of them when it is
+// alone.  By work, not by calls: one snapshot of 2^26 particles among fifteen of 10^4 on
+// eight lanes takes 3.42 ms (2.95 alone; 11.5 with an eighth of the SMs), and 24 of 10^6 in
+// plain calls from eight host threads 2.2 ms (3.8 when each asks for all SMs).
+uint64_t sm_share(uint64_t n, uint64_t sms) {
+  const Load &load = in_flight();
+  const uint64_t calls = load.calls, particles = std::max<uint64_t>(load.particles, n);
+  if (calls <= 1) return sms;
+  const uint64_t left = sms > calls - 1 ? sms - (calls - 1) : 1;
+  return std::max<uint64_t>(1, std::min(left, sms * n / particles));
 }
 
 // Scratch of a launch of `grid` CTAs, in the order in which it is laid out.
@@ -682,7 +711,7 @@ struct RunFacts {
 
 int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                   void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                  uint32_t *perm, cudaStream_t st, int share = 1, Sweep *sweep = nullptr,
+                  uint32_t *perm, cudaStream_t st, bool counted = false, Sweep *sweep = nullptr,
                   RunFacts *facts = nullptr) {
   if (sweep) {
     if (!cfg || !(cfg->flags & PC_FLAG_AUTOTUNE_LEAF) || perm) return PC_ERR_ARG;
@@ -705,6 +734,8 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
   uint8_t *ws = static_cast<uint8_t *>(workspace);
   uint32_t *err = reinterpret_cast<uint32_t *>(ws + p.off_err);
   uint64_t *total_dev = reinterpret_cast<uint64_t *>(ws + p.off_total);
+  std::optional<InFlight> flight;
+  if (!counted) flight.emplace(n);
   HostBlock hb;  // the value range, then the call's end
   PC_TRY(cudaMemsetAsync(ws + p.off_zero, 0, p.zero_bytes, st));
 
@@ -831,8 +862,9 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
              ((n + (1ull << split_to) - 1) >> split_to) > p.warp_node_max)
         ++split_to;
     }
-    const SplitPlan sp = split_plan(n, split_to, int(bit_length(qmax)), share <= 1, uint64_t(device_sm_count()),
-                                    spare_room(n), p.hist_bytes);
+    const bool alone = in_flight().calls <= 1;
+    const SplitPlan sp =
+        split_plan(n, split_to, int(bit_length(qmax)), alone, uint64_t(device_sm_count()), spare_room(n), p.hist_bytes);
     // a4-a5 on the arrangement at depth `depth` (leaves = its 2^depth nodes when split_level = depth - 1)
     auto leaf_launch = [&](void *const *codes, const uint32_t *idxs, int split_level, uint32_t r,
                            uint64_t num_leaves, bool cost_only, bool box_only = false) {
@@ -1006,11 +1038,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.n = n;
       sl.depth = sp.depth[k];
       sl.levels = sp.levels[k];
-      // this call's share of the SMs when others run beside it: 48 snapshots of 10^4 to 10^7
-      // particles on 8 lanes took 8.3 ms when every launch asked for all SMs, 5.8 with its share
-      const uint64_t sms = uint64_t(device_sm_count());
-      const uint64_t cap = share > 1 ? std::max<uint64_t>(1, sms / uint64_t(share)) : sms;
-      sl.grid = int(split_grid(n, cap));
+      sl.grid = int(split_grid(n, sm_share(n, uint64_t(device_sm_count()))));
       sl.chunk = uint32_t(((n + sl.grid - 1) / sl.grid + 15) & ~15ull);
       uint8_t *const counters = sp.in_spare ? spare : ws + p.off_hist;
       uint8_t *const scratch = spare + (sp.in_spare ? sp.room : 0);
@@ -1039,7 +1067,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.out_nodes = nodes + ((1ull << (sl.depth + sl.levels - 1)) - 1);
       if (k + 1 < sp.count) sl.zero_next = split_counters(sp.depth[k + 1], sp.bins, sp.low_cap) / 16;
       else if (!sp.in_spare) sl.zero_next = split_counters(sl.depth, sp.bins, sp.low_cap) / 16;
-      sl.alone = share <= 1;
+      sl.alone = alone;
       sl.err = err;
       PC_TRY(launch_split(sl, st));
       if (facts)
@@ -1101,7 +1129,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       rl.seqs = reinterpret_cast<LeafRec *>(ws + p.off_seqrec);
       rl.scratch = ws + p.off_reduce;
       rl.err = err;
-      rl.alone = share <= 1;
+      rl.alone = alone;
       uint64_t num_seq = 0, rounds = 0;
       PC_TRY(launch_reduce(rl, st, &num_seq, &rounds));
       hl.num_leaves = num_seq;
@@ -1143,7 +1171,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sa.total_words = reinterpret_cast<uint64_t *>(ws + p.off_words);
       sa.payload_cap = payload_words(out_capacity, num_leaves);
       sa.err = err;
-      sa.alone = share <= 1;
+      sa.alone = alone;
       return sa;
     };
     // a4-a5: bit boxes, payload offsets, packing
@@ -1463,10 +1491,10 @@ int knob_find(uint64_t key, uint32_t leaf_size, bool claim, bool *claimed) {
 // same stream into `out` (its size is checked).
 int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config &base,
                void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-               uint32_t *perm, cudaStream_t st, int share, uint32_t *node_max, uint32_t *leaf_max) {
+               uint32_t *perm, cudaStream_t st, bool counted, uint32_t *node_max, uint32_t *leaf_max) {
   RunFacts facts;
   int rc = compress_impl(positions, n, dtype, eb_mode, eb, &base, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st, share, nullptr, &facts);
+                         workspace_bytes, perm, st, counted, nullptr, &facts);
   if (rc) return rc;
   const uint64_t size0 = *out_size;
   uint32_t best_node = base.warp_node_max ? base.warp_node_max : PC_DEFAULT_WARP_NODE_MAX;
@@ -1480,7 +1508,7 @@ int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double
       uint64_t size = 0;
       const auto t0 = std::chrono::steady_clock::now();
       const int r = compress_impl(positions, n, dtype, eb_mode, eb, &c, out, out_capacity, &size, workspace,
-                                  workspace_bytes, perm, st, share);
+                                  workspace_bytes, perm, st, counted);
       const double t = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
       if (r) return r;
       if (size != size0) return PC_ERR_CUDA;  // a launch knob changed the stream: never expected
@@ -1551,10 +1579,10 @@ int tune_knobs(const void *positions, uint64_t n, int dtype, int eb_mode, double
 // the call's class (tuning the class when this call is its first).
 int compress_entry(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                    void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                   uint32_t *perm, cudaStream_t st, int share = 1) {
+                   uint32_t *perm, cudaStream_t st, bool counted = false) {
   if (!cfg || !(cfg->flags & PC_FLAG_AUTOTUNE_KNOBS))
     return compress_impl(positions, n, dtype, eb_mode, eb, cfg, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st, share);
+                         workspace_bytes, perm, st, counted);
   pc_config base = *cfg;
   base.flags &= ~PC_FLAG_AUTOTUNE_KNOBS;
   {
@@ -1582,10 +1610,10 @@ int compress_entry(const void *positions, uint64_t n, int dtype, int eb_mode, do
   }
   if (!claimed)
     return compress_impl(positions, n, dtype, eb_mode, eb, &base, out, out_capacity, out_size, workspace,
-                         workspace_bytes, perm, st, share);
+                         workspace_bytes, perm, st, counted);
   uint32_t node_max = 0, leaf_max = 0;
   const int rc = tune_knobs(positions, n, dtype, eb_mode, eb, base, out, out_capacity, out_size, workspace,
-                            workspace_bytes, perm, st, share, &node_max, &leaf_max);
+                            workspace_bytes, perm, st, counted, &node_max, &leaf_max);
   std::lock_guard<std::mutex> g(g_knob_mu);
   if (g_knob_gen == gen) {
     if (rc == PC_OK) {
@@ -1603,11 +1631,22 @@ int compress_entry(const void *positions, uint64_t n, int dtype, int eb_mode, do
 
 namespace pcx {
 
+InFlight::InFlight(uint64_t n) : dev_(0), n_(n) {
+  cudaGetDevice(&dev_);
+  load_of(dev_).calls += 1;
+  load_of(dev_).particles += n_;
+}
+
+InFlight::~InFlight() {
+  load_of(dev_).calls -= 1;
+  load_of(dev_).particles -= n_;
+}
+
 int compress_device(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                     void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                    cudaStream_t st, int share) {
+                    cudaStream_t st, bool counted) {
   return compress_entry(positions, n, dtype, eb_mode, eb, cfg, out, out_capacity, out_size, workspace,
-                        workspace_bytes, nullptr, st, share);
+                        workspace_bytes, nullptr, st, counted);
 }
 
 }  // namespace pcx
@@ -1765,7 +1804,7 @@ int pc_leaf_size_sweep(const void *positions, uint64_t n, int dtype, int eb_mode
   pc_config cfg = {r_max, PC_FLAG_AUTOTUNE_LEAF};
   Sweep sw = {points, capacity, 0, r_min};
   int rc = compress_impl(positions, n, dtype, eb_mode, eb, &cfg, nullptr, 0, nullptr, workspace, workspace_bytes,
-                         nullptr, static_cast<cudaStream_t>(stream), 1, &sw);
+                         nullptr, static_cast<cudaStream_t>(stream), false, &sw);
   *count = sw.count;
   return rc;
 }

@@ -21,6 +21,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <optional>
 #include <thread>
 #include <vector>
 
@@ -417,8 +418,6 @@ struct pc_server {
         cv_work.wait(lk);
       }
       ++running;
-      // compressions that may run beside this one
-      const int share = int(std::min<uint64_t>(lanes.size(), running + queue.size()));
       lk.unlock();
       pc_completion c = {};
       c.tag = job.req.tag;
@@ -431,7 +430,7 @@ struct pc_server {
         pc_config cfg = {r.leaf_size, r.flags};
         uint64_t size = 0;
         c.status = pcx::compress_device(r.input, r.n, r.dtype, r.eb_mode, r.eb, &cfg, base + ooff, obytes, &size,
-                                        base + soff, sbytes, s, share);
+                                        base + soff, sbytes, s);
         c.output_bytes = size;
       } else {
         c.status = pc_decompress(r.input, r.input_bytes, base + ooff, obytes, base + soff, sbytes, s);
@@ -484,12 +483,18 @@ int pc_compress_batch(pc_compress_item *items, uint32_t count, uint32_t lanes, v
   std::iota(order.begin(), order.end(), 0u);
   std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return items[a].n > items[b].n; });
   uint8_t *ws = static_cast<uint8_t *>(workspace);
+  // the first item of every lane counts from the start, so that the first of them to get
+  // to its partition does not take the SMs of the others
+  std::vector<std::optional<pcx::InFlight>> flight(count);
+  for (uint32_t k = 0; k < lanes; ++k) flight[order[k]].emplace(items[order[k]].n);
   rc = run_lanes(lanes, order, static_cast<cudaStream_t>(stream), [&](uint32_t lane, cudaStream_t s, uint32_t i) {
     pc_compress_item &it = items[i];
     pc_config cfg = {it.leaf_size, it.flags};
     uint64_t size = 0;
+    if (!flight[i]) flight[i].emplace(it.n);
     it.status = pcx::compress_device(it.positions, it.n, it.dtype, it.eb_mode, it.eb, &cfg, it.out, it.out_capacity,
-                                     &size, ws + lane * slice, slice, s, int(lanes));
+                                     &size, ws + lane * slice, slice, s, true);
+    flight[i].reset();
     it.out_size = it.status == PC_OK ? size : 0;
   });
   if (rc) return rc;

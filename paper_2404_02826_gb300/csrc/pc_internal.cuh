@@ -501,10 +501,23 @@ cudaError_t resident_blocks(int threads, size_t smem, int *per_sm) {
 // Self-test switch of the calling host thread: its compress calls issue no
 // tile copy in the partition's scatter (pc_selftest_scatter_timeout).
 void set_drop_tile_copies(bool on);
+// A compression in flight: counted with its n particles on the current device, over all
+// host threads, until it is destroyed.
+class InFlight {
+ public:
+  explicit InFlight(uint64_t n);
+  ~InFlight();
+  InFlight(const InFlight &) = delete;
+  InFlight &operator=(const InFlight &) = delete;
+
+ private:
+  int dev_;
+  uint64_t n_;
+};
 // pc_compress without the optional permutation, on a caller-provided workspace;
-// `share`: compressions that run at the same time (the lanes of a batch or a server).
+// `counted`: the caller holds the call's InFlight.
 int compress_device(const void *positions, uint64_t n, int dtype, int eb_mode, double eb, const pc_config *cfg,
                     void *out, uint64_t out_capacity, uint64_t *out_size, void *workspace, uint64_t workspace_bytes,
-                    cudaStream_t st, int share = 1);
+                    cudaStream_t st, bool counted = false);
 
 }  // namespace pcx
