@@ -1161,12 +1161,13 @@ cudaError_t move_dispatch(const SplitLaunch &a, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st) {
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st, bool *refused) {
   constexpr size_t smem = sizeof(Smem);
   int per_sm = 0;
   cudaError_t e = resident_blocks<k_split>(kT, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1 || a.grid < 1 || a.grid > per_sm * device_sm_count()) return cudaErrorInvalidConfiguration;
+  *refused = per_sm < 1 || a.grid > per_sm * device_sm_count();
+  if (*refused) return cudaSuccess;
   SplitLaunch arg = a;
   arg.part = ((a.chunk + kSplitParts - 1) / kSplitParts + 31u) & ~31u;
   void *args[] = {&arg};
@@ -1174,7 +1175,10 @@ cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st) {
     TraceScope ts("k_split", st);
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_split), dim3(unsigned(a.grid)), dim3(kT), args,
                                     smem, st);
-    if (e != cudaSuccess) return e;
+    *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+               e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
+    if (*refused) cudaGetLastError();
+    if (e != cudaSuccess) return *refused ? cudaSuccess : e;
   }
   return a.src_idx ? move_dispatch<true>(arg, st) : move_dispatch<false>(arg, st);
 }

@@ -1069,7 +1069,9 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       else if (!sp.in_spare) sl.zero_next = split_counters(sl.depth, sp.bins, sp.low_cap) / 16;
       sl.alone = alone;
       sl.err = err;
-      PC_TRY(launch_split(sl, st));
+      bool refused = false;
+      PC_TRY(launch_split(sl, st, &refused));
+      if (refused) break;  // what is left goes level by level
       if (facts)
         for (int l = sl.depth; l < sl.depth + sl.levels; ++l) facts->hbm_levels |= 1ull << l;
       void **t = src;

@@ -237,7 +237,9 @@ struct SplitLaunch {
   uint32_t *barrier;          // zero on entry
   uint32_t *err;
 };
-cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st);
+// `refused`: nothing was queued, because not all CTAs can be placed at once (a stream or context
+// with fewer SMs than the device); the level-by-level launches do without that.
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st, bool *refused);
 uint32_t scatter_tile(int code_bytes, bool with_idx);    // largest tile of one scatter CTA
 uint32_t scatter_groups(int code_bytes, bool with_idx);  // 16-byte group records per tile
 
