@@ -9,6 +9,7 @@
 #include <cstring>
 #include <mutex>
 #include <optional>
+#include <thread>
 #include <vector>
 
 #include "../../include/pc.h"
@@ -58,13 +59,20 @@ void pinned_give(void *p) {
 
 }  // namespace
 
-cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st) {
-  for (uint32_t spins = 0;; ++spins) {
-    if (*word != unset) break;
-    if ((spins & 4095u) != 4095u) continue;
-    const cudaError_t e = cudaStreamQuery(st);
+unsigned wait_mode() {
+  unsigned flags = cudaDeviceScheduleAuto;
+  if (cudaGetDeviceFlags(&flags) != cudaSuccess) cudaGetLastError();
+  return flags & cudaDeviceScheduleMask;
+}
+
+cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st, unsigned mode) {
+  constexpr uint32_t kLook = 4096, kLong = 16 * kLook;  // polls: a look takes a nanosecond or two
+  for (uint32_t spins = 1; *word == unset; ++spins) {
+    if (spins % kLook) continue;
+    const cudaError_t e = mode == cudaDeviceScheduleBlockingSync ? cudaStreamSynchronize(st) : cudaStreamQuery(st);
     if (e == cudaSuccess) break;  // done, the word as the kernels left it
     if (e != cudaErrorNotReady) return e;
+    if (spins % kLong == 0 && mode != cudaDeviceScheduleSpin) std::this_thread::yield();
   }
   std::atomic_thread_fence(std::memory_order_acquire);
   return cudaSuccess;
@@ -103,7 +111,8 @@ cudaError_t HeaderCopy::start(const void *src, uint32_t *ws64, cudaStream_t stre
 cudaError_t HeaderCopy::finish() {
   if (done) return cudaSuccess;
   const volatile uint32_t *flag = reinterpret_cast<volatile uint32_t *>(b.host + kHeaderBytes + 4);
-  const cudaError_t e = wait_word(flag, 0u, st);
+  // work is queued behind the word and more is to follow it: not in a synchronisation
+  const cudaError_t e = wait_word(flag, 0u, st, cudaDeviceScheduleYield);
   if (e != cudaSuccess) return e;
   if (*flag == 0u) return cudaErrorUnknown;
   std::memcpy(h, b.host, kHeaderBytes);
@@ -737,6 +746,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
   std::optional<InFlight> flight;
   if (!counted) flight.emplace(n);
   HostBlock hb;  // the value range, then the call's end
+  unsigned mode = cudaDeviceScheduleAuto;
   PC_TRY(cudaMemsetAsync(ws + p.off_zero, 0, p.zero_bytes, st));
 
   HeaderLaunch hl = {};
@@ -778,7 +788,8 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     PC_TRY(launch_range(ra, st));
     RangeResult rr;
     if (hb.host) {
-      PC_TRY(wait_word(flag, 0u, st));
+      mode = wait_mode();  // while the range kernel runs
+      PC_TRY(wait_word(flag, 0u, st, mode));
       if (*flag == 0u) return PC_ERR_CUDA;
       std::memcpy(&rr, hb.host, sizeof(rr));
       hb.pending = false;
@@ -1298,7 +1309,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
     hb.pending = true;
     hl.host_end = reinterpret_cast<CallEnd *>(hb.dev + 192);
     PC_TRY(launch_header(hl, st));
-    PC_TRY(wait_word(&end->done, 0u, st));
+    PC_TRY(wait_word(&end->done, 0u, st, mode));
     if (end->done == 0u) return PC_ERR_CUDA;
     back.total = end->total;
     back.err = end->err;
@@ -1375,6 +1386,7 @@ int decompress_impl(const void *stream_data, uint64_t stream_bytes, void *out_po
   if (early)
     PC_TRY(launch_decode_prologue(static_cast<const uint8_t *>(stream_data), stream_bytes,
                                   (workspace_bytes - tab_end) / decode_chunk_bytes(1), err, qb, tab, chunks, st));
+  const unsigned mode = wait_mode();  // while those run
   PC_TRY(hc.finish());
   pc_info I = {};
   int rc = parse_header(hc.h, PC_HEADER_BYTES, &I);
@@ -1423,7 +1435,7 @@ int decompress_impl(const void *stream_data, uint64_t stream_bytes, void *out_po
   PC_TRY(launch_decode(da, st));
   uint32_t e = kUnset;
   if (da.host_err) {
-    PC_TRY(wait_word(hc.host_err(), kUnset, st));
+    PC_TRY(wait_word(hc.host_err(), kUnset, st, mode));
     e = *hc.host_err();
     hc.b.pending = false;
   }

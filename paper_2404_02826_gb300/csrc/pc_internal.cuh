@@ -415,8 +415,12 @@ inline cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStrea
 // Waits until the word, in page-locked host memory that a kernel of `st` writes,
 // is no longer `unset`, or the stream is done.  The word is watched by the
 // calling thread: a result arrives 1 to 2 us after it is written, a copy and a
-// synchronisation of the stream take 8.
-cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st);
+// synchronisation of the stream take 8.  Past the first few microseconds the wait goes
+// on as `mode` says (wait_mode, the device's scheduling flags): blocked in a
+// synchronisation of the stream with cudaDeviceScheduleBlockingSync; watching without
+// a pause with cudaDeviceScheduleSpin; else yielding the processor now and then.
+cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st, unsigned mode);
+unsigned wait_mode();
 
 // A page-locked staging block for the results that kernels write to host memory
 // (null without one, and while kernels are traced: each then needs its events).
