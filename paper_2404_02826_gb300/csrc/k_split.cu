@@ -8,9 +8,9 @@
 // in) - and then every particle moves once, straight into its node of depth +
 // levels.
 //
-// k_split: one persistent CTA per SM, launched cooperatively; CTA c owns the
-// contiguous positions [c * chunk, (c + 1) * chunk), and a segment is what a
-// CTA holds of one subroot.  Per level:
+// k_split: one persistent CTA per SM, as many as start in time (join); CTA c of
+// those owns the contiguous positions [c * chunk, (c + 1) * chunk), and a
+// segment is what a CTA holds of one subroot.  Per level:
 //   A     every particle takes its child of the level above (code against the
 //         split plane) and is counted in a shared histogram of its code on the
 //         level's axis, one run of bins per node; the bins of all nodes share
@@ -81,6 +81,8 @@ constexpr uint32_t kStateWords = kSplitStateWords;
 static_assert(kStateWords == 17 * kHalf, "kept part of NodeTab");
 
 struct Misc {
+  uint32_t c, members;          // this CTA among those that take part
+  uint32_t chunk, part;         // positions of a CTA; of one of the move
   uint32_t s0, s1;              // subroots of this CTA
   uint32_t soff, scnt;          // current subroot
   uint32_t b0, b1;              // current segment
@@ -102,6 +104,74 @@ struct Smem {
 static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
 static_assert(offsetof(Smem, bins) % 16 == 0 && offsetof(Smem, sum) % 16 == 0, "16-byte accesses");
 
+// Positions of a CTA when m take part, a multiple of 16, and of a CTA of the move.
+__device__ __forceinline__ uint32_t chunk_of(uint64_t n, uint32_t m) { return uint32_t(((n + m - 1) / m + 15u) & ~15ull); }
+__device__ __forceinline__ uint32_t part_size(uint32_t chunk) {
+  return ((chunk + kSplitParts - 1) / kSplitParts + 31u) & ~31u;
+}
+
+// The CTAs wait for one another, so those that take part have to be running, and the launch
+// does not ask for all of them to be placed at once: a kernel of somebody else's that stays
+// on an SM would hold up such a launch, and a stream with fewer SMs than the device would
+// refuse it.  Instead the CTAs count themselves as they start (join), and the first to have
+// waited as long as the missing ones would save (in cycles: 0.49 a particle and level on one
+// CTA, shared by the k that came instead of all; kJoinLeast to kJoinMost), or the last of
+// all, closes the count: the k that came split the work, one that starts later leaves.  Nobody
+// waits for a CTA that has not started, and every wait ends: each CTA closes the count itself
+// when its time is up.  The count starts ahead of the wait for the kernel before, so that it
+// is complete by then where all come at once, the usual case.
+// A cooperative launch took as long: 2^20 particles 166.0 us a call, so 165.7; 3,000,017 with
+// the permutation 265.2, so 264.8; a batch of 48 snapshots 4.32 ms, so 4.35.
+constexpr uint64_t kJoinLeast = 20000;         // cycles, about 10 us
+constexpr uint64_t kJoinMost = 100000000;      // about 50 ms
+constexpr uint32_t kJoinClosed = 0x80000000u;  // bit of the count
+
+__device__ __forceinline__ uint32_t join_count(const SplitLaunch &a) {
+  uint32_t m;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(m) : "l"(a.sync + 2) : "memory");
+  return m;
+}
+__device__ __forceinline__ void join_close(const SplitLaunch &a, uint32_t m) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.sync + 2), "r"(m) : "memory");
+}
+// Thread 0: `mine` CTAs came before this one; how many take part, if that is known soon (else 0).
+__device__ __forceinline__ uint32_t join(const SplitLaunch &a, uint32_t &mine) {
+  mine = atomicAdd(a.sync + 1, 1u);
+  if (mine + 1u == gridDim.x) {
+    join_close(a, gridDim.x);
+    return gridDim.x;
+  }
+  uint32_t m = 0;
+  for (int i = 0; i < 8 && !m && !(mine & kJoinClosed); ++i) m = join_count(a);
+  return m;
+}
+// The same, once it is known (0: not this CTA).
+__device__ __forceinline__ uint32_t join_wait(const SplitLaunch &a, uint32_t mine, uint32_t m) {
+  if (mine & kJoinClosed) return 0;
+  if (m) return m;
+  uint32_t *const came = a.sync + 1;
+  const uint32_t all = gridDim.x;
+  const long long t0 = clock64();
+  for (uint32_t spins = 0; spins < kGridSpin; ++spins) {
+    m = join_count(a);
+    if (m) return m;
+    const uint64_t waited = uint64_t(clock64() - t0);
+    if (waited < kJoinLeast) continue;
+    uint32_t k;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(k) : "l"(came) : "memory");
+    if (k & kJoinClosed) continue;  // the count follows
+    if (waited >= min(kJoinMost, uint64_t(a.levels) * (a.n / 2) * (all - k) / (uint64_t(all) * k))) {
+      const uint32_t was = atomicOr(came, kJoinClosed);
+      if (!(was & kJoinClosed)) {
+        join_close(a, was);
+        return was;
+      }
+    }
+  }
+  atomicOr(a.err, kErrTimeout);
+  return 0;
+}
+
 // Grid barrier in two halves: between them a CTA does what no other CTA waits
 // for.  Bounded; the wait is true when it gave up or the call has failed: the
 // caller leaves the kernel, as every other CTA does at its next barrier.
@@ -109,18 +179,18 @@ __device__ __forceinline__ void grid_arrive(const SplitLaunch &a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(a.barrier, 1u);
+    atomicAdd(a.sync, 1u);
   }
 }
-__device__ __forceinline__ bool grid_wait(const SplitLaunch &a, uint32_t &epoch) {
+__device__ __forceinline__ bool grid_wait(const SplitLaunch &a, const Misc &M, uint32_t &epoch) {
   bool bad = false;
   ++epoch;
   if (threadIdx.x == 0) {
-    const uint32_t want = epoch * gridDim.x;
+    const uint32_t want = epoch * M.members;
     uint32_t spins = 0;
     for (;;) {
       uint32_t v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.barrier) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.sync) : "memory");
       if (v >= want) break;
       ++spins;
       if (spins > kGridSpin) {
@@ -137,9 +207,9 @@ __device__ __forceinline__ bool grid_wait(const SplitLaunch &a, uint32_t &epoch)
   }
   return __syncthreads_or(bad) != 0;
 }
-__device__ __forceinline__ bool grid_sync(const SplitLaunch &a, uint32_t &epoch) {
+__device__ __forceinline__ bool grid_sync(const SplitLaunch &a, const Misc &M, uint32_t &epoch) {
   grid_arrive(a);
-  return grid_wait(a, epoch);
+  return grid_wait(a, M, epoch);
 }
 
 __device__ __forceinline__ uint32_t half_of(const uint4 &w, int e) {
@@ -167,14 +237,14 @@ __device__ __forceinline__ void enter_seg(const Ctx &x, uint32_t s, int l, bool 
     node_range(a.n, a.depth, s, off, cnt);
     x.M.soff = uint32_t(off);
     x.M.scnt = uint32_t(cnt);
-    const uint32_t r0 = blockIdx.x * a.chunk;
-    const uint64_t r1 = min(uint64_t(r0) + a.chunk, a.n);
+    const uint32_t r0 = x.M.c * x.M.chunk;
+    const uint64_t r1 = min(uint64_t(r0) + x.M.chunk, a.n);
     x.M.b0 = max(uint32_t(off), r0);
     x.M.b1 = uint32_t(min(off + cnt, r1));
-    x.M.clo = uint32_t(off) / a.chunk;
+    x.M.clo = uint32_t(off) / x.M.chunk;
   }
   if (load) {
-    const uint32_t *src = a.state + uint64_t(blockIdx.x + s) * kStateWords;
+    const uint32_t *src = a.state + uint64_t(x.M.c + s) * kStateWords;
     uint32_t *dst = reinterpret_cast<uint32_t *>(&x.N);
     for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
   }
@@ -198,7 +268,7 @@ __device__ __forceinline__ void enter_seg(const Ctx &x, uint32_t s, int l, bool 
 
 __device__ __forceinline__ void keep_seg(const Ctx &x, uint32_t s) {
   __syncthreads();
-  uint32_t *dst = x.a.state + uint64_t(blockIdx.x + s) * kStateWords;
+  uint32_t *dst = x.a.state + uint64_t(x.M.c + s) * kStateWords;
   const uint32_t *src = reinterpret_cast<const uint32_t *>(&x.N);
   for (uint32_t i = threadIdx.x; i < kStateWords; i += kT) dst[i] = src[i];
 }
@@ -360,15 +430,15 @@ __device__ __noinline__ uint32_t select_block(Misc &M, const uint32_t *list, uin
 }
 
 // Counters of the children in F: one row per part of the chunk and warp.
-__device__ __forceinline__ uint32_t part_of(const SplitLaunch &a, uint32_t pos) {
-  const uint32_t q = (pos - blockIdx.x * a.chunk) / a.part;
+__device__ __forceinline__ uint32_t part_of(const Misc &M, uint32_t pos) {
+  const uint32_t q = (pos - M.c * M.chunk) / M.part;
   return min(q, uint32_t(kSplitParts - 1));
 }
 
 // The CTA of the move that holds a position.
-__device__ __forceinline__ uint32_t move_part(const SplitLaunch &a, uint32_t pos) {
-  const uint32_t c = pos / a.chunk;
-  return c * kSplitParts + min((pos - c * a.chunk) / a.part, uint32_t(kSplitParts - 1));
+__device__ __forceinline__ uint32_t move_part(const Misc &M, uint32_t pos) {
+  const uint32_t c = pos / M.chunk;
+  return c * kSplitParts + min((pos - c * M.chunk) / M.part, uint32_t(kSplitParts - 1));
 }
 
 // 8 consecutive particles: their codes on the axis of the level above and on
@@ -418,7 +488,7 @@ __device__ __forceinline__ void pass_a(const Ctx &x, const Pass &a, Step &next, 
     uint32_t mask = 0xffu;
     if (pos < b0) mask &= 0xffu << (b0 - pos);
     if (pos + 8u > b1) mask &= 0xffu >> (pos + 8u - b1);
-    uint32_t *const bins = LAST ? x.bins + (part_of(x.a, pos) * kW + x.warp) * kNodes : x.bins;
+    uint32_t *const bins = LAST ? x.bins + (part_of(x.M, pos) * kW + x.warp) * kNodes : x.bins;
     const int32_t off0 = FIRST ? N.off[0] : 0;
     uint32_t w0 = 0, w1 = 0, hit = 0;
     auto one = [&](int e) {
@@ -472,7 +542,7 @@ __device__ __forceinline__ void resolve_ties(const Ctx &x, const Pass &a, const 
       x.a.node[p] = uint8_t(2 * j);
       uint32_t *left, *right;
       if (LAST) {
-        left = x.bins + (part_of(x.a, p) * kW + x.warp) * kNodes + 2 * j;
+        left = x.bins + (part_of(x.M, p) * kW + x.warp) * kNodes + 2 * j;
         right = left + 1;
       } else {  // the code lies beside a list of up to half the room
         const uint32_t c = x.M.ties <= kBins / 2 ? l[i + kBins / 2] : uint32_t(__ldcg(a.cur + p));
@@ -552,19 +622,26 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
   Smem &P = *reinterpret_cast<Smem *>(sm);
   Misc &M = P.M;
   NodeTab &N = P.N;
+  uint32_t mine = 0, members = 0;
+  if (threadIdx.x == 0) members = join(a, mine);  // its words were zeroed ahead of the kernel before
+  dep_wait();
   if (call_failed(a.err)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const Ctx x = {a, M, N, P.bins, P.sum, lane, warp};
-  const uint32_t c = blockIdx.x, S = 1u << a.depth;
+  const uint32_t S = 1u << a.depth;
   const int K = a.levels;
   uint32_t epoch = 0;
   if (threadIdx.x == 0) {
-    const uint64_t r0 = uint64_t(c) * a.chunk;
+    M.c = mine;
+    M.members = join_wait(a, mine, members);
+    M.chunk = chunk_of(a.n, max(M.members, 1u));
+    M.part = part_size(M.chunk);
+    const uint64_t r0 = uint64_t(M.c) * M.chunk;
     M.s0 = 1;
     M.s1 = 0;
     M.nbins = 0;
-    if (r0 < a.n) {  // the subroots holding the first and the last position
-      const uint64_t r1 = min(r0 + a.chunk, a.n) - 1;
+    if (M.members && r0 < a.n) {  // the subroots holding the first and the last position
+      const uint64_t r1 = min(r0 + M.chunk, a.n) - 1;
       for (int e = 0; e < 2; ++e) {
         uint32_t lo = 0, hi = S - 1;
         while (lo < hi) {
@@ -580,9 +657,10 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     }
   }
   __syncthreads();
-  const uint32_t s0 = M.s0, s1 = M.s1;
+  if (M.members == 0) return;
+  const uint32_t c = M.c, s0 = M.s0, s1 = M.s1;
   const bool multi = s1 > s0;
-  const uint32_t gthreads = gridDim.x * kT, gtid = c * kT + threadIdx.x;
+  const uint32_t gthreads = M.members * kT, gtid = c * kT + threadIdx.x;
 
   for (int l = 0; l < K; ++l) {
     const uint32_t nodes = 1u << l, half = nodes >> 1;
@@ -620,7 +698,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
       uint4 *z = reinterpret_cast<uint4 *>(a.hist + uint64_t((l + 1) & 1) * S * a.bins);
       for (uint32_t i = gtid; i < S * (a.bins / 4); i += gthreads) z[i] = make_uint4(0, 0, 0, 0);
     }
-    if (grid_wait(a, epoch)) return;
+    if (grid_wait(a, M, epoch)) return;
     // ---- sel1 and B ----
     for (uint32_t s = s0; s <= s1; ++s) {
       if (multi) {
@@ -718,7 +796,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     }
     if (!multi)
       for (uint32_t b = threadIdx.x; b < M.nbins; b += kT) P.bins[b] = 0;
-    if (grid_wait(a, epoch)) return;
+    if (grid_wait(a, M, epoch)) return;
     // ---- sel2: a warp per node ----
     for (uint32_t s = s0; s <= s1; ++s) {
       if (multi) {
@@ -810,26 +888,26 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
     run_a<false, true>(x, pf, step);
     for (uint32_t i = threadIdx.x; i < kSplitParts * kNodes; i += kT) {
       const uint32_t q = i / kNodes, b = i % kNodes;
-      if (q < part_of(a, M.b0) || q > part_of(a, M.b1 - 1) || b >= 2 * half) continue;
+      if (q < part_of(M, M.b0) || q > part_of(M, M.b1 - 1) || b >= 2 * half) continue;
       uint32_t v = 0;
 #pragma unroll 8
       for (int w = 0; w < kW; ++w) v += P.bins[(q * kW + w) * kNodes + b];
       a.segcnt[uint64_t(b) * (gridDim.x * kSplitParts + S) + c * kSplitParts + q + s] = v;
     }
   }
-  if (grid_sync(a, epoch)) return;
+  if (grid_sync(a, M, epoch)) return;
   dep_launch();
   // first place of every child for every part: exclusive sums along the parts of a
   // subroot, in place, a warp per subroot and child
   const uint64_t msegs = uint64_t(gridDim.x) * kSplitParts + S;
-  for (uint32_t i = c + gridDim.x * warp; i < S << K; i += gridDim.x * kW) {
+  for (uint32_t i = c + M.members * warp; i < S << K; i += M.members * kW) {
     const uint32_t s = i >> K, b = i & ((1u << K) - 1u);
     uint64_t soff, scnt, off, cnt;
     node_range(a.n, a.depth, s, soff, scnt);
     node_range(scnt, K, b, off, cnt);
     uint32_t run = uint32_t(soff + off);
     uint32_t *const row = a.segcnt + b * msegs + s;
-    const uint32_t m0 = move_part(a, uint32_t(soff)), m1 = move_part(a, uint32_t(soff + scnt - 1));
+    const uint32_t m0 = move_part(M, uint32_t(soff)), m1 = move_part(M, uint32_t(soff + scnt - 1));
     for (uint32_t k0 = m0; k0 <= m1; k0 += 4 * 32) {
       uint32_t v[4];
 #pragma unroll
@@ -1036,9 +1114,12 @@ __global__ void __launch_bounds__(kMT, 2) k_move(const __grid_constant__ SplitLa
   const uint32_t m = blockIdx.x, S = 1u << a.depth;
   const int K = a.levels;
   const uint32_t NB = 1u << K;
-  const uint64_t c0 = uint64_t(m / kSplitParts) * a.chunk, c1 = min(c0 + a.chunk, a.n);
-  const uint64_t q0 = c0 + uint64_t(m % kSplitParts) * a.part;
-  const uint64_t q1 = m % kSplitParts == kSplitParts - 1 ? c1 : min(q0 + a.part, c1);
+  const uint32_t members = __ldcg(a.sync + 2);  // the CTAs that found the planes
+  if (m >= members * kSplitParts) return;
+  const uint32_t chunk = chunk_of(a.n, members), part = part_size(chunk);
+  const uint64_t c0 = uint64_t(m / kSplitParts) * chunk, c1 = min(c0 + chunk, a.n);
+  const uint64_t q0 = c0 + uint64_t(m % kSplitParts) * part;
+  const uint64_t q1 = m % kSplitParts == kSplitParts - 1 ? c1 : min(q0 + part, c1);
   if (q0 >= q1) return;
   if (threadIdx.x < 2) {  // the subroots holding the first and the last position
     const uint64_t p = threadIdx.x ? q1 - 1 : q0;
@@ -1147,7 +1228,7 @@ cudaError_t move_launch(const SplitLaunch &a, cudaStream_t st) {
 template <bool IDX, int BITS>
 cudaError_t move_rows(const SplitLaunch &a, cudaStream_t st) {
   if constexpr (!IDX && BITS <= 7) {
-    if (a.part > 8u * kMT) return move_launch<IDX, BITS, 16>(a, st);
+    if (a.n / (uint64_t(a.grid) * kSplitParts) > 8u * kMT) return move_launch<IDX, BITS, 16>(a, st);
   }
   return move_launch<IDX, BITS, 8>(a, st);
 }
@@ -1161,26 +1242,18 @@ cudaError_t move_dispatch(const SplitLaunch &a, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st, bool *refused) {
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st) {
   constexpr size_t smem = sizeof(Smem);
   int per_sm = 0;
   cudaError_t e = resident_blocks<k_split>(kT, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  *refused = per_sm < 1 || a.grid > per_sm * device_sm_count();
-  if (*refused) return cudaSuccess;
-  SplitLaunch arg = a;
-  arg.part = ((a.chunk + kSplitParts - 1) / kSplitParts + 31u) & ~31u;
-  void *args[] = {&arg};
+  if (per_sm < 1 || a.grid < 1) return cudaErrorInvalidConfiguration;
   {
     TraceScope ts("k_split", st);
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_split), dim3(unsigned(a.grid)), dim3(kT), args,
-                                    smem, st);
-    *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
-               e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
-    if (*refused) cudaGetLastError();
-    if (e != cudaSuccess) return *refused ? cudaSuccess : e;
+    e = launch_dependent(a.alone, k_split, dim3(unsigned(a.grid)), dim3(kT), smem, st, a);
+    if (e != cudaSuccess) return e;
   }
-  return a.src_idx ? move_dispatch<true>(arg, st) : move_dispatch<false>(arg, st);
+  return a.src_idx ? move_dispatch<true>(a, st) : move_dispatch<false>(a, st);
 }
 
 }  // namespace pcx

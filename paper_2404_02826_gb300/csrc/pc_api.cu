@@ -307,9 +307,8 @@ int split_max_levels(int bits, int b) {
 }
 constexpr uint64_t kSplitMinRoot = 1u << 17;
 constexpr uint64_t kSplitMinChunk = 4096;  // particles of a CTA: fewer CTAs for small inputs
-constexpr uint64_t kSplitOwnTies = 4 * kSplitBins;  // up to here a CTA's ties always fit its shared memory
-constexpr int kSplitLaunches = 16;         // one barrier word each
-constexpr uint64_t kBarrierAt = 128;       // their place after the error word, a cache line of its own
+constexpr int kSplitLaunches = 8;          // kSplitSync words each
+constexpr uint64_t kSyncAt = 128;          // their place after the error word, a cache line of its own
 
 bool split_roots_ok(uint64_t n, int depth) {
   return depth == 0 || ((1ull << depth) <= kSplitMaxRoots && (n >> depth) >= kSplitMinRoot);
@@ -317,8 +316,7 @@ bool split_roots_ok(uint64_t n, int depth) {
 
 // CTAs of a launch: one per SM of the call's `cap`, fewer for small inputs.
 uint64_t split_grid(uint64_t n, uint64_t cap) {
-  const uint64_t g = std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap));
-  return n <= kSplitOwnTies ? std::max(g, (n + kSplitBins - 1) / kSplitBins) : g;
+  return std::max<uint64_t>(1, std::min<uint64_t>(n / kSplitMinChunk, cap));
 }
 
 // Compressions in flight, by device.
@@ -335,11 +333,11 @@ Load &in_flight() {
   return load_of(dev);
 }
 
-// SMs of a call of n particles for a launch whose CTAs must all be placed at once: its part
-// of the particles in flight, and one left to every other call; all of them when it is
-// alone.  By work, not by calls: one snapshot of 2^26 particles among fifteen of 10^4 on
-// eight lanes takes 3.42 ms (2.95 alone; 11.5 with an eighth of the SMs), and 24 of 10^6 in
-// plain calls from eight host threads 2.2 ms (3.8 when each asks for all SMs).
+// SMs of a call of n particles for a launch whose CTAs wait for one another: its part of the
+// particles in flight, and one left to every other call; all of them when it is alone.  By
+// work, not by calls: one snapshot of 2^26 particles among fifteen of 10^4 on eight lanes
+// takes 3.42 ms (2.95 alone; 11.5 with an eighth of the SMs), and 24 of 10^6 in plain calls
+// from eight host threads 2.2 ms (3.8 when each asks for all SMs).
 uint64_t sm_share(uint64_t n, uint64_t sms) {
   const Load &load = in_flight();
   const uint64_t calls = load.calls, particles = std::max<uint64_t>(load.particles, n);
@@ -350,7 +348,7 @@ uint64_t sm_share(uint64_t n, uint64_t sms) {
 
 // Scratch of a launch of `grid` CTAs, in the order in which it is laid out.
 struct SplitScratch {
-  uint64_t node, seglow, segcnt, ties, state, seghist, total;
+  uint64_t node, seglow, segcnt, state, seghist, total;
 };
 SplitScratch split_scratch(uint64_t n, int depth, uint32_t low_cap, uint64_t grid) {
   const uint64_t roots = 1ull << depth, segs = grid + roots;
@@ -364,7 +362,6 @@ SplitScratch split_scratch(uint64_t n, int depth, uint32_t low_cap, uint64_t gri
   s.node = take(n + 64);
   s.seglow = take(segs * low_cap * 4);
   s.segcnt = take((kSplitParts * grid + roots) * 4 << kSplitMaxLevels);
-  s.ties = take(n > kSplitOwnTies ? 4 * n : 0);
   if (depth > 0) {
     s.state = take(segs * kSplitStateWords * 4);
     s.seghist = take(2 * roots * kSplitBins * 4);
@@ -565,8 +562,8 @@ int make_plan(uint64_t n, int dtype, const pc_config *cfg, bool idx, int sm_coun
   o = align_up(o + 8 * (kSubMaxLevels + 1));
   p.off_status = o;
   o = align_up(o + 8 * subtree_status_entries(p.levels));
-  p.off_err = o;  // the error word; from kBarrierAt on the barrier words of the launches of k_split.cu
-  o = align_up(o + kBarrierAt + 4 * kSplitLaunches);
+  p.off_err = o;  // the error word; from kSyncAt on the words of the launches of k_split.cu
+  o = align_up(o + kSyncAt + 4 * kSplitSync * kSplitLaunches);
   p.off_total = o;
   o = align_up(o + 8);
   p.zero_bytes = o - p.off_zero;
@@ -1050,7 +1047,6 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.depth = sp.depth[k];
       sl.levels = sp.levels[k];
       sl.grid = int(split_grid(n, sm_share(n, uint64_t(device_sm_count()))));
-      sl.chunk = uint32_t(((n + sl.grid - 1) / sl.grid + 15) & ~15ull);
       uint8_t *const counters = sp.in_spare ? spare : ws + p.off_hist;
       uint8_t *const scratch = spare + (sp.in_spare ? sp.room : 0);
       const SplitScratch at = split_scratch(n, sl.depth, sp.low_cap, uint64_t(sl.grid));
@@ -1059,12 +1055,12 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       sl.low_cap = sp.low_cap;
       sl.seglow = reinterpret_cast<uint32_t *>(scratch + at.seglow);
       sl.segcnt = reinterpret_cast<uint32_t *>(scratch + at.segcnt);
-      sl.ties = n > kSplitOwnTies ? reinterpret_cast<uint32_t *>(scratch + at.ties) : nullptr;
+      sl.ties = static_cast<uint32_t *>(dst[0]);  // 4 of the 6 bytes a particle that the move writes later
       if (sl.depth > 0) {
         sl.state = reinterpret_cast<uint32_t *>(scratch + at.state);
         sl.seghist = reinterpret_cast<uint32_t *>(scratch + at.seghist);
       }
-      sl.barrier = reinterpret_cast<uint32_t *>(ws + p.off_err + kBarrierAt) + k;
+      sl.sync = reinterpret_cast<uint32_t *>(ws + p.off_err + kSyncAt) + kSplitSync * k;
       sl.hist = reinterpret_cast<uint32_t *>(counters);
       sl.low = sl.hist + (2ull << sl.depth) * sp.bins;
       for (int d = 0; d < 3; ++d) {
@@ -1080,9 +1076,7 @@ int compress_impl(const void *positions, uint64_t n, int dtype, int eb_mode, dou
       else if (!sp.in_spare) sl.zero_next = split_counters(sl.depth, sp.bins, sp.low_cap) / 16;
       sl.alone = alone;
       sl.err = err;
-      bool refused = false;
-      PC_TRY(launch_split(sl, st, &refused));
-      if (refused) break;  // what is left goes level by level
+      PC_TRY(launch_split(sl, st));
       if (facts)
         for (int l = sl.depth; l < sl.depth + sl.levels; ++l) facts->hbm_levels |= 1ull << l;
       void **t = src;

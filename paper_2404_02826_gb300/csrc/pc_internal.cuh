@@ -200,7 +200,7 @@ struct LevelLaunch {
 };
 cudaError_t launch_level(const LevelLaunch &a, cudaStream_t st);
 cudaError_t launch_scatter(const LevelLaunch &a, cudaStream_t st);
-// Several levels in one cooperative launch (k_split.cu): 16-bit codes, split
+// Several levels in one launch (k_split.cu): 16-bit codes, split
 // axis depth mod 3, every node above depth + levels larger than a leaf.
 constexpr int kSplitMaxLevels = 8;         // a particle's node below its subroot fits a byte
 constexpr uint32_t kSplitBins = 16384;     // counters of one level's histogram, shared by its nodes, at most
@@ -208,11 +208,11 @@ constexpr uint32_t kSplitLow = 8192;       // counters of the codes in the nodes
 constexpr uint32_t kSplitStateWords = 17u << (kSplitMaxLevels - 1);
 constexpr int kSplitParts = 2;             // parts of a CTA's positions, one per CTA of the move
 constexpr uint32_t kSplitMaxRoots = 512;   // subroots of one launch
+constexpr int kSplitSync = 3;              // words by which a launch's CTAs find together
 struct SplitLaunch {
   uint64_t n;
   int depth, levels;          // the subroots' depth, levels below them (1 .. kSplitMaxLevels)
-  int grid;                   // CTAs, at most one per SM
-  uint32_t chunk;             // positions per CTA, a multiple of 16
+  int grid;                   // CTAs, at most one per SM; those that start in time take part
   uint32_t root_hi[3];        // codes of axis d lie in [0, root_hi[d]]
   const LevelNode *parents;   // the records of depth - 1 (null at depth 0)
   LevelNode *out_nodes;       // the records of depth + levels - 1 (written)
@@ -223,23 +223,20 @@ struct SplitLaunch {
   uint8_t *node;              // [n + 64] scratch: node below the subroot
   uint32_t *hist;             // [2][2^depth][bins], zero on entry
   uint32_t *low;              // [2][2^depth][low_cap], zero on entry
-  uint32_t part;              // positions per CTA of the move (set by launch_split)
   // scratch; a segment is what a CTA holds of a subroot (at most grid + 2^depth of them)
   uint32_t *seglow;           // [low_cap][grid + 2^depth] codes in the median bins, by segment
   uint32_t bins;              // counters of a level's histogram: a power of two, at most kSplitBins
   uint32_t low_cap;           // at least 2^l << shift of every level l, whatever the codes; a multiple of 4
   uint32_t *segcnt;           // [2^kSplitMaxLevels][kSplitParts grid + 2^depth] children, by part of a segment
-  uint32_t *ties;             // [n] positions of ties (null with chunks of at most kSplitBins)
+  uint32_t *ties;             // [n] positions of ties
   uint32_t *state;            // [grid + 2^depth][kSplitStateWords] (depth > 0)
   uint32_t *seghist;          // [2^(depth + 1)][kSplitBins] (depth > 0)
   uint64_t zero_next;         // 16-byte words left zero from hist on: what the next launch counts in
   bool alone;                 // no other call shares the GPU
-  uint32_t *barrier;          // zero on entry
+  uint32_t *sync;             // kSplitSync words, zero on entry: barrier, CTAs that came, CTAs that take part
   uint32_t *err;
 };
-// `refused`: nothing was queued, because not all CTAs can be placed at once (a stream or context
-// with fewer SMs than the device); the level-by-level launches do without that.
-cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st, bool *refused);
+cudaError_t launch_split(const SplitLaunch &a, cudaStream_t st);
 uint32_t scatter_tile(int code_bytes, bool with_idx);    // largest tile of one scatter CTA
 uint32_t scatter_groups(int code_bytes, bool with_idx);  // 16-byte group records per tile
 

@@ -1,7 +1,7 @@
 """Compression on a stream that has a part of the device's SMs (a green context):
-the launch of several levels (csrc/k_split.cu) needs all its CTAs placed at once
-and is refused there when it asks for more, and the levels then go one by one.
-Streams, permutations and decoded positions equal the oracle's.
+the launch of several levels (csrc/k_split.cu), whose CTAs wait for one another,
+takes the SMs there are.  Streams, permutations and decoded positions equal the
+oracle's.
 """
 import ctypes
 
