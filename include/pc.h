@@ -25,7 +25,7 @@
  *     and decompress each wait for a few bytes (the value range, then the
  *     final size or the error word) and so return with their work finished.
  *     The kernels write those bytes into page-locked host blocks of 4 KB, where
- *     the calling thread watches for them: past the first few microseconds as
+ *     the calling thread watches for them: past some 20 us as
  *     the device's scheduling flags ask (cudaSetDeviceFlags: blocked with
  *     cudaDeviceScheduleBlockingSync, without a pause with
  *     cudaDeviceScheduleSpin, else yielding the processor now and then).  The

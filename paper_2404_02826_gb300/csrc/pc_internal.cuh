@@ -412,7 +412,7 @@ inline cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStrea
 // Waits until the word, in page-locked host memory that a kernel of `st` writes,
 // is no longer `unset`, or the stream is done.  The word is watched by the
 // calling thread: a result arrives 1 to 2 us after it is written, a copy and a
-// synchronisation of the stream take 8.  Past the first few microseconds the wait goes
+// synchronisation of the stream take 8.  Past some 20 us the wait goes
 // on as `mode` says (wait_mode, the device's scheduling flags): blocked in a
 // synchronisation of the stream with cudaDeviceScheduleBlockingSync; watching without
 // a pause with cudaDeviceScheduleSpin; else yielding the processor now and then.
