@@ -20,8 +20,9 @@
 //            smaller (key, index) meets its bit box (the box found blocking it
 //            in an earlier round is checked first).  Taken boxes are pairwise
 //            disjoint, so no particle lies in two of them.
-//   take     a cluster of blocks per taken box (a round takes a few boxes, so
-//            that what bounds it is the time of one): ranks in its sequence
+//   take     a cluster of blocks per taken box while the round's boxes are few
+//            and large (what bounds it is the time of one), else a block per
+//            box: ranks in its sequence
 //            for its centre, its other live particles in slot order, then, for
 //            every alive box c that is not taken and meets it, the live
 //            particles of c inside its bit box, by c and slot (counted first,
@@ -349,7 +350,7 @@ __device__ __forceinline__ Box6 box6(const RBox &b) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_rd_select(State S) {
-  dep_launch();
+  if (gridDim.x <= 2048u) dep_launch();  // in each of 8192 blocks it costs more than it saves: 18.2 us a launch, 15.8
   dep_wait();
   if (S.ctr->alive == 0) return;
   const uint32_t a = (blockIdx.x * kThreads + threadIdx.x) >> 5;
@@ -394,6 +395,7 @@ __global__ void __launch_bounds__(kThreads) k_rd_select(State S) {
 
 constexpr int kTakeThreads = 1024;
 constexpr uint32_t kTakeCluster = 4;  // blocks per taken box
+constexpr uint32_t kClusterBox = 1024;  // leaves of at most this many particles have none
 constexpr int kTakeWarps = kTakeThreads / 32;
 static_assert(kTakeWarps >= 2 && kTakeWarps <= 32, "take: a search warp and an own-particle warp, one scan warp");
 
@@ -557,19 +559,24 @@ __device__ __forceinline__ uint32_t warp_pick_inside(const State &S, const C *q0
 // the taken box's own particles.
 __device__ __forceinline__ void search_sync(int nthreads) { asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory"); }
 
-// A cluster of blocks per taken box: the ranks of its sequence, its length into
-// seq_cnt.  The last warp of every block ranks its share of the box's own
+// A group of blocks per taken box, a cluster or one block: the ranks of its sequence, its
+// length into seq_cnt.  The last warp of every block ranks its share of the box's own
 // particles while the others search the tree breadth first (one level per
 // step, all nodes of a level at once; a level of more than kListCap boxes falls
 // back to a depth-first search in batches by warp 0), every block for itself.
-// Then every warp of the cluster counts, and after a scan (the blocks' sums
+// Then every warp of the group counts, and after a scan (the blocks' sums
 // through distributed shared memory) ranks, pieces of the boxes met.
 //
 // Bound by latency: a round has few boxes for 152 SMs, and each is a chain of
 // dependent steps on one box's data.  2^21 clustered particles, 64 rounds, a
 // launch with 1, 2, 4, 8 blocks per box: 27.3, 20.5, 17.5, 17.5 us; four leave
-// twice as many clusters as eight for rounds of many boxes.
-template <typename C>
+// twice as many clusters as eight.  With more boxes than clusters (76 on 152 SMs) the blocks
+// do better on a box each: 2^27 particles, 32,768 leaves, 53.5 us a launch with a block per
+// box, 61.0 with clusters for all, 41.5 so.  Small boxes have too little to share: 2^24
+// particles in leaves of 256 23.9, 92.4 (29.4 by that rule alone) and 24.1 us; the line lies
+// at leaves of 1024, where both sides take 17.3 and 17.7 (2^22 particles), 14.0 and 14.0
+// (2^18).
+template <typename C, bool CLUSTERS>
 __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__restrict__ q0,
                                                           const C *__restrict__ q1, const C *__restrict__ q2) {
   constexpr int kSearchWarps = kTakeWarps - 1;
@@ -580,15 +587,25 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
   __shared__ uint32_t s_sum[2][kTakeCluster], s_own[kTakeCluster];  // by block of the cluster
   namespace cg = cooperative_groups;
   const cg::cluster_group cluster = cg::this_cluster();
-  cluster.sync();  // every block of the cluster runs before one writes to another's shared memory
+  if (CLUSTERS) cluster.sync();  // every block of the cluster runs before one writes to another's shared memory
   dep_launch();
   dep_wait();
   if (S.ctr->alive == 0) return;
-  const uint32_t rank = cluster.block_rank();
   const uint32_t ntaken = S.ctr->taken;
+  // blocks of a box: the cluster while every box can have one at once, else a block each
+  const uint32_t size = CLUSTERS && ntaken <= gridDim.x / kTakeCluster ? kTakeCluster : 1u;
+  const uint32_t rank = size > 1 ? cluster.block_rank() : 0u;
+  auto group_sync = [&] {
+    if (size > 1) cluster.sync();
+    else __syncthreads();
+  };
+  // `x` of this block's shared memory in that of the group's block `lane`, to all of them
+  auto tell = [&](uint32_t &x, uint32_t v, uint32_t lane) {
+    if (lane < size) *(size > 1 ? cluster.map_shared_rank(&x, lane) : &x) = v;
+  };
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t turn = 0;  // which of the sums is in use
-  for (uint32_t i = blockIdx.x / kTakeCluster; i < ntaken; i += gridDim.x / kTakeCluster) {
+  for (uint32_t i = blockIdx.x / size; i < ntaken; i += gridDim.x / size) {
     const uint32_t a = S.taken[i];
     const RBox A = S.t.box[a];
     const Box6 bx = box6(A);
@@ -599,14 +616,14 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
     };
     // this block's share of the box's own slots, whole groups of four
     const uint32_t og = IA.off >> 2, on = ((IA.off + IA.cnt + 3) >> 2) - og;
-    const uint32_t o0 = max(IA.off, 4 * (og + on * rank / kTakeCluster));
-    const uint32_t o1 = max(o0, min(IA.off + IA.cnt, 4 * (og + on * (rank + 1) / kTakeCluster)));
+    const uint32_t o0 = max(IA.off, 4 * (og + on * rank / size));
+    const uint32_t o1 = max(o0, min(IA.off + IA.cnt, 4 * (og + on * (rank + 1) / size)));
     Picks own;
     if (warp == kTakeWarps - 1) {  // the box's live particles but the centre, in slot order
       const uint32_t centre = IA.centre;
       const uint32_t k = warp_pick<C, false>(S, q0, q1, q2, o0, o1,
                                              [=](uint32_t s, uint32_t, uint32_t, uint32_t) { return s != centre; }, own);
-      if (uint32_t(lane) < kTakeCluster) *cluster.map_shared_rank(&s_own[rank], lane) = k;
+      tell(s_own[rank], k, lane);
     } else {
       const Tree &t = S.t;
       int cur = 0;
@@ -654,7 +671,7 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
       }
       if (threadIdx.x == 0) s_cur = uint32_t(cur);
     }
-    cluster.sync();
+    group_sync();
     if (warp == kTakeWarps - 1) {
       uint32_t p = 1;
       for (uint32_t b = 0; b < rank; ++b) p += s_own[b];
@@ -669,10 +686,10 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
     // counts, then ranks, of `parts` pieces of each of the nlist boxes in list,
     // at most one piece per warp at a time (its picks stay in the warp's registers)
     auto batch = [&](const uint32_t *list, uint32_t nlist) {
-      constexpr uint32_t kAll = kTakeCluster * uint32_t(kTakeWarps);
-      const uint32_t parts = nlist ? max(1u, min(16u, kAll / nlist)) : 1u;
+      const uint32_t all_warps = size * uint32_t(kTakeWarps);
+      const uint32_t parts = nlist ? max(1u, min(16u, all_warps / nlist)) : 1u;
       const uint32_t items = nlist * parts;
-      for (uint32_t i0 = 0; i0 < items; i0 += kAll) {
+      for (uint32_t i0 = 0; i0 < items; i0 += all_warps) {
         const uint32_t it = i0 + rank * uint32_t(kTakeWarps) + uint32_t(warp);
         uint32_t c = 0, off = 0, end = 0, k = 0;
         Picks rec;
@@ -693,11 +710,11 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
           }
           lpos[lane] = incl - x;
           const uint32_t sum = __shfl_sync(0xffffffffu, incl, 31);
-          if (uint32_t(lane) < kTakeCluster) *cluster.map_shared_rank(&s_sum[turn][rank], lane) = sum;
+          tell(s_sum[turn][rank], sum, lane);
         }
-        cluster.sync();
+        group_sync();
         uint32_t before = 0, total = 0;
-        for (uint32_t b = 0; b < kTakeCluster; ++b) {
+        for (uint32_t b = 0; b < size; ++b) {
           before += b < rank ? s_sum[turn][b] : 0u;
           total += s_sum[turn][b];
         }
@@ -740,7 +757,7 @@ __global__ void __launch_bounds__(kTakeThreads) k_rd_take(State S, const C *__re
       }
     }
     if (rank == 0 && threadIdx.x == 0) S.seq_cnt[a] = pos;
-    cluster.sync();  // s_own and the frontiers are reused
+    group_sync();  // s_own and the frontiers are reused
   }
 }
 
@@ -828,24 +845,29 @@ __global__ void __launch_bounds__(1024) k_rd_scan(State S, LeafRec *seqs) {
 
 // ---- rebuild --------------------------------------------------------------
 
-constexpr int kBoxThreads = 256;  // a launch of 2^21 particles' rounds with 128, 256, 512: 12.8, 11.7, 12.1 us
-constexpr int kBoxWarps = kBoxThreads / 32;
+// Threads of a block: 128, which walk 2048 particles at a time, and 256 for larger boxes
+// while these are few enough to fill no more than the SMs.  A launch with 128 and 256: leaves
+// of 8192 particles, 2048 of them, 20.3 and 17.3 us; of 4096, 512 and 2048 of them, 12.9 and
+// 11.7, 15.5 and 15.0, 8192 of them 17.0 and 17.0, 32,768 22.6 and 25.3; of 256, 65,536 of
+// them, 17.6 and 25.6.
+constexpr uint32_t kWideBox = 2048;
+constexpr uint64_t kWideBoxes = 8192;
 
 // The block's threads visit the live slots of [off, end) (every slot when
 // INIT) in aligned groups of four, four groups per thread at a time with their
 // loads issued first; f(s, x, y, z) sees each slot in increasing order per thread.
-template <typename C, bool INIT, class F>
+template <typename C, bool INIT, int THREADS, class F>
 __device__ __forceinline__ void box_walk(const State &S, const C *q0, const C *q1, const C *q2, uint32_t off,
                                          uint32_t end, F f) {
   using Raw = typename Codes4<C>::Raw;
   constexpr int U = 4;
   const uint32_t g0 = off >> 2, g1 = (end + 3) >> 2;
-  for (uint32_t gb = g0; gb < g1; gb += U * kBoxThreads) {
+  for (uint32_t gb = g0; gb < g1; gb += U * THREADS) {
     uint32_t lw[U];
     Raw cx[U], cy[U], cz[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const uint32_t g = min(gb + uint32_t(u) * kBoxThreads + threadIdx.x, g1 - 1);
+      const uint32_t g = min(gb + uint32_t(u) * THREADS + threadIdx.x, g1 - 1);
       lw[u] = INIT ? 0xffffffffu : __ldcg(S.live + (g >> 3));
       cx[u] = Codes4<C>::load(q0, g);
       cy[u] = Codes4<C>::load(q1, g);
@@ -853,7 +875,7 @@ __device__ __forceinline__ void box_walk(const State &S, const C *q0, const C *q
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const uint32_t g = gb + uint32_t(u) * kBoxThreads + threadIdx.x;
+      const uint32_t g = gb + uint32_t(u) * THREADS + threadIdx.x;
       if (g >= g1) continue;
       const uint32_t lb = (lw[u] >> (4 * (g & 7))) & 0xfu;
 #pragma unroll
@@ -869,10 +891,11 @@ __device__ __forceinline__ void box_walk(const State &S, const C *q0, const C *q
 // INIT: every leaf's first box (all particles live; the counters start).
 // Otherwise: the boxes listed by place get the bit box of their live
 // particles or die when none is left; taken boxes die.
-template <typename C, bool INIT>
-__global__ void __launch_bounds__(kBoxThreads) k_rd_rebuild(State S, const C *__restrict__ q0,
-                                                            const C *__restrict__ q1, const C *__restrict__ q2,
-                                                            const LeafRec *__restrict__ leafs) {
+template <typename C, bool INIT, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_rd_rebuild(State S, const C *__restrict__ q0, const C *__restrict__ q1,
+                                                        const C *__restrict__ q2,
+                                                        const LeafRec *__restrict__ leafs) {
+  constexpr int kBoxWarps = THREADS / 32;
   __shared__ uint32_t red[7][kBoxWarps];
   __shared__ unsigned long long rd[kBoxWarps];
   __shared__ uint32_t rp[kBoxWarps];
@@ -911,7 +934,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_rd_rebuild(State S, const C *__
     }
     const uint32_t end = off + cnt;
     uint32_t lo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi[3] = {0, 0, 0}, live = 0;
-    box_walk<C, INIT>(S, q0, q1, q2, off, end, [&](uint32_t, uint32_t x, uint32_t y, uint32_t z) {
+    box_walk<C, INIT, THREADS>(S, q0, q1, q2, off, end, [&](uint32_t, uint32_t x, uint32_t y, uint32_t z) {
       lo[0] = min(lo[0], x);
       hi[0] = max(hi[0], x);
       lo[1] = min(lo[1], y);
@@ -960,7 +983,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_rd_rebuild(State S, const C *__
     unsigned long long bd = ~0ull;
     uint32_t bp = 0xffffffffu;
     const long long s0 = (long long)lo[0] + hi[0], s1 = (long long)lo[1] + hi[1], s2 = (long long)lo[2] + hi[2];
-    box_walk<C, INIT>(S, q0, q1, q2, off, end, [&](uint32_t s, uint32_t x, uint32_t y, uint32_t z) {
+    box_walk<C, INIT, THREADS>(S, q0, q1, q2, off, end, [&](uint32_t s, uint32_t x, uint32_t y, uint32_t z) {
       const long long a = 2ll * x - s0, b = 2ll * y - s1, e = 2ll * z - s2;
       const unsigned long long d2 =
           (unsigned long long)(a * a) + (unsigned long long)(b * b) + (unsigned long long)(e * e);
@@ -1108,13 +1131,17 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
 
   const uint32_t sms = uint32_t(device_sm_count());
   const unsigned box_blocks = unsigned(a.num_leaves < 16ull * sms ? a.num_leaves : 16ull * sms);
-  const uint64_t most_clusters = 2ull * sms / kTakeCluster;  // one wave
-  const unsigned take_blocks = unsigned(a.num_leaves < most_clusters ? a.num_leaves : most_clusters) * kTakeCluster;
+  const bool wide = a.leaf_size > kWideBox && a.num_leaves <= kWideBoxes;
+  const bool clusters = a.leaf_size > kClusterBox;
+  const uint32_t per_box = clusters ? kTakeCluster : 1u;
+  const uint64_t most = 2ull * sms / per_box;  // one wave
+  const unsigned take_blocks = unsigned(a.num_leaves < most ? a.num_leaves : most) * per_box;
   const unsigned refit_blocks = unsigned((uint64_t(L.count[1]) + kWarps - 1) / kWarps);
   const unsigned select_blocks = unsigned((a.num_leaves + kWarps - 1) / kWarps);
   {
     TraceScope ts("k_rd_rebuild", st);
-    k_rd_rebuild<C, true><<<box_blocks, kBoxThreads, 0, st>>>(S, q0, q1, q2, a.leafs);
+    if (wide) k_rd_rebuild<C, true, 256><<<box_blocks, 256, 0, st>>>(S, q0, q1, q2, a.leafs);
+    else k_rd_rebuild<C, true, 128><<<box_blocks, 128, 0, st>>>(S, q0, q1, q2, a.leafs);
   }
   {
     TraceScope ts("k_rd_refit", st);
@@ -1134,20 +1161,24 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
       }
       {
         TraceScope ts("k_rd_take", s);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(take_blocks);
-        cfg.blockDim = dim3(kTakeThreads);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kTakeCluster;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = a.alone ? 2 : 1;
-        ok(cudaLaunchKernelEx(&cfg, k_rd_take<C>, S, q0, q1, q2));
+        if (!clusters) {
+          ok(launch_dependent(a.alone, k_rd_take<C, false>, dim3(take_blocks), dim3(kTakeThreads), 0, s, S, q0, q1, q2));
+        } else {
+          cudaLaunchConfig_t cfg = {};
+          cfg.gridDim = dim3(take_blocks);
+          cfg.blockDim = dim3(kTakeThreads);
+          cfg.stream = s;
+          cudaLaunchAttribute attr[2];
+          attr[0].id = cudaLaunchAttributeClusterDimension;
+          attr[0].val.clusterDim.x = kTakeCluster;
+          attr[0].val.clusterDim.y = 1;
+          attr[0].val.clusterDim.z = 1;
+          attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+          attr[1].val.programmaticStreamSerializationAllowed = 1;
+          cfg.attrs = attr;
+          cfg.numAttrs = a.alone ? 2 : 1;
+          ok(cudaLaunchKernelEx(&cfg, k_rd_take<C, true>, S, q0, q1, q2));
+        }
       }
       {
         TraceScope ts("k_rd_scan", s);
@@ -1155,8 +1186,8 @@ cudaError_t reduce_dispatch(const ReduceLaunch &a, cudaStream_t st, uint64_t *nu
       }
       {
         TraceScope ts("k_rd_rebuild", s);
-        ok(launch_dependent(a.alone, k_rd_rebuild<C, false>, dim3(box_blocks), dim3(kBoxThreads), 0, s, S, q0, q1, q2,
-                            a.leafs));
+        ok(launch_dependent(a.alone, wide ? k_rd_rebuild<C, false, 256> : k_rd_rebuild<C, false, 128>, dim3(box_blocks),
+                            dim3(wide ? 256 : 128), 0, s, S, q0, q1, q2, a.leafs));
       }
     }
   };
