@@ -24,7 +24,8 @@
 //         segments before its own, how many of its particles with code v go
 //         left: all, none, or (one segment per node) the first `quota` in
 //         position order.  The next A lists those ties as it meets them and
-//         moves the first `quota` over at its end.
+//         moves the first `quota` over at its end; where they are too many for a
+//         list, it counts them by warp in two more passes (count_ties).
 // Then F gives every particle its final child and counts the children.  Every
 // step between two grid barriers reads only what was complete before the first
 // of them; a barrier costs 1.3 us.
@@ -75,7 +76,8 @@ struct NodeTab {
   // derived, not kept
   int32_t off[kHalf];     // bin of code x: off + (x >> shift)
   uint32_t roff[kHalf], rcnt[kHalf];  // node's place in the subroot
-  uint32_t lbase[kHalf], cursor[kHalf];  // the node's part of the tie list, and its end so far
+  uint32_t lbase[kHalf], cursor[kHalf];  // the node's part of the tie list, and its end so far; without a
+                                         // list: the warp whose ties go both ways, and how many go left
 };
 constexpr uint32_t kStateWords = kSplitStateWords;
 static_assert(kStateWords == 17 * kHalf, "kept part of NodeTab");
@@ -88,7 +90,8 @@ struct Misc {
   uint32_t b0, b1;              // current segment
   uint32_t clo;                 // first CTA of the current subroot
   uint32_t shift, nbins;
-  uint32_t ties, many;          // listed ties of the segment; whether a node has more than a warp selects among
+  uint32_t ties, many;          // ties of the segment; whether a node has more than a warp selects among
+  uint32_t counted;             // whether they are counted by warp instead of listed
   uint32_t fd, fbefore;         // tie selection: digit, ties below it
   uint32_t wt[kW + 1];
   uint32_t wh[kW][32];
@@ -99,8 +102,11 @@ struct Smem {
   Misc M;
   NodeTab N;
   alignas(16) uint32_t bins[kBins];
-  alignas(16) uint32_t sum[kBins];  // sel1: prefixes of the summed histogram; B: counts per code; A, F: the tie list
+  // sel1: prefixes of the summed histogram; B: counts per code; A, F: the tie list or the ties by
+  // warp and node
+  alignas(16) uint32_t sum[kBins];
 };
+static_assert(kW * kHalf <= kBins, "ties by warp and node");
 static_assert(sizeof(Smem) <= 232448, "shared memory of one CTA");
 static_assert(offsetof(Smem, bins) % 16 == 0 && offsetof(Smem, sum) % 16 == 0, "16-byte accesses");
 
@@ -225,6 +231,7 @@ struct Ctx {
   NodeTab &N;
   uint32_t *const bins, *const sum;
   int lane, warp;
+  Smem &P;
 };
 
 // The segment of subroot s (thread 0 fills the geometry) and its kept state when
@@ -342,6 +349,10 @@ __device__ __forceinline__ void level_setup(const Ctx &x, int l) {
     if (x.lane == 31) {
       x.M.ties = ex;
       x.M.many = many;
+      // A list takes this CTA some 3 cycles a tie, counting 0.1 a position and up to 1 a tie:
+      // levels of 883,024 positions a CTA with up to 16,155 ties took 50 us more counted,
+      // levels of 441,512 with as many ties 600 us more listed
+      x.M.counted = ex > max(2048u, (x.M.b1 - x.M.b0) / 8u);
     }
   } else if (l < x.a.levels && threadIdx.x >= 64 && threadIdx.x - 64 < (1u << l)) {
     uint64_t off, cnt;
@@ -479,7 +490,7 @@ __device__ __forceinline__ void pass_a(const Ctx &x, const Pass &a, Step &next, 
   NodeTab &N = x.N;
   const uint32_t b0 = x.M.b0, b1 = x.M.b1, shift = x.M.shift;
   uint8_t *const nid = x.a.node;
-  const uint32_t room = x.M.ties;
+  const uint32_t room = x.M.ties, listed = x.M.counted ? 0u : 0xffu;
   uint32_t pos = (b0 & ~7u) + 8u * threadIdx.x;
   for (; pos < b1; pos += kStep) {
     const uint4 p = next.p, c = next.c;
@@ -516,7 +527,7 @@ __device__ __forceinline__ void pass_a(const Ctx &x, const Pass &a, Step &next, 
           if (!FIRST) nid[pos + e] = uint8_t((e < 4 ? w0 : w1) >> (8 * (e & 3)));
         }
     }
-    for (; hit; hit &= hit - 1) {
+    for (hit &= listed; hit; hit &= hit - 1) {
       const int e = __ffs(hit) - 1;
       const uint32_t at = atomicAdd(&N.cursor[byte_of(n0, e) & (kHalf - 1)], 1u);
       if (at < room) {
@@ -573,14 +584,183 @@ __device__ __forceinline__ void resolve_ties(const Ctx &x, const Pass &a, const 
   }
 }
 
+// The ties of a segment with many, without a list; all are counted as going right so far.  A
+// warp owns a contiguous part of the segment.  First the ties are counted by warp and node;
+// then, per node, the warps before the one that holds the quota's end turn all of theirs
+// left, and that one its first, in position order: two passes of 5 to 7 bytes a particle,
+// whatever the ties are, bound by their instructions.  A list is appended to by one atomic a
+// tie and read three times, by the one CTA that holds it while all others wait: 2^24
+// particles of which half are one point took 1.75 ms in k_split with one, 0.58 so (0.36
+// without ties); every other one the same point 1.52 and 0.81, all on a line 1.18 and 0.62.
+template <bool LAST>
+__device__ __noinline__ void count_ties(const SplitLaunch &a, Smem &P, const uint16_t *prev, const uint16_t *cur,
+                                        uint32_t half) {
+  Misc &M = P.M;
+  NodeTab &N = P.N;
+  const uint32_t b0 = M.b0, b1 = M.b1, shift = M.shift;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t g0 = b0 / 8u, rows = ((b1 + 7u) / 8u - g0 + 31u) / 32u;  // rows of 32 groups of 8 positions
+  const uint32_t r0 = rows * uint32_t(warp) / kW, r1 = rows * (uint32_t(warp) + 1u) / kW;
+  uint8_t *const nid = a.node;
+  uint32_t *const tc = P.sum, *const mine = tc + uint32_t(warp) * kHalf;
+  struct Row {
+    uint4 p;
+    uint2 n;
+  };
+  auto pos_of = [&](uint32_t r) { return 8u * (g0 + 32u * r + uint32_t(lane)); };
+  auto load = [&](uint32_t r, Row &t) {
+    const uint32_t pos = pos_of(r);
+    t.p = make_uint4(0, 0, 0, 0);
+    t.n = make_uint2(0, 0);
+    if (r < r1 && pos < b1) {
+      t.p = __ldcg(reinterpret_cast<const uint4 *>(prev + pos));
+      t.n = __ldcg(reinterpret_cast<const uint2 *>(nid + pos));
+    }
+  };
+  // the row's ties of this lane, by position in its group; the node of position e is its child / 2.
+  // Every loop over the 8 positions is unrolled: they are what the two passes are made of.
+  auto node_of = [&](const Row &t, int e) { return (byte_of(t.n, e) >> 1) & (kHalf - 1); };
+  auto ties = [&](const Row &t, uint32_t pos) {
+    uint32_t hit = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (2u * half_of(t.p, e) + 1u == N.plane[node_of(t, e)]) hit |= 1u << e;
+    if (pos < b0) hit &= pos + 8u > b0 ? 0xffu << (b0 - pos) : 0u;
+    if (pos + 8u > b1) hit &= pos < b1 ? 0xffu >> (pos + 8u - b1) : 0u;
+    return hit & 0xffu;
+  };
+  // whether the row is 256 ties of one node (a run of one point): counted at once, since every lane's
+  // atomics on one counter take their turns
+  auto run_of_one = [&](const Row &t, uint32_t hit) {
+    const uint32_t b = t.n.x & 0xffu;
+    int all;
+    __match_all_sync(0xffffffffu, hit == 0xffu && t.n.x == t.n.y && t.n.x == b * 0x01010101u ? b : 256u + uint32_t(lane), &all);
+    return all != 0;
+  };
+
+  for (uint32_t j = lane; j < half; j += 32) mine[j] = 0;
+  __syncwarp();
+  Row nx;
+  load(r0, nx);
+  for (uint32_t r = r0; r < r1; ++r) {
+    const Row t = nx;
+    load(r + 1, nx);
+    const uint32_t hit = ties(t, pos_of(r));
+    if (run_of_one(t, hit)) {
+      if (lane == 0) atomicAdd(&mine[node_of(t, 0)], 256u);
+      continue;
+    }
+    if (!hit) continue;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if ((hit >> e) & 1u) atomicAdd(&mine[node_of(t, e)], 1u);
+  }
+  __syncthreads();
+  for (uint32_t j = warp; j < half; j += kW) {
+    if (!(N.plane[j] & 1u)) continue;
+    const uint32_t v = tc[uint32_t(lane) * kHalf + j], incl = warp_excl(v, lane) + v;
+    const uint32_t after = __ballot_sync(0xffffffffu, incl > N.quota[j]);
+    const int cut = after ? __ffs(after) - 1 : 31;
+    if (lane == cut) {
+      N.lbase[j] = uint32_t(cut);
+      N.cursor[j] = N.quota[j] - (incl - v);
+    }
+    if (lane == 31 && incl != N.mine[j]) atomicOr(a.err, kErrInternal);  // never expected
+  }
+  __syncthreads();
+  for (uint32_t j = lane; j < half; j += 32) mine[j] = 0;  // now: the ties of a cut node met so far
+  __syncwarp();
+  load(r0, nx);
+  for (uint32_t r = r0; r < r1; ++r) {
+    const Row t = nx;
+    load(r + 1, nx);
+    const uint32_t pos = pos_of(r), hit = ties(t, pos);
+    const bool one = run_of_one(t, hit);
+    uint32_t left = 0, pend = 0;
+    if (one) {
+      const uint32_t cut = N.lbase[node_of(t, 0)];
+      left = uint32_t(warp) < cut ? hit : 0u;
+      pend = uint32_t(warp) == cut ? hit : 0u;
+    } else if (hit) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t cut = N.lbase[node_of(t, e)];
+        if (uint32_t(warp) < cut) left |= 1u << e;
+        if (uint32_t(warp) == cut) pend |= 1u << e;
+      }
+      left &= hit;
+      pend &= hit;
+    }
+    for (;;) {  // the cut nodes of the row, one by one: the first ones in position order
+      const uint32_t any = __ballot_sync(0xffffffffu, pend != 0);
+      if (!any) break;
+      const uint32_t j = __shfl_sync(0xffffffffu, pend ? node_of(t, __ffs(pend) - 1) : 0u, __ffs(any) - 1);
+      uint32_t m = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (node_of(t, e) == j) m |= 1u << e;
+      m &= pend;
+      const uint32_t cnt = __popc(m), ex = warp_excl(cnt, lane), seen = mine[j], quota = N.cursor[j];
+      uint32_t take = seen + ex < quota ? min(cnt, quota - seen - ex) : 0u;
+      pend &= ~m;
+      if (take == cnt) left |= m;
+      else
+        for (; take; --take, m &= m - 1) left |= m & (0u - m);
+      __syncwarp();
+      if (lane == 31) mine[j] = seen + ex + cnt;
+      __syncwarp();
+    }
+    const bool turn = one && __all_sync(0xffffffffu, left == 0xffu);  // all 256
+    if (!left) continue;
+    uint4 c = make_uint4(0, 0, 0, 0);
+    if (!LAST) c = __ldcg(reinterpret_cast<const uint4 *>(cur + pos));
+    int same = 0;
+    if (turn) {  // of one code on the next axis too, or of one part of the chunk?
+      if (!LAST)
+        __match_all_sync(0xffffffffu, c.x == c.y && c.x == c.z && c.x == c.w && c.x >> 16 == (c.x & 0xffffu)
+                                          ? c.x & 0xffffu
+                                          : 65536u + uint32_t(lane),
+                         &same);
+      else __match_all_sync(0xffffffffu, part_of(M, pos), &same);
+    }
+    uint32_t *const row = P.bins + (part_of(M, pos) * kW + warp) * kNodes;
+    uint32_t w0 = t.n.x, w1 = t.n.y;
+    const uint32_t by = same ? 256u : 1u;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (!((left >> e) & 1u)) continue;
+      const uint32_t j = node_of(t, e);
+      if (e < 4) w0 ^= 1u << (8 * e);
+      else w1 ^= 1u << (8 * (e - 4));
+      if (same && (e > 0 || lane > 0)) continue;
+      if (LAST) {  // (a group of 8 lies in one part: parts start at multiples of 16)
+        atomicAdd(row + 2 * j, by);
+        atomicSub(row + 2 * j + 1, by);
+      } else {
+        const int32_t q = int32_t(half_of(c, e) >> shift);
+        atomicAdd(P.bins + (uint32_t(q + N.off[2 * j]) & (kBins - 1)), by);
+        atomicSub(P.bins + (uint32_t(q + N.off[2 * j + 1]) & (kBins - 1)), by);
+      }
+    }
+    if (pos >= b0 && pos + 8u <= b1) {
+      *reinterpret_cast<uint2 *>(nid + pos) = make_uint2(w0, w1);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if ((left >> e) & 1u) nid[pos + e] = uint8_t((e < 4 ? w0 : w1) >> (8 * (e & 3)));
+    }
+  }
+}
+
 template <bool FIRST, bool LAST>
 __device__ __forceinline__ void run_a(const Ctx &x, const Pass &a, Step &t) {
-  // in shared memory when the list fits, else in this segment's part of the global one
+  // the list: in shared memory when it fits, else in this segment's part of the global one
   uint32_t *const list = x.M.ties <= kBins ? x.sum : x.a.ties + x.M.b0;
   pass_a<FIRST, LAST>(x, a, t, list);
   __syncthreads();
   if (!FIRST && x.M.ties) {
-    resolve_ties<LAST>(x, a, list);
+    if (x.M.counted) count_ties<LAST>(x.a, x.P, a.prev, a.cur, a.half);
+    else resolve_ties<LAST>(x, a, list);
     __syncthreads();
   }
 }
@@ -627,7 +807,7 @@ __global__ void __launch_bounds__(kT, 1) k_split(const __grid_constant__ SplitLa
   dep_wait();
   if (call_failed(a.err)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const Ctx x = {a, M, N, P.bins, P.sum, lane, warp};
+  const Ctx x = {a, M, N, P.bins, P.sum, lane, warp, P};
   const uint32_t S = 1u << a.depth;
   const int K = a.levels;
   uint32_t epoch = 0;
