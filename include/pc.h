@@ -25,12 +25,12 @@
  *     and decompress each wait for a few bytes (the value range, then the
  *     final size or the error word) and so return with their work finished.
  *     The kernels write those bytes into page-locked host blocks of 4 KB, where
- *     the calling thread watches for them: past some 20 us as
- *     the device's scheduling flags ask (cudaSetDeviceFlags: blocked with
- *     cudaDeviceScheduleBlockingSync, without a pause with
- *     cudaDeviceScheduleSpin, else yielding the processor now and then).  The
- *     library allocates the blocks on first use, sixteen at a time, and keeps
- *     them for the life of the process
+ *     the calling thread watches for them: past some 20 us as the device's
+ *     scheduling flags ask (cudaSetDeviceFlags: blocked with
+ *     cudaDeviceScheduleBlockingSync, yielding the processor now and then with
+ *     cudaDeviceScheduleYield, else without a pause).  The library allocates the
+ *     blocks on first use, sixteen at a time, and keeps them for the life of the
+ *     process
  *     (one block per call in flight); pc_compress_noalloc allocates none (it
  *     uses blocks that exist, else plain copies).
  *

@@ -68,14 +68,15 @@ unsigned wait_mode() {
 cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st, unsigned mode) {
   // A poll takes a third of a nanosecond, a look at the stream 1.5 us, by which a word that
   // comes meanwhile is seen later: one look in about 20 us (a call of 10,007 particles
-  // takes 63.3 us with one in 1.3 us, 60.1 so).
+  // takes 63.3 us with one in 1.3 us, 60.1 so).  Yielding with every look, unasked, took
+  // another 1.5 us of a call of 155.
   constexpr uint32_t kLook = 1u << 16;
   for (uint32_t spins = 1; *word == unset; ++spins) {
     if (spins % kLook) continue;
     const cudaError_t e = mode == cudaDeviceScheduleBlockingSync ? cudaStreamSynchronize(st) : cudaStreamQuery(st);
     if (e == cudaSuccess) break;  // done, the word as the kernels left it
     if (e != cudaErrorNotReady) return e;
-    if (mode != cudaDeviceScheduleSpin) std::this_thread::yield();
+    if (mode == cudaDeviceScheduleYield) std::this_thread::yield();
   }
   std::atomic_thread_fence(std::memory_order_acquire);
   return cudaSuccess;
@@ -115,7 +116,7 @@ cudaError_t HeaderCopy::finish() {
   if (done) return cudaSuccess;
   const volatile uint32_t *flag = reinterpret_cast<volatile uint32_t *>(b.host + kHeaderBytes + 4);
   // work is queued behind the word and more is to follow it: not in a synchronisation
-  const cudaError_t e = wait_word(flag, 0u, st, cudaDeviceScheduleYield);
+  const cudaError_t e = wait_word(flag, 0u, st, cudaDeviceScheduleSpin);
   if (e != cudaSuccess) return e;
   if (*flag == 0u) return cudaErrorUnknown;
   std::memcpy(h, b.host, kHeaderBytes);

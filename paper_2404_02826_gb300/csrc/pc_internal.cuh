@@ -414,8 +414,8 @@ inline cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStrea
 // calling thread: a result arrives 1 to 2 us after it is written, a copy and a
 // synchronisation of the stream take 8.  Past some 20 us the wait goes
 // on as `mode` says (wait_mode, the device's scheduling flags): blocked in a
-// synchronisation of the stream with cudaDeviceScheduleBlockingSync; watching without
-// a pause with cudaDeviceScheduleSpin; else yielding the processor now and then.
+// synchronisation of the stream with cudaDeviceScheduleBlockingSync; yielding the
+// processor now and then with cudaDeviceScheduleYield; else watching without a pause.
 cudaError_t wait_word(const volatile uint32_t *word, uint32_t unset, cudaStream_t st, unsigned mode);
 unsigned wait_mode();
 
